@@ -30,15 +30,15 @@ template <> struct FaceShape<64> { static constexpr int D = 3, N = 4; };
 template <int D, int N>
 struct FaceIdx {
   static constexpr int NN = N * N, NF = (D == 2) ? N : NN;
-  __device__ __forceinline__ static int stride(int a) { return a == 0 ? 1 : (a == 1 ? N : NN); }
-  __device__ __forceinline__ static int tang(int k, int r) {
+  __host__ __device__ __forceinline__ static int stride(int a) { return a == 0 ? 1 : (a == 1 ? N : NN); }
+  __host__ __device__ __forceinline__ static int tang(int k, int r) {
     if constexpr (D == 2) return r * stride(1 - k);
     return (r % N) * stride(k == 0 ? 1 : 0) + (r / N) * stride(k == 2 ? 1 : 2);
   }
-  __device__ __forceinline__ static int face(int f, int r) {
+  __host__ __device__ __forceinline__ static int face(int f, int r) {
     return (f & 1) * (N - 1) * stride(f >> 1) + tang(f >> 1, r);
   }
-  __device__ __forceinline__ static int off(int f, int r) {
+  __host__ __device__ __forceinline__ static int off(int f, int r) {
     return (r / NF + 1 - (f & 1)) * stride(f >> 1) + tang(f >> 1, r % NF);
   }
 };

@@ -1,0 +1,1033 @@
+// Level-0 operator A0 = c M + A as symmetric element blocks, one thread per
+// (element, row): the float64 operator of the outer CG, and the assembled
+// smoother, residual and transfers of level 0 in the V-cycle precision.
+//
+// Storage. A0 is symmetric, so each coupling is kept once: per element the
+// packed triangle of its diagonal block, and per interior face one face block
+// that both elements read (the second one finds it in the L2: elements are
+// numbered so that neighbours are near). Only the part of a coupling that a
+// GLL nodal basis can make nonzero is stored. With the DoFs of either element
+// in "face-first" order (the NF DoFs of the shared face, then the others),
+// the block K of owner e and neighbour n (owner: the lower internal index) is
+//   F[c][r] (c < NF, r < B): n's face DoF c against every DoF of e,
+//   G[c][j] (c < B - NF, j < NF): n's other DoFs against e's face DoFs,
+// i.e. the columns of K one after the other; n reads the same entries as the
+// rows of K^T. Column strides are odd, so that both directions are free of
+// bank conflicts in shared memory. 2D Q2: 135 instead of 261 stored entries
+// per element, 3D Q2: 1,593 instead of 3,159, 3D Q3: 7,456 instead of 14,848.
+//
+// A block of threads owns a few elements, copies their blocks to shared memory
+// with cp.async, gathers its own and its neighbours' DoFs (coalesced: the
+// threads of an element read one neighbour's DoFs together) and multiplies.
+//
+// Float64 products run on the integer pipe. GB300 issues 2 float64 FMAs per
+// SM and clock against 64 32-bit integer multiply-adds, so a float64 block
+// product is bound by the FP64 pipe, not by HBM. Here the operator is kept in
+// 60-bit fixed point and x is converted to 58-bit fixed point with one exponent
+// per element; the sum of the products is formed exactly in 64-bit integers (up
+// to the product of the low halves, 2^-60 of the row's scale) and rounded once.
+// Fixed point needs entries of one magnitude: element e's rows and columns are
+// scaled by 2^-s_e, 2^{2 s_e} >= its largest diagonal entry, after which an SPD
+// operator's entries are at most 1. An entry is a1 2^28 + a0 with |a0| <= 2^27, an
+// x is x1 2^31 + x0 with |x0| <= 2^30. With sum_j |A_ij| <= 2^60, |A_ij| <= 2^58
+// (global exponent kA) and |x| <= 2^58, and T <= 304 entries in a row:
+//   hi = sum a1 x1 <= 2^32 2^27,  m1 = sum a1 x0 <= 2^32 2^30,
+//   m2 = sum a0 x1 <= T 2^27 2^27 < 2^62.3,
+// so none overflows, and every a1 and x1 fits 32 bits. A NaN or infinity in the
+// neighbourhood takes a float64 path over the same entries (products) or gives
+// NaN (smoother).
+#pragma once
+#include "face_op.cuh"
+#include "kernels.cuh"
+
+namespace aggmg {
+
+// ---------------------------------------------------------------- fixed point
+// bits of a row's entries in sum, of a single entry, of x; of the low halves of
+// an entry and of x
+constexpr int FX_A = 60, FX_AE = 58, FX_X = 58, FX_P = 28, FX_Q = 31;
+constexpr int kFxNone = -100000;                    // below every exponent
+constexpr int kFxBad = 1 << 20;                     // marks a NaN or an infinity
+// exponent of the unit of FxAcc::sum() for x with shared biased exponent E, less E
+constexpr int kFxBias = FX_P + FX_Q - 1075 - (FX_X - 53);
+
+// biased exponent of x (1 for zero and subnormals; 2047 for NaN and Inf)
+__device__ __forceinline__ int fx_exp(double x) {
+  const int e = (__double2hiint(x) >> 20) & 0x7ff;
+  return e ? e : 1;
+}
+// x in units of 2^{E - 1075 - (FX_X - 53)} rounded to an integer (at most 2^FX_X for
+// E >= fx_exp(x)), as halves (lo, hi)
+__device__ __forceinline__ int2 fx_split(double x, int E) {
+  const int h = __double2hiint(x);
+  int e = (h >> 20) & 0x7ff;
+  unsigned long long m = ((unsigned long long)(unsigned)(h & 0xfffff) << 32) | (unsigned)__double2loint(x);
+  if (e) m |= 1ull << 52;
+  else e = 1;
+  const int sh = min(E - e, 63);
+  long long v = (long long)((((m << (FX_X - 52)) >> sh) + 1) >> 1);
+  v = h < 0 ? -v : v;
+  const int lo = ((int)v << (32 - FX_Q)) >> (32 - FX_Q);
+  return make_int2(lo, (int)((v - lo) >> FX_Q));
+}
+// S * 2^q for an integer S
+__device__ __forceinline__ double fx_scale(long long S, int q) {
+  const double d = (double)S;
+  if (q > -1000 && q < 1000) return d * __hiloint2double((q + 1023) << 20, 0);
+  return scalbn(d, q);
+}
+
+struct FxAcc {
+  long long hi = 0, m1 = 0, m2 = 0;
+  __device__ __forceinline__ void fma(int2 a, int2 x) {
+    hi += (long long)a.y * x.y;
+    m1 += (long long)a.y * x.x;
+    m2 += (long long)a.x * x.y;
+  }
+  using Sum = long long;
+  // the sum in units of 2^{FX_P + FX_Q}
+  __device__ __forceinline__ long long sum() const {
+    return hi + ((m1 + (1ll << (FX_Q - 1))) >> FX_Q) + ((m2 + (1ll << (FX_P - 1))) >> FX_P);
+  }
+};
+// S / 2^sh, rounded
+__device__ __forceinline__ long long sum_shift(long long S, int sh) {
+  if (sh == 0) return S;
+  return sh > 62 ? 0 : (S + (1ll << (sh - 1))) >> sh;
+}
+__device__ __forceinline__ float sum_shift(float s, int) { return s; }
+struct FlAcc {
+  float s = 0.0f;
+  __device__ __forceinline__ void fma(float a, float x) { s += a * x; }
+  using Sum = float;
+  __device__ __forceinline__ float sum() const { return s; }
+};
+
+// Stored entry, x entry and accumulator of a value type
+template <typename T> struct SymNum;
+template <> struct SymNum<double> { using ST = int2; using SX = int2; using SX2 = int4; using Acc = FxAcc; };
+template <> struct SymNum<float> { using ST = float; using SX = float; using SX2 = float2; using Acc = FlAcc; };
+__device__ __forceinline__ int2 sx_first(int4 v) { return make_int2(v.x, v.y); }
+__device__ __forceinline__ int2 sx_second(int4 v) { return make_int2(v.z, v.w); }
+__device__ __forceinline__ float sx_first(float2 v) { return v.x; }
+__device__ __forceinline__ float sx_second(float2 v) { return v.y; }
+__device__ __forceinline__ int2 sym_val(int2 v) { return v; }
+__device__ __forceinline__ float sym_val(float v) { return v; }
+__device__ __forceinline__ float sym_val(__nv_bfloat16 v) { return __bfloat162float(v); }
+
+// ---------------------------------------------------------------- layout
+constexpr int round_to(int k, int q) { return (k + q - 1) / q * q; }
+
+template <int B> struct SymShape {
+  static constexpr int D = FaceShape<B>::D, N = FaceShape<B>::N;
+  static constexpr int NF = FaceIdx<D, N>::NF, NFACE = 2 * D, BO = B - NF;
+  static constexpr int LDF = B | 1, LDG = NF | 1, LDP = B | 1;
+  static constexpr int TRI = B * (B + 1) / 2;
+  // x of one element in shared memory: face DoFs, then the others from an even offset
+  static constexpr int XO = round_to(NF, 2), BX = XO + round_to(BO, 2);
+};
+// entries per element (diagonal), per face block, per transfer block, padded to 16 bytes
+template <typename ST, int B> struct SymLay {
+  using S = SymShape<B>;
+  static constexpr int Q = 16 / (int)sizeof(ST);
+  static constexpr int KD = round_to(S::TRI, Q);
+  static constexpr int KB = round_to(S::NF * S::LDF + S::BO * S::LDG, Q);
+  static constexpr int KP = round_to(B * S::LDP, Q);
+};
+
+// Elements per block (U) and thread groups per element (G: group 0 takes the
+// diagonal block, the others share the faces; their sums are added at the end).
+#ifndef AGG_SYM_D9
+#define AGG_SYM_D9 14, 1
+#endif
+#ifndef AGG_SYM_D16
+#define AGG_SYM_D16 8, 1
+#endif
+#ifndef AGG_SYM_D27
+#define AGG_SYM_D27 1, 4
+#endif
+#ifndef AGG_SYM_F9
+#define AGG_SYM_F9 14, 1
+#endif
+template <int U_, int G_> struct SymCfgOf { static constexpr int U = U_, G = G_; };
+template <typename T, int B> struct SymCfg;
+template <> struct SymCfg<double, 4> : SymCfgOf<32, 1> {};
+template <> struct SymCfg<double, 8> : SymCfgOf<16, 1> {};
+template <> struct SymCfg<double, 9> : SymCfgOf<AGG_SYM_D9> {};
+template <> struct SymCfg<double, 16> : SymCfgOf<AGG_SYM_D16> {};
+template <> struct SymCfg<double, 27> : SymCfgOf<AGG_SYM_D27> {};
+template <> struct SymCfg<double, 64> : SymCfgOf<1, 4> {};
+template <> struct SymCfg<float, 4> : SymCfgOf<32, 1> {};
+template <> struct SymCfg<float, 8> : SymCfgOf<16, 1> {};
+template <> struct SymCfg<float, 9> : SymCfgOf<AGG_SYM_F9> {};
+template <> struct SymCfg<float, 16> : SymCfgOf<8, 1> {};
+template <> struct SymCfg<float, 27> : SymCfgOf<4, 1> {};
+template <> struct SymCfg<float, 64> : SymCfgOf<1, 4> {};
+
+template <typename T, int B>
+struct SymView {
+  using ST = typename SymNum<T>::ST;
+  const ST* diag;         // [n][KD] packed triangle, entry (i, j), j <= i, at i (i + 1) / 2 + j
+  const ST* face;         // [face block][KB]
+  const int2* info;       // [n][2d] neighbour's internal index (-1 none), face block
+  const int8_t* code;     // [n][2d] neighbour's local face
+  const int16_t* sc;      // [n] scale exponents s_e (float64)
+  int kA;                 // global exponent of the fixed-point entries (float64)
+  int64_t n;
+};
+
+// smoother block inverses (packed triangles) or transfer blocks of level 0, one
+// per element; float64: fixed point with an exponent per element
+template <typename TS>
+struct SymBlk {
+  const TS* v;
+  const int16_t* k;
+};
+
+__device__ __forceinline__ void cp_async16(void* dst, const void* src) {
+  const unsigned d = (unsigned)__cvta_generic_to_shared(dst);
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(d), "l"(src) : "memory");
+}
+__device__ __forceinline__ void cp_async8(void* dst, const void* src) {
+  const unsigned d = (unsigned)__cvta_generic_to_shared(dst);
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(d), "l"(src) : "memory");
+}
+__device__ __forceinline__ void cp_async4(void* dst, const void* src) {
+  const unsigned d = (unsigned)__cvta_generic_to_shared(dst);
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(d), "l"(src) : "memory");
+}
+__device__ __forceinline__ void cp_async_x(int2* dst, const int2* src) { cp_async8(dst, src); }
+__device__ __forceinline__ void cp_async_x(float* dst, const float* src) { cp_async4(dst, src); }
+
+// position of DoF r in the face-first order of local face f
+template <int B>
+__device__ __forceinline__ int face_first(int f, int r, bool& on) {
+  using S = SymShape<B>;
+  constexpr int N = S::N;
+  const int k = f >> 1, s = f & 1;
+  const int a = r % N, b = (r / N) % N, c = r / (N * N);
+  const int ik = (k == 0) ? a : (k == 1 ? b : c);
+  int j;
+  if constexpr (S::D == 2) j = (k == 0) ? b : a;
+  else j = ((k == 0) ? b : a) + N * ((k == 2) ? b : c);
+  on = ik == s * (N - 1);
+  return on ? j : S::NF + j + S::NF * (ik - (1 - s));
+}
+
+// acc += sum_{t < CNT} p[t stride] x[t]
+template <typename T, int CNT, typename ST>
+__device__ __forceinline__ void sym_dot(const ST* p, int stride, const typename SymNum<T>::SX* x,
+                                        typename SymNum<T>::Acc& acc) {
+  constexpr int kUnroll = (CNT <= 27) ? (CNT + 1) / 2 : 8;
+#pragma unroll kUnroll
+  for (int t = 0; t < CNT; t += 2) {
+    const auto xx = *reinterpret_cast<const typename SymNum<T>::SX2*>(x + t);
+    acc.fma(sym_val(p[t * stride]), sx_first(xx));
+    if (CNT % 2 == 0 || t + 1 < CNT) acc.fma(sym_val(p[(t + 1) * stride]), sx_second(xx));
+  }
+}
+// the same for x at any (unpaired) position
+template <typename T, int CNT, typename ST>
+__device__ __forceinline__ void sym_dot_any(const ST* p, int stride, const typename SymNum<T>::SX* x,
+                                            typename SymNum<T>::Acc& acc) {
+#pragma unroll
+  for (int t = 0; t < CNT; ++t) acc.fma(sym_val(p[t * stride]), x[t]);
+}
+// acc += sum_c M(r, c) x[c] for a packed triangle M
+template <typename T, int B, typename ST>
+__device__ __forceinline__ void sym_tri(const ST* m, int r, const typename SymNum<T>::SX* x,
+                                        typename SymNum<T>::Acc& acc) {
+  const int row = r * (r + 1) / 2;
+  constexpr int kUnroll = (B <= 27) ? (B + 1) / 2 : 8;
+#pragma unroll kUnroll
+  for (int c = 0; c < B; c += 2) {
+    const auto xx = *reinterpret_cast<const typename SymNum<T>::SX2*>(x + c);
+    acc.fma(sym_val(m[c <= r ? row + c : c * (c + 1) / 2 + r]), sx_first(xx));
+    if (B % 2 == 0 || c + 1 < B)
+      acc.fma(sym_val(m[c + 1 <= r ? row + c + 1 : (c + 1) * (c + 2) / 2 + r]), sx_second(xx));
+  }
+}
+
+enum { SYM_SPMV = 0, SYM_CHEB = 1, SYM_RESTRICT = 2 };
+
+// A vector as the kernels read it: T = double: fixed point, X[unit B + i] and one
+// exponent per element (the largest biased exponent of its x plus its scale, kFxBad
+// with a NaN or Inf); T = float: the vector itself.
+template <typename T> struct SymVec {
+  const typename SymNum<T>::SX* X;
+  const int* E;
+};
+
+// Shared memory of a block. Two stages (of everything a tile reads: operator
+// blocks, Dinv or P blocks, x), so that one tile's copies are in flight while
+// the other one is multiplied: GB300 needs about 100 KB in flight per SM to reach
+// its HBM rate. Then the face rows' partial sums, the groups' sums, exponents.
+template <typename T, typename TD, int B, int OP, int KIND>
+struct SymSmem {
+  using C = SymCfg<T, B>;
+  using S = SymShape<B>;
+  using ST = typename SymNum<T>::ST;
+  using SX = typename SymNum<T>::SX;
+  using Sum = typename SymNum<T>::Acc::Sum;
+  using SD = typename std::conditional<OP != SYM_CHEB || std::is_same<T, double>::value, ST, TD>::type;
+  using L = SymLay<ST, B>;
+  static constexpr bool kFx = std::is_same<T, double>::value;
+  static constexpr bool kProduct = !(OP == SYM_CHEB && KIND == 0);
+  static constexpr int U = C::U, G = kProduct ? C::G : 1;
+  static constexpr int KE = kProduct ? L::KD + S::NFACE * L::KB : 0;
+  static constexpr int KX = (OP == SYM_SPMV) ? 0 : (OP == SYM_CHEB ? SymLay<SD, B>::KD : L::KP);
+  static constexpr int NX = kProduct ? 1 + S::NFACE : 0;
+  static constexpr int NTH = round_to(U * B * G, 32);
+  static constexpr size_t kBlk = (size_t)U * KE * sizeof(ST);
+  static constexpr size_t kExt = (size_t)U * KX * sizeof(SD);
+  static constexpr size_t kXs = round_to(U * NX * S::BX * (int)sizeof(SX), 16);
+  static constexpr size_t kEx = kFx ? round_to(U * NX * 4, 16) : 0;
+  static constexpr size_t kStage = kBlk + kExt + kXs + kEx;
+  static constexpr size_t kPart = kProduct ? round_to(U * S::NFACE * B * (int)sizeof(Sum), 16) : 0;
+  static constexpr size_t kRed = round_to((G - 1) * U * B * (int)sizeof(Sum), 16);
+  static constexpr size_t kTs = (OP == SYM_SPMV) ? 0 : round_to(U * S::BX * (int)sizeof(SX), 16);
+  static constexpr size_t kRest = kPart + kRed + kTs + round_to(2 * U * (int)sizeof(int), 16);
+  static constexpr int kStages = (2 * kStage + kRest <= 225 * 1024) ? 2 : 1;
+  static constexpr size_t bytes = kStages * kStage + kRest;
+};
+
+// Ring slots, warps per block and blocks per SM of the streaming form.
+#ifndef AGG_RING_S27
+#define AGG_RING_S27 4
+#endif
+#ifndef AGG_RING_W27
+#define AGG_RING_W27 5
+#endif
+#ifndef AGG_RING_B27
+#define AGG_RING_B27 3
+#endif
+#ifndef AGG_RING_S9
+#define AGG_RING_S9 5
+#endif
+#ifndef AGG_RING_W9
+#define AGG_RING_W9 5
+#endif
+#ifndef AGG_RING_B9
+#define AGG_RING_B9 4
+#endif
+template <typename T, int B> struct SymRingSlots {
+  static constexpr int value = (B == 27) ? AGG_RING_S27 : AGG_RING_S9;
+};
+template <typename T, int B> struct SymRingWarps {
+  static constexpr int value = (B == 27) ? AGG_RING_W27 : AGG_RING_W9;
+};
+template <typename T, int B> struct SymRingBlocks {
+  static constexpr int value = (B == 27) ? AGG_RING_B27 : AGG_RING_B9;
+};
+
+// The row's product over stored entries in float64, for neighbourhoods that
+// hold a NaN or an infinity (agg_operator_apply passes those on as before).
+template <int B>
+__device__ __noinline__ double sym_row_nonfinite(const SymView<double, B>& A, int64_t unit, int r, const double* x) {
+  using S = SymShape<B>;
+  using L = SymLay<int2, B>;
+  using FI = FaceIdx<S::D, S::N>;
+  const int se = A.sc[unit];
+  double y = 0.0;
+  auto val = [&](int2 a, int s) { return scalbn((double)(((long long)a.y << FX_P) + a.x), se + s - A.kA); };
+  for (int c = 0; c < B; ++c) {
+    const int hi = max(r, c), lo = min(r, c);
+    y += val(A.diag[(size_t)unit * L::KD + hi * (hi + 1) / 2 + lo], se) * x[(size_t)unit * B + c];
+  }
+  for (int f = 0; f < S::NFACE; ++f) {
+    const int2 nf = A.info[unit * S::NFACE + f];
+    if (nf.x < 0) continue;
+    const int fn = A.code[unit * S::NFACE + f], sn = A.sc[nf.x];
+    const bool tr = nf.x < unit;
+    bool on;
+    const int pos = face_first<B>(f, r, on);
+    const int2* blk = A.face + (size_t)nf.y * L::KB;
+    const int2* g = blk + S::NF * S::LDF;
+    const double* xn = x + (size_t)nf.x * B;
+    for (int t = 0; t < (on ? B : S::NF); ++t) {
+      const int dof = t < S::NF ? FI::face(fn, t) : FI::off(fn, t - S::NF);
+      const int2 a = tr ? (on ? blk[pos * S::LDF + t] : g[(pos - S::NF) * S::LDG + t])
+                        : (t < S::NF ? blk[t * S::LDF + pos] : g[(t - S::NF) * S::LDG + pos]);
+      y += val(a, sn) * xn[dof];
+    }
+  }
+  return y;
+}
+
+// Fixed-point copy of one value per thread, a block of threads holding whole
+// elements (thread = slot B + r): X and E of SymVec. se: shared int per slot.
+template <int B>
+__device__ __forceinline__ void fx_store(double v, bool active, int slot, int64_t unit, int r, const int16_t* sc, int2* X,
+                                         int* E, int* se, int U) {
+  if (threadIdx.x < U) se[threadIdx.x] = 1;
+  __syncthreads();
+  if (active) atomicMax(se + slot, fx_exp(v));
+  __syncthreads();
+  if (active) {
+    const int e = se[slot];
+    X[(size_t)unit * B + r] = fx_split(v, e);
+    if (r == 0) E[unit] = e == 2047 ? kFxBad : e + sc[unit];
+  }
+}
+
+// One level-0 step, y = A0 x inside.
+//   SYM_SPMV, KIND 0: out = y; 1: out = rhs - y; 2: out = y and (x, y) -> alpha
+//   SYM_CHEB, KIND as in k_cheb: Chebyshev step with the block inverses `ext`;
+//     float64: also writes the new iterate's fixed-point copy (Xo, Eo)
+//   SYM_RESTRICT: out = P^T (rhs - y) with the transfer blocks `ext`
+// x: the vector itself (own values); xv: what the products read. The blocks of
+// a launch loop over tiles of U elements, so that the tiles in flight are
+// neighbours and share face blocks through the L2.
+// A face costs a row NF products with the neighbour's face DoFs, and its NF face
+// rows BO more; those are dealt to all B threads of the element (B / NF partial
+// sums per face row), which keeps every lane busy.
+template <typename T, typename TD, int B, int OP, int KIND>
+static __global__ void __launch_bounds__(SymSmem<T, TD, B, OP, KIND>::NTH)
+    k_sym(SymView<T, B> A, SymBlk<typename SymSmem<T, TD, B, OP, KIND>::SD> ext, SymVec<T> xv,
+          const T* __restrict__ rhs, const T* __restrict__ x, T* __restrict__ out, T* __restrict__ d, int2* Xo, int* Eo,
+          T c1, T c2, double* partials, CGState* st) {
+  using M = SymSmem<T, TD, B, OP, KIND>;
+  using S = SymShape<B>;
+  using ST = typename M::ST;
+  using SD = typename M::SD;
+  using SX = typename M::SX;
+  using Sum = typename M::Sum;
+  using Acc = typename SymNum<T>::Acc;
+  using L = typename M::L;
+  constexpr int U = M::U, G = M::G, NFACE = S::NFACE, BX = S::BX, NF = S::NF, BO = S::BO, N = S::N;
+  constexpr bool kFx = M::kFx;
+  constexpr int kShare = BO / N;                      // off-face terms of a face row per thread
+  constexpr int FPG = (G == 1) ? NFACE : (NFACE + G - 2) / (G - 1);   // faces per group
+  if (st && st->done) return;
+  extern __shared__ __align__(16) unsigned char sym_sm[];
+  Sum* spart = reinterpret_cast<Sum*>(sym_sm + M::kStages * M::kStage);
+  Sum* sred = reinterpret_cast<Sum*>(sym_sm + M::kStages * M::kStage + M::kPart);
+  SX* sts = reinterpret_cast<SX*>(sym_sm + M::kStages * M::kStage + M::kPart + M::kRed);
+  int* smax = reinterpret_cast<int*>(sym_sm + M::kStages * M::kStage + M::kPart + M::kRed + M::kTs);
+
+  const int tid = threadIdx.x;
+  const int g = (G == 1) ? 0 : tid / (U * B);
+  const int slot = (tid - g * U * B) / B;
+  const int r = tid - g * U * B - slot * B;
+  const bool mine = (G == 1) ? tid < U * B : g < G;
+  const int64_t ntiles = (A.n + U - 1) / U;
+  double part = 0.0;
+  // the group's k-th face
+  auto face_of = [&](int k) { return G == 1 ? k : g - 1 + k * (G - 1); };
+
+  int2 info[FPG];
+  int8_t code[FPG];
+  auto load_info = [&](int64_t tile) {
+    if constexpr (M::kProduct) {
+      const int64_t unit = tile * U + slot;
+#pragma unroll
+      for (int k = 0; k < FPG; ++k) {
+        info[k] = make_int2(-1, 0);
+        code[k] = 0;
+        if (mine && unit < A.n && (G == 1 || g > 0) && face_of(k) < NFACE) {
+          info[k] = A.info[unit * NFACE + face_of(k)];
+          code[k] = A.code[unit * NFACE + face_of(k)];
+        }
+      }
+    }
+  };
+  // copies of a tile into stage `sg` (its face info has been loaded)
+  auto issue = [&](int64_t tile, int sg) {
+    const int64_t unit = tile * U + slot;
+    if (mine && unit < A.n) {
+      unsigned char* base = sym_sm + sg * M::kStage;
+      ST* eb = reinterpret_cast<ST*>(base) + slot * M::KE;
+      SX* ex = reinterpret_cast<SX*>(base + M::kBlk + M::kExt) + slot * M::NX * BX;
+      int* ee = reinterpret_cast<int*>(base + M::kBlk + M::kExt + M::kXs) + slot * M::NX;
+      if constexpr (OP != SYM_SPMV) {
+        constexpr int QD = 16 / (int)sizeof(SD);
+        const SD* src = ext.v + (size_t)unit * M::KX;
+        SD* dst = reinterpret_cast<SD*>(base + M::kBlk) + slot * M::KX;
+        for (int p = r + B * g; p < M::KX / QD; p += B * G) cp_async16(dst + p * QD, src + p * QD);
+      }
+      if constexpr (M::kProduct) {
+        if (g == 0) {
+          const ST* src = A.diag + (size_t)unit * L::KD;
+#pragma unroll 4
+          for (int p = r; p < L::KD / L::Q; p += B) cp_async16(eb + p * L::Q, src + p * L::Q);
+          cp_async_x(ex + r, xv.X + (size_t)unit * B + r);
+          if (kFx && r == 0) cp_async4(ee, xv.E + unit);
+        }
+#pragma unroll
+        for (int k = 0; k < FPG; ++k) {
+          const int f = face_of(k);
+          if (info[k].x < 0) {
+            if (kFx && r == 0 && (G == 1 || g > 0)) ee[f + 1] = kFxNone;
+            continue;
+          }
+          const ST* src = A.face + (size_t)info[k].y * L::KB;
+          ST* dst = eb + L::KD + f * L::KB;
+#pragma unroll 4
+          for (int p = r; p < L::KB / L::Q; p += B) cp_async16(dst + p * L::Q, src + p * L::Q);
+          bool on;
+          int pos = face_first<B>(code[k], r, on);
+          if (!on) pos += S::XO - NF;
+          cp_async_x(ex + (f + 1) * BX + pos, xv.X + (size_t)info[k].x * B + r);
+          if (kFx && r == 0) cp_async4(ee + f + 1, xv.E + info[k].x);
+        }
+      }
+    }
+  };
+
+  int64_t tile = blockIdx.x;
+  unsigned mask = 0, next_mask = 0;                   // the group's faces with a neighbour (and its orientation)
+  auto face_mask = [&](int64_t t) {
+    unsigned m = 0;
+    if constexpr (M::kProduct) {
+#pragma unroll
+      for (int k = 0; k < FPG; ++k)
+        if (info[k].x >= 0) m |= (info[k].x < t * U + slot ? 3u : 1u) << (2 * k);
+    }
+    return m;
+  };
+  int sg = 0;
+  if (tile < ntiles) {
+    load_info(tile);
+    issue(tile, 0);
+    mask = face_mask(tile);
+    if (M::kStages == 2 && tile + gridDim.x < ntiles) load_info(tile + gridDim.x);
+  }
+  asm volatile("cp.async.commit_group;" ::: "memory");
+  for (; tile < ntiles; tile += gridDim.x) {
+    const int64_t unit = tile * U + slot;
+    const bool active = mine && unit < A.n;
+    const bool lead = active && g == 0;
+    const size_t o = (size_t)unit * B + r;
+    const int64_t next = tile + gridDim.x;
+    if constexpr (M::kStages == 2) {
+      if (next < ntiles) {
+        issue(next, sg ^ 1);
+        next_mask = face_mask(next);
+        if (next + gridDim.x < ntiles) load_info(next + gridDim.x);
+      }
+      asm volatile("cp.async.commit_group;\n\tcp.async.wait_group 1;" ::: "memory");
+    } else {
+      asm volatile("cp.async.wait_group 0;" ::: "memory");
+    }
+    if (OP != SYM_SPMV && tid < 2 * U) smax[tid] = 1;
+    __syncthreads();
+    unsigned char* base = sym_sm + sg * M::kStage;
+    const ST* eb = reinterpret_cast<ST*>(base) + slot * M::KE;
+    const SD* sext = reinterpret_cast<SD*>(base + M::kBlk) + slot * M::KX;
+    const SX* ex = reinterpret_cast<SX*>(base + M::kBlk + M::kExt) + slot * M::NX * BX;
+    const int* ee = reinterpret_cast<int*>(base + M::kBlk + M::kExt + M::kXs) + slot * M::NX;
+    T own = T(0), rh = T(0), dv = T(0);               // loaded ahead of their use
+    if (lead) {
+      if (M::kProduct && (KIND == 2 || OP == SYM_CHEB)) own = x[o];
+      if (!(OP == SYM_SPMV && KIND != 1)) rh = rhs[o];
+      if (OP == SYM_CHEB && KIND == 2) dv = d[o];
+    }
+
+    // ---- y = (A0 x)_r
+    T y = T(0);
+    int E = kFxNone;
+    if constexpr (M::kProduct) {
+      Sum sum = Sum(0);
+      if (active) {
+        if constexpr (kFx) {
+          E = ee[0];
+#pragma unroll
+          for (int f = 0; f < NFACE; ++f) E = max(E, ee[f + 1]);
+        }
+        if (g == 0) {
+          Acc acc;
+          sym_tri<T, B>(eb, r, ex, acc);
+          sum = sum_shift(acc.sum(), kFx ? E - ee[0] : 0);
+        }
+        Sum* pp = spart + slot * NFACE * B + r;
+        constexpr int kFaceUnroll = (S::D == 2) ? FPG : 1;
+#pragma unroll kFaceUnroll
+        for (int k = 0; k < FPG; ++k) {
+          if (G > 1 && g == 0) break;
+          const int f = face_of(k);
+          const unsigned m = mask >> (2 * k);
+          if (!(m & 1)) {
+            pp[f * B] = Sum(0);
+            continue;
+          }
+          const bool tr = m & 2;                      // the block is the neighbour's: row of K^T
+          bool on;
+          const int pos = face_first<B>(f, r, on);
+          const ST* F = eb + L::KD + f * L::KB;
+          const ST* Gb = F + NF * S::LDF;
+          const SX* xf = ex + (f + 1) * BX;
+          const int sh = kFx ? E - ee[f + 1] : 0;
+          Acc acc;
+          sym_dot<T, NF>(tr ? (on ? F + pos * S::LDF : Gb + (pos - NF) * S::LDG) : F + pos, tr ? 1 : S::LDF, xf, acc);
+          sum += sum_shift(acc.sum(), sh);
+          // this thread's share of face row j's off-face terms
+          const int j = r % NF, a0 = r / NF * kShare;
+          Acc pa;
+          sym_dot_any<T, kShare>(tr ? F + j * S::LDF + NF + a0 : Gb + a0 * S::LDG + j, tr ? 1 : S::LDG, xf + S::XO + a0, pa);
+          pp[f * B] = sum_shift(pa.sum(), sh);
+        }
+        if (G > 1 && g > 0) sred[(g - 1) * U * B + slot * B + r] = sum;
+      }
+      __syncthreads();
+      if (lead) {
+#pragma unroll
+        for (int k = 0; k < G - 1; ++k) sum += sred[k * U * B + slot * B + r];
+#pragma unroll
+        for (int f = 0; f < NFACE; ++f) {
+          bool on;
+          const int j = face_first<B>(f, r, on);
+          if (on) {
+#pragma unroll
+            for (int a = 0; a < N; ++a) sum += spart[(slot * NFACE + f) * B + a * NF + j];
+          }
+        }
+        if constexpr (kFx) {
+          if (E != kFxBad) y = fx_scale(sum, A.sc[unit] - A.kA + E + kFxBias);
+          else if (OP == SYM_SPMV) y = sym_row_nonfinite<B>(A, unit, r, x);
+          else y = nan("");
+        } else {
+          y = sum;
+        }
+      }
+    }
+
+    if constexpr (OP == SYM_SPMV) {
+      if (lead) {
+        out[o] = (KIND == 1) ? rh - y : y;
+        if (KIND == 2) part += (double)own * (double)y;
+      }
+    } else {
+      // ---- the element's residual t, then its block inverse or P^T
+      const T t = rh - y;
+      int Et = 0;
+      if constexpr (kFx) {
+        if (lead) atomicMax(smax + slot, fx_exp(t));
+        __syncthreads();
+        if (lead) Et = smax[slot];
+      }
+      SX* ts = sts + slot * BX;
+      if (lead) {
+        if constexpr (kFx) ts[r] = fx_split(t, Et);
+        else ts[r] = t;
+      }
+      __syncthreads();
+      T res = T(0);
+      if (lead) {
+        Acc acc;
+        if constexpr (OP == SYM_CHEB) sym_tri<T, B>(sext, r, ts, acc);
+        else sym_dot<T, B>(sext + r * S::LDP, 1, ts, acc);
+        T sv;
+        if constexpr (kFx) sv = Et == 2047 ? nan("") : fx_scale(acc.sum(), Et + kFxBias - ext.k[unit]);
+        else sv = acc.sum();
+        if constexpr (OP == SYM_RESTRICT) {
+          out[o] = sv;
+        } else {
+          const T dn = (KIND == 2) ? c1 * dv + c2 * sv : c2 * sv;
+          d[o] = dn;
+          res = M::kProduct ? own + dn : dn;
+          out[o] = res;
+        }
+      }
+      if constexpr (kFx && OP == SYM_CHEB) {
+        if (lead) atomicMax(smax + U + slot, fx_exp(res));
+        __syncthreads();
+        if (lead) {
+          const int e = smax[U + slot];
+          Xo[o] = fx_split(res, e);
+          if (r == 0) Eo[unit] = e == 2047 ? kFxBad : e + A.sc[unit];
+        }
+      }
+    }
+    __syncthreads();                                  // the stage and the sums are free again
+    if constexpr (M::kStages == 2) {
+      sg ^= 1;
+      mask = next_mask;
+    } else if (next < ntiles) {
+      load_info(next);
+      issue(next, 0);
+      mask = face_mask(next);
+      asm volatile("cp.async.commit_group;" ::: "memory");
+    }
+  }
+  asm volatile("cp.async.wait_group 0;" ::: "memory");
+  if constexpr (OP == SYM_SPMV && KIND == 2) {
+    if (partial_and_last<M::NTH>(part, partials, &st->ticket[0])) {
+      const double pq = sum_partials<M::NTH>(partials, gridDim.x);
+      if (threadIdx.x == 0) {
+        st->pq = pq;
+        st->alpha = st->rho / pq;
+        st->ticket[0] = 0;
+      }
+    }
+  }
+}
+
+// ---------------------------------------------------------------- streaming form (B <= 32)
+// One warp per 32 / B elements, one lane per row; each warp streams its blocks
+// (diagonal, faces, Dinv) through a private ring of NS slots in shared memory,
+// so that NS - 1 blocks are always in flight and no warp waits for another.
+template <typename T, typename TD, int B, int OP, int KIND>
+struct SymRing {
+  using S = SymShape<B>;
+  using ST = typename SymNum<T>::ST;
+  using SX = typename SymNum<T>::SX;
+  using Sum = typename SymNum<T>::Acc::Sum;
+  using SD = typename std::conditional<OP != SYM_CHEB || std::is_same<T, double>::value, ST, TD>::type;
+  using L = SymLay<ST, B>;
+  static constexpr bool kFx = std::is_same<T, double>::value;
+  static constexpr bool kProduct = !(OP == SYM_CHEB && KIND == 0);
+  static constexpr int EPW = 32 / B;
+  static constexpr int K0 = kProduct ? 0 : 1 + S::NFACE;                  // first block of an element
+  static constexpr int K1 = 1 + S::NFACE + (OP == SYM_CHEB ? 1 : 0);      // one past the last
+  static constexpr int NS = kProduct ? SymRingSlots<T, B>::value : 2;     // at most K1 - K0 + 1
+  static constexpr int KM = L::KD > L::KB ? L::KD : L::KB;                // entries of a slot and element
+  static constexpr size_t kSlot = round_to(EPW * (KM * (int)sizeof(ST) + S::BX * (int)sizeof(SX)) + (kFx ? EPW * 4 : 0), 16);
+  static constexpr size_t kWarp = NS * kSlot + round_to(EPW * S::BX * (int)sizeof(Sum), 16);
+  static constexpr int NWARP = SymRingWarps<T, B>::value, NTH = NWARP * 32;
+  static constexpr size_t bytes = NWARP * kWarp;
+};
+
+template <typename T, typename TD, int B, int OP, int KIND>
+static __global__ void __launch_bounds__(SymRing<T, TD, B, OP, KIND>::NTH, SymRingBlocks<T, B>::value)
+    k_symw(SymView<T, B> A, SymBlk<typename SymRing<T, TD, B, OP, KIND>::SD> ext, SymVec<T> xv,
+           const T* __restrict__ rhs, const T* __restrict__ x, T* __restrict__ out, T* __restrict__ d, int2* Xo, int* Eo,
+           T c1, T c2, double* partials, CGState* st) {
+  using M = SymRing<T, TD, B, OP, KIND>;
+  using S = SymShape<B>;
+  using ST = typename M::ST;
+  using SD = typename M::SD;
+  using SX = typename M::SX;
+  using Sum = typename M::Sum;
+  using Acc = typename SymNum<T>::Acc;
+  using L = typename M::L;
+  constexpr int EPW = M::EPW, NFACE = S::NFACE, BX = S::BX, NF = S::NF, BO = S::BO, N = S::N, NS = M::NS;
+  constexpr int K0 = M::K0, K1 = M::K1, NB = K1 - K0;
+  constexpr bool kFx = M::kFx;
+  constexpr int kShare = BO / N;                      // off-face terms of a face row per lane
+  if (st && st->done) return;
+  extern __shared__ __align__(16) unsigned char sym_sm[];
+  const int lane = threadIdx.x & 31;
+  const int sub = lane / B, r = lane - sub * B;
+  const bool in = sub < EPW;
+  unsigned char* wsm = sym_sm + (threadIdx.x >> 5) * M::kWarp;
+  Sum* part = reinterpret_cast<Sum*>(wsm + NS * M::kSlot) + sub * BX;
+  auto slot_blk = [&](int s) { return reinterpret_cast<ST*>(wsm + s * M::kSlot) + sub * M::KM; };
+  auto slot_x = [&](int s) { return reinterpret_cast<SX*>(wsm + s * M::kSlot + EPW * M::KM * sizeof(ST)) + sub * BX; };
+  auto slot_e = [&](int s) {
+    return reinterpret_cast<int*>(wsm + s * M::kSlot + EPW * (M::KM * sizeof(ST) + BX * sizeof(SX))) + sub;
+  };
+  const int64_t ntiles = (A.n + EPW - 1) / EPW;
+  const int64_t gw = ((int64_t)blockIdx.x * M::NTH + threadIdx.x) >> 5, nw = ((int64_t)gridDim.x * M::NTH) >> 5;
+  // lanes 0 .. 2d-1 of an element hold the neighbour and face block of its faces
+  auto load_info = [&](int64_t tile, int2& in_, int& code_) {
+    in_ = make_int2(-1, 0);
+    code_ = 0;
+    const int64_t unit = tile * EPW + sub;
+    if (M::kProduct && in && unit < A.n && r < NFACE) {
+      in_ = A.info[unit * NFACE + r];
+      code_ = A.code[unit * NFACE + r];
+    }
+  };
+  auto issue = [&](int64_t tile, int k, int2 ti, int tc, int s) {
+    const int64_t unit = tile * EPW + sub;
+    ST* dst = slot_blk(s);
+    if (k == 0) {
+      if (in && unit < A.n) {
+        const ST* src = A.diag + (size_t)unit * L::KD;
+#pragma unroll
+        for (int p = 0; p < (L::KD / L::Q + B - 1) / B; ++p)
+          if (p * B + r < L::KD / L::Q) cp_async16(dst + (p * B + r) * L::Q, src + (p * B + r) * L::Q);
+        cp_async_x(slot_x(s) + r, xv.X + (size_t)unit * B + r);
+        if (kFx && r == 0) cp_async4(slot_e(s), xv.E + unit);
+      }
+    } else if (k <= NFACE) {
+      const int from = in ? sub * B + k - 1 : 0;
+      const int nb = __shfl_sync(0xffffffffu, ti.x, from), id = __shfl_sync(0xffffffffu, ti.y, from);
+      const int fn = __shfl_sync(0xffffffffu, tc, from);
+      if (in && unit < A.n && nb >= 0) {
+        const ST* src = A.face + (size_t)id * L::KB;
+#pragma unroll
+        for (int p = 0; p < (L::KB / L::Q + B - 1) / B; ++p)
+          if (p * B + r < L::KB / L::Q) cp_async16(dst + (p * B + r) * L::Q, src + (p * B + r) * L::Q);
+        bool on;
+        int pos = face_first<B>(fn, r, on);
+        if (!on) pos += S::XO - NF;
+        cp_async_x(slot_x(s) + pos, xv.X + (size_t)nb * B + r);
+        if (kFx && r == 0) cp_async4(slot_e(s), xv.E + nb);
+      }
+    } else if constexpr (OP == SYM_CHEB) {
+      if (in && unit < A.n) {
+        constexpr int KX = SymLay<SD, B>::KD, QD = 16 / (int)sizeof(SD);
+        const SD* src = ext.v + (size_t)unit * KX;
+        SD* dd = reinterpret_cast<SD*>(dst);
+#pragma unroll
+        for (int p = 0; p < (KX / QD + B - 1) / B; ++p)
+          if (p * B + r < KX / QD) cp_async16(dd + (p * B + r) * QD, src + (p * B + r) * QD);
+      }
+    }
+  };
+
+  int2 ic, in1, in2;
+  int cc, cn1, cn2;
+  load_info(gw, ic, cc);
+  load_info(gw + nw, in1, cn1);
+  int slot = 0;
+#pragma unroll
+  for (int j = 0; j < NS - 1; ++j) {
+    if (j < NB) {
+      if (gw < ntiles) issue(gw, K0 + j, ic, cc, j);
+    } else if (gw + nw < ntiles) {
+      issue(gw + nw, K0 + j - NB, in1, cn1, j);
+    }
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  }
+  double dot = 0.0;
+  const unsigned emask = (B == 27) ? 0x07ffffffu : (((1u << (B & 31)) - 1u) << (in ? sub * B : 0));
+  for (int64_t tile = gw; tile < ntiles; tile += nw) {
+    const int64_t unit = tile * EPW + sub;
+    const bool active = in && unit < A.n;
+    const size_t o = (size_t)unit * B + r;
+    load_info(tile + 2 * nw, in2, cn2);
+    T own = T(0), rh = T(0), dv = T(0);
+    int se = 0;
+    if (active) {
+      if (M::kProduct && (KIND == 2 || OP == SYM_CHEB)) own = x[o];
+      if (!(OP == SYM_SPMV && KIND != 1)) rh = rhs[o];
+      if (OP == SYM_CHEB && KIND == 2) dv = d[o];
+      if (kFx) se = A.sc[unit];
+    }
+    Sum sum = Sum(0);
+    int E = kFxNone;
+    T res = T(0);
+    constexpr int kBlkUnroll = (S::D == 2) ? NB : 1;
+#pragma unroll kBlkUnroll
+    for (int k = K0; k < K1; ++k) {
+      {
+        // keep NS - 1 blocks in flight
+        const int ka = k + NS - 1, sa = slot == 0 ? NS - 1 : slot - 1;
+        if (ka < K1) issue(tile, ka, ic, cc, sa);
+        else if (tile + nw < ntiles) issue(tile + nw, ka - NB, in1, cn1, sa);
+        asm volatile("cp.async.commit_group;\n\tcp.async.wait_group %0;" ::"n"(NS - 1) : "memory");
+        __syncwarp();
+      }
+      const ST* blk = slot_blk(slot);
+      const SX* xs = slot_x(slot);
+      if (k == 0) {
+        if (active) {
+          Acc acc;
+          sym_tri<T, B>(blk, r, xs, acc);
+          sum = acc.sum();
+          if constexpr (kFx) E = *slot_e(slot);
+        }
+      } else if (k <= NFACE) {
+        const int f = k - 1;
+        const int nb = __shfl_sync(0xffffffffu, ic.x, in ? sub * B + f : 0);
+        const bool have = active && nb >= 0;
+        bool on = false;
+        int pos = 0;
+        Sum s = Sum(0);
+        if (have) {
+          pos = face_first<B>(f, r, on);
+          const ST* F = blk;
+          const ST* Gb = F + NF * S::LDF;
+          const bool tr = nb < unit;                  // the block is the neighbour's: row of K^T
+          Acc acc;
+          sym_dot<T, NF>(tr ? (on ? F + pos * S::LDF : Gb + (pos - NF) * S::LDG) : F + pos, tr ? 1 : S::LDF, xs, acc);
+          s = acc.sum();
+          // this lane's share of face row j's off-face terms
+          const int j = r % NF, a0 = r / NF * kShare;
+          Acc pa;
+          sym_dot_any<T, kShare>(tr ? F + j * S::LDF + NF + a0 : Gb + a0 * S::LDG + j, tr ? 1 : S::LDG, xs + S::XO + a0, pa);
+          part[r] = pa.sum();
+        }
+        __syncwarp();
+        if (have) {
+          if (on) {
+#pragma unroll
+            for (int a = 0; a < N; ++a) s += part[a * NF + pos];
+          }
+          if constexpr (kFx) {
+            const int e = *slot_e(slot);
+            if (e > E) {
+              sum = sum_shift(sum, e - E) + s;
+              E = e;
+            } else {
+              sum += sum_shift(s, E - e);
+            }
+          } else {
+            sum += s;
+          }
+        }
+      }
+      if (k == NFACE || !M::kProduct) {
+        // ---- the row's product, and what the operation makes of it
+        T y = T(0);
+        if (M::kProduct && active) {
+          if constexpr (kFx) {
+            if (E < kFxBad / 2) y = fx_scale(sum, se - A.kA + E + kFxBias);
+            else if (OP == SYM_SPMV) y = sym_row_nonfinite<B>(A, unit, r, x);
+            else y = nan("");
+          } else {
+            y = sum;
+          }
+        }
+        if constexpr (OP == SYM_SPMV) {
+          if (active) {
+            out[o] = (KIND == 1) ? rh - y : y;
+            if (KIND == 2) dot += (double)own * (double)y;
+          }
+        } else {
+          res = rh - y;                               // the residual's row
+        }
+      }
+      if constexpr (OP != SYM_SPMV) {
+        if (k == K1 - 1) {
+          const T t = res;
+          int Et = 0;
+          SX* ts = reinterpret_cast<SX*>(part);
+          __syncwarp();
+          if (active) {
+            if constexpr (kFx) {
+              Et = __reduce_max_sync(emask, fx_exp(t));
+              ts[r] = fx_split(t, Et);
+            } else {
+              ts[r] = t;
+            }
+          }
+          __syncwarp();
+          if (active) {
+            Acc acc;
+            if constexpr (OP == SYM_CHEB) {
+              sym_tri<T, B>(reinterpret_cast<const SD*>(blk), r, ts, acc);
+            } else {
+              const ST* p = ext.v + (size_t)unit * L::KP + r;
+#pragma unroll
+              for (int i = 0; i < B; ++i) acc.fma(__ldcs(p + i * S::LDP), ts[i]);
+            }
+            T sv;
+            if constexpr (kFx) sv = Et == 2047 ? nan("") : fx_scale(acc.sum(), Et + kFxBias - ext.k[unit]);
+            else sv = acc.sum();
+            if constexpr (OP == SYM_RESTRICT) {
+              out[o] = sv;
+            } else {
+              const T dn = (KIND == 2) ? c1 * dv + c2 * sv : c2 * sv;
+              d[o] = dn;
+              const T xn = M::kProduct ? own + dn : dn;
+              out[o] = xn;
+              if constexpr (kFx) {
+                const int e = __reduce_max_sync(emask, fx_exp(xn));
+                Xo[o] = fx_split(xn, e);
+                if (r == 0) Eo[unit] = e == 2047 ? kFxBad : e + se;
+              }
+            }
+          }
+        }
+      }
+      __syncwarp();                                   // the slot is free again
+      slot = slot + 1 == NS ? 0 : slot + 1;
+    }
+    ic = in1;
+    cc = cn1;
+    in1 = in2;
+    cn1 = cn2;
+  }
+  asm volatile("cp.async.wait_group 0;" ::: "memory");
+  if constexpr (OP == SYM_SPMV && KIND == 2) {
+    if (partial_and_last<M::NTH>(dot, partials, &st->ticket[0])) {
+      const double pq = sum_partials<M::NTH>(partials, gridDim.x);
+      if (threadIdx.x == 0) {
+        st->pq = pq;
+        st->alpha = st->rho / pq;
+        st->ticket[0] = 0;
+      }
+    }
+  }
+}
+
+// Threads of the element-wise kernels below: U whole elements per block.
+template <int B> struct SymRows {
+  static constexpr int U = (B <= 64) ? 128 / B : 1, NT = round_to(U * B, 32);
+};
+
+// Level-0 prolongation x_u += P_u e_{parent(u)}, one thread per (element, row):
+// a row's entries of consecutive columns lie LDP apart, so the threads of an
+// element read each column contiguously, straight from HBM (no reuse).
+template <typename T, int B>
+static __global__ void __launch_bounds__(SymRows<B>::NT)
+    k_sym_prolong(SymBlk<typename SymNum<T>::ST> P, const int32_t* __restrict__ parent, const T* __restrict__ ec,
+                  T* __restrict__ x, const int16_t* __restrict__ sc, int2* Xo, int* Eo, int64_t n, const CGState* st) {
+  if (st && st->done) return;
+  using S = SymShape<B>;
+  using ST = typename SymNum<T>::ST;
+  using SX = typename SymNum<T>::SX;
+  constexpr int KP = SymLay<ST, B>::KP, U = SymRows<B>::U, BX = (B + 1) / 2 * 2;
+  constexpr bool kFx = std::is_same<T, double>::value;
+  __shared__ __align__(16) SX sx[U * BX];
+  __shared__ int smax[U];
+  const int slot = threadIdx.x / B, r = threadIdx.x - slot * B;
+  const int64_t unit = (int64_t)blockIdx.x * U + slot;
+  const bool active = slot < U && unit < n;
+  T e = T(0);
+  if (active) e = ec[(size_t)parent[unit] * B + r];
+  int E = 0;
+  if constexpr (kFx) {
+    if (threadIdx.x < U) smax[threadIdx.x] = 1;
+    __syncthreads();
+    if (active) atomicMax(smax + slot, fx_exp(e));
+    __syncthreads();
+    if (active) {
+      E = smax[slot];
+      sx[slot * BX + r] = fx_split(e, E);
+    }
+  } else {
+    if (active) sx[slot * BX + r] = e;
+  }
+  __syncthreads();
+  T v = T(0);
+  if (active) {
+    const ST* p = P.v + (size_t)unit * KP + r;
+    typename SymNum<T>::Acc acc;
+    constexpr int kUnroll = (B <= 27) ? B : 16;
+#pragma unroll kUnroll
+    for (int j = 0; j < B; ++j) acc.fma(__ldcs(p + j * S::LDP), sx[slot * BX + j]);
+    T s;
+    if constexpr (kFx) s = E == 2047 ? nan("") : fx_scale(acc.sum(), E + kFxBias - P.k[unit]);
+    else s = acc.sum();
+    v = x[(size_t)unit * B + r] + s;
+    x[(size_t)unit * B + r] = v;
+  }
+  if constexpr (kFx) fx_store<B>(v, active, slot, unit, r, sc, Xo, Eo, smax, U);
+}
+
+// x's fixed-point copy
+template <int B>
+static __global__ void __launch_bounds__(SymRows<B>::NT)
+    k_fx(const double* __restrict__ x, int64_t n, const int16_t* __restrict__ sc, int2* __restrict__ X,
+         int* __restrict__ E, const CGState* st) {
+  if (st && st->done) return;
+  __shared__ int se[SymRows<B>::U];
+  const int slot = threadIdx.x / B, r = threadIdx.x - slot * B;
+  const int64_t unit = (int64_t)blockIdx.x * SymRows<B>::U + slot;
+  const bool active = slot < SymRows<B>::U && unit < n;
+  fx_store<B>(active ? x[(size_t)unit * B + r] : 0.0, active, slot, unit, r, sc, X, E, se, SymRows<B>::U);
+}
+// p = z + beta p (INIT: p = z), as k_pupd, with p's fixed-point copy
+template <int B, bool INIT>
+static __global__ void __launch_bounds__(SymRows<B>::NT)
+    k_pupd_fx(const double* __restrict__ z, double* __restrict__ p, int64_t n, const int16_t* __restrict__ sc,
+              int2* __restrict__ X, int* __restrict__ E, const CGState* st) {
+  if (st->done) return;
+  __shared__ int se[SymRows<B>::U];
+  const int slot = threadIdx.x / B, r = threadIdx.x - slot * B;
+  const int64_t unit = (int64_t)blockIdx.x * SymRows<B>::U + slot;
+  const bool active = slot < SymRows<B>::U && unit < n;
+  const size_t o = (size_t)unit * B + r;
+  double v = 0.0;
+  if (active) {
+    v = INIT ? z[o] : z[o] + st->beta * p[o];
+    p[o] = v;
+  }
+  fx_store<B>(v, active, slot, unit, r, sc, X, E, se, SymRows<B>::U);
+}
+
+}  // namespace aggmg
