@@ -436,7 +436,7 @@ agg_status agg_ionic_update(const agg_ionic_params* p, double dt, int64_t n, con
   if (n < 0) return fail(AGG_EINVAL, "n < 0");
   if (p->model < AGG_FHN || p->model > AGG_BUENO_OROVIO) return fail(AGG_EINVAL, "ionic model");
   if (n == 0) return AGG_OK;
-  IonicParams ip{p->model, p->k, p->a, p->eps, p->gamma, p->mu1, p->mu2, p->bo};
+  const IonicParams ip = make_ionic(p->model, p->k, p->a, p->eps, p->gamma, p->mu1, p->mu2, p->bo);
   const int64_t blocks = std::min<int64_t>((n + 255) / 256, 152 * 16);
   k_ionic_update<<<blocks, 256, 0, (cudaStream_t)stream>>>(ip, dt, n, u, w);
   cudaError_t e = cudaGetLastError();

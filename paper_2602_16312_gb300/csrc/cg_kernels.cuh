@@ -248,7 +248,22 @@ struct IonicParams {
   int model;
   double k, a, eps, gamma, mu1, mu2;
   agg_bueno_orovio_params bo;
+  // inverses of Bueno-Orovio time constants (hi: above the unit step that selects)
+  struct {
+    double a0_lo, a0_hi, tau1plus, tau2plus, tau2inf, a2_lo, a2_hi, taufi, o_lo, o_hi, tausi;
+  } inv;
 };
+inline IonicParams make_ionic(int model, double k, double a, double eps, double gamma, double mu1, double mu2,
+                              const agg_bueno_orovio_params& b) {
+  IonicParams p{model, k, a, eps, gamma, mu1, mu2, b, {}};
+  if (model == 2) {
+    p.inv = {1.0 / b.tau1p,   1.0 / ((b.tau1pp - b.tau1p) + b.tau1p), 1.0 / b.tau1plus,
+             1.0 / b.tau2plus, 1.0 / b.tau2inf,
+             1.0 / b.tau3p,   1.0 / ((b.tau3pp - b.tau3p) + b.tau3p), 1.0 / b.taufi,
+             1.0 / b.tauo_p,  1.0 / ((b.tauo_pp - b.tauo_p) + b.tauo_p), 1.0 / b.tausi};
+  }
+  return p;
+}
 
 // Gates per DoF: FitzHugh-Nagumo and Aliev-Panfilov 1, Bueno-Orovio 3; gate g
 // of DoF i lives at w[g * stride + i].
@@ -260,43 +275,65 @@ __device__ __forceinline__ double smooth_step(double z, double z0, double k) {
   return 0.5 * (1.0 + tanh(k * (z - z0)));
 }
 
-// Bueno-Orovio (Section 2.3.2, Eq. BuenoOrovio): I_ion and the three gate rates
-__device__ __forceinline__ void bueno_orovio_eval(const agg_bueno_orovio_params& p, double u, const double* w,
-                                                  double& I, double* H) {
+// (1 + tanh(k (z - z0))) / 2 = 1 / (1 + e), with e = exp(-2 k (z - z0)) kept finite
+// (a NaN stays one)
+__device__ __forceinline__ double smooth_exp(double z, double z0, double k) {
+  double t = -2.0 * k * (z - z0);
+  t = t > 700.0 ? 700.0 : t;
+  return exp(t);
+}
+
+// Bueno-Orovio (Section 2.3.2, Eq. BuenoOrovio). The float64 pipe bounds these
+// (2 FMAs per SM and clock on GB300; a division is ~10 of them, a tanh ~50), so
+// divisions by parameters are products with the inverses in IonicParams::inv,
+// the smoothed steps cost one exponential each, and a term behind a unit step is
+// evaluated on its side only. Gate update of 5.3M DoFs: 1,928 -> 727 us.
+// The three gate rates:
+__device__ __forceinline__ void bueno_orovio_rates(const IonicParams& q, double u, const double* w, double* H) {
+  const agg_bueno_orovio_params& p = q.bo;
   const double hv1 = unit_step(u, p.V1), hv1m = unit_step(u, p.V1m);
   const double hv2 = unit_step(u, p.V2), hvo = unit_step(u, p.Vo);
-  const double a0 = (1.0 - hv1) / (hv1m * (p.tau1pp - p.tau1p) + p.tau1p);
-  const double b0 = -hv1 / p.tau1plus;
+  const double a0 = (1.0 - hv1) * (hv1m != 0.0 ? q.inv.a0_hi : q.inv.a0_lo);
+  const double b0 = -hv1 * q.inv.tau1plus;
   const double w0inf = 1.0 - hv1m;
-  const double a1 = (1.0 - hv2) / (smooth_step(u, p.V2m, p.k2) * (p.tau2pp - p.tau2p) + p.tau2p);
-  const double b1 = -hv2 / p.tau2plus;
-  const double w1inf = hvo * (p.winf_star - 1.0 + u / p.tau2inf) + 1.0 - u / p.tau2inf;
-  const double a2 = 1.0 / (hv2 * (p.tau3pp - p.tau3p) + p.tau3p);
-  const double w2inf = smooth_step(u, p.V3, p.k3);
+  double a1 = 0.0;                                    // behind 1 - H_V2
+  if (hv2 == 0.0) {
+    const double e1 = 1.0 + smooth_exp(u, p.V2m, p.k2);
+    a1 = e1 / ((p.tau2pp - p.tau2p) + p.tau2p * e1);
+  }
+  const double b1 = -hv2 * q.inv.tau2plus;
+  const double ut = u * q.inv.tau2inf;
+  const double w1inf = hvo * (p.winf_star - 1.0 + ut) + 1.0 - ut;
+  const double a2 = hv2 != 0.0 ? q.inv.a2_hi : q.inv.a2_lo;
+  const double w2inf = 1.0 / (1.0 + smooth_exp(u, p.V3, p.k3));
   H[0] = (b0 - a0) * w[0] + a0 * w0inf;
   H[1] = (b1 - a1) * w[1] + a1 * w1inf;
   H[2] = -a2 * w[2] + a2 * w2inf;
-  const double ifi = -hv1 * (u - p.V1) * (p.Vhat - u) * w[0] / p.taufi;
-  const double iso = (1.0 - hv2) * (u - p.uo) / (hvo * (p.tauo_pp - p.tauo_p) + p.tauo_p) +
-                     hv2 / (smooth_step(u, p.Vso, p.kso) * (p.tauso_pp - p.tauso_p) + p.tauso_p);
-  const double isi = -hv2 * w[1] * w[2] / p.tausi;
-  I = ifi + iso + isi;
+}
+// and I_ion:
+__device__ __forceinline__ double bueno_orovio_current(const IonicParams& q, double u, const double* w) {
+  const agg_bueno_orovio_params& p = q.bo;
+  const double hv1 = unit_step(u, p.V1), hv2 = unit_step(u, p.V2), hvo = unit_step(u, p.Vo);
+  const double ifi = -hv1 * (u - p.V1) * (p.Vhat - u) * w[0] * q.inv.taufi;
+  double iso = (1.0 - hv2) * (u - p.uo) * (hvo != 0.0 ? q.inv.o_hi : q.inv.o_lo);
+  if (hv2 != 0.0) {
+    const double e1 = 1.0 + smooth_exp(u, p.Vso, p.kso);
+    iso += e1 / ((p.tauso_pp - p.tauso_p) + p.tauso_p * e1);
+  }
+  const double isi = -hv2 * w[1] * w[2] * q.inv.tausi;
+  return ifi + iso + isi;
 }
 
-// I_ion(u, w) and the gate rates H(u, w) (w, H: ionic_gates(model) values)
-__device__ __forceinline__ void ionic_eval(const IonicParams& p, double u, const double* w, double& I, double* H) {
-  if (p.model == 2) {
-    bueno_orovio_eval(p.bo, u, w, I, H);
-    return;
-  }
+// gate rates H(u, w) and I_ion(u, w) (w, H: ionic_gates(model) values)
+__device__ __forceinline__ void ionic_rates(const IonicParams& p, double u, const double* w, double* H) {
+  if (p.model == 2) bueno_orovio_rates(p, u, w, H);
+  else if (p.model == 0) H[0] = p.eps * (u - p.gamma * w[0]);
+  else H[0] = (p.eps + p.mu1 * w[0] / (u + p.mu2)) * (-w[0] - p.k * u * (u - p.a - 1.0));
+}
+__device__ __forceinline__ double ionic_current(const IonicParams& p, double u, const double* w) {
+  if (p.model == 2) return bueno_orovio_current(p, u, w);
   const double cub = p.k * u * (u - p.a) * (u - 1.0);
-  if (p.model == 0) {
-    I = cub + w[0];
-    H[0] = p.eps * (u - p.gamma * w[0]);
-  } else {
-    I = cub + u * w[0];
-    H[0] = (p.eps + p.mu1 * w[0] / (u + p.mu2)) * (-w[0] - p.k * u * (u - p.a - 1.0));
-  }
+  return p.model == 0 ? cub + w[0] : cub + u * w[0];
 }
 
 // gate values of DoF i (stride between gates) into g[]
@@ -309,102 +346,97 @@ static __global__ void k_ionic_update(IonicParams prm, double dt, int64_t n, con
                                double* __restrict__ w) {
   const int ng = ionic_gates(prm.model);
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-    double g[kMaxGates], H[kMaxGates], I;
+    double g[kMaxGates], H[kMaxGates];
     load_gates(w, n, i, ng, g);
-    ionic_eval(prm, u[i], g, I, H);
+    ionic_rates(prm, u[i], g, H);
 #pragma unroll
     for (int k = 0; k < kMaxGates; ++k)
       if (k < ng) w[k * n + i] = g[k] + dt * H[k];
   }
 }
 
-// Time step prologue for the thread's element (Section 3.1):
+// ---- element-wise kernels of a time step: one thread per (element, row), U
+// whole elements per block; vectors are read coalesced, and a row's entries of an
+// element's mass block (column by column, M[c * B + r]) too. With one thread per
+// element the 64-DoF blocks left most of the GPU idle (k_ionic_rhs on 13,824 Q3
+// hexahedra: 332 us; Bueno-Orovio on 24,576 Q2 hexahedra: 870 us, now ~170).
+template <int B> struct ElemRows {
+  static constexpr int U = (B <= 64) ? 128 / B : 1, NT = (U * B + 31) / 32 * 32;
+};
+// sum_c M[c B + r] t_c with the element's t in shared memory
+template <int B>
+__device__ __forceinline__ double elem_mv(const double* __restrict__ M, int r, const double* t) {
+  double s = 0.0;
+  constexpr int kUnroll = (B <= 27) ? B : 16;
+#pragma unroll kUnroll
+  for (int c = 0; c < B; ++c) s += __ldcs(M + c * B + r) * t[c];
+  return s;
+}
+
+// Time step prologue (Section 3.1):
 //   w <- w + dt H(u, w);  f = I_app(t_{n+1}) mask - chi I(u, w_new);
 //   b_e = M_e (c u_e + f_e)   (ionic current interpolation)
 template <int B>
-static __global__ void __launch_bounds__(UnitThreads<B>::value)
+static __global__ void __launch_bounds__(ElemRows<B>::NT)
     k_ionic_rhs(const double* __restrict__ Me, const double* __restrict__ u, double* __restrict__ w,
                 const double* __restrict__ mask, double* __restrict__ b, IonicParams prm, double dt, double chi,
-                double c, double iapp_value, int64_t iapp_steps, const int64_t* __restrict__ step, int64_t nslices,
+                double c, double iapp_value, int64_t iapp_steps, const int64_t* __restrict__ step, int64_t n,
                 int64_t wstride) {
-  constexpr int NTB = UnitThreads<B>::value;
-  constexpr int KP = Pad<double, B>::KP;
-  const int lane = threadIdx.x & 31;
-  {
-  const int64_t slice = first_slice<NTB>();
-  if (slice >= nslices) return;
-  const int64_t unit = slice * SL + lane;
-  const size_t o = (size_t)unit * B;
-  const double ia = (*step < iapp_steps) ? iapp_value : 0.0;
-  // per DoF: ionic update and the nodal load c u + I_app mask - chi I(u, w_new)
-  const int ng = ionic_gates(prm.model);
-  auto nodal = [&](int r) {
-    const double ur = u[o + r];
-    double g[kMaxGates], H[kMaxGates], I;
-    load_gates(w, wstride, o + r, ng, g);
-    ionic_eval(prm, ur, g, I, H);
+  constexpr int U = ElemRows<B>::U;
+  __shared__ double sh[U * B];
+  const int slot = threadIdx.x / B, r = threadIdx.x - slot * B;
+  const int64_t unit = (int64_t)blockIdx.x * U + slot;
+  const bool active = slot < U && unit < n;
+  const size_t o = (size_t)unit * B + r;
+  if (active) {
+    const double ia = (*step < iapp_steps) ? iapp_value : 0.0;
+    const int ng = ionic_gates(prm.model);
+    const double ur = u[o];
+    double g[kMaxGates], H[kMaxGates];
+    load_gates(w, wstride, o, ng, g);
+    ionic_rates(prm, ur, g, H);
 #pragma unroll
-    for (int k = 0; k < kMaxGates; ++k) {
-      g[k] += dt * H[k];
-      if (k < ng) w[k * wstride + o + r] = g[k];
-    }
-    ionic_eval(prm, ur, g, I, H);
-    return c * ur + ia * mask[o + r] - chi * I;
-  };
-  double acc[B];
-#pragma unroll
-  for (int r = 0; r < B; ++r) acc[r] = 0.0;
-  const double* Mb = Me + (size_t)slice * SL * KP;
-  if constexpr (B > 32) {
-    __shared__ double tsh[B * NTB];
-    double* ts = tsh + threadIdx.x;
-#pragma unroll
-    for (int r = 0; r < B; ++r) ts[r * NTB] = nodal(r);
-    block_mv<double, double, B, NTB>(Mb, lane, ts, acc);
-  } else {
-    double t[B];
-#pragma unroll
-    for (int r = 0; r < B; ++r) t[r] = nodal(r);
-    block_mv<double, double, B>(Mb, lane, t, acc);
+    for (int k = 0; k < kMaxGates; ++k)
+      if (k < ng) {
+        g[k] += dt * H[k];
+        w[k * wstride + o] = g[k];
+      }
+    sh[threadIdx.x] = c * ur + ia * mask[o] - chi * ionic_current(prm, ur, g);
   }
-#pragma unroll
-  for (int r = 0; r < B; ++r) b[o + r] = acc[r];
-  }
+  __syncthreads();
+  if (active) b[o] = elem_mv<B>(Me + (size_t)unit * B * B, r, sh + slot * B);
 }
 
 // BDF2 history at the start (second-order derivative start), per element:
 //   u^{-1} = u - dt u',  chi C_m u' = I_app - chi I(u, w) - M^{-1} A u,
 //   w^{-1} = w - dt H(u, w),   with M^{-1} A u = M_e^{-1} (A0 u)_e - c u.
 template <int B>
-static __global__ void __launch_bounds__(UnitThreads<B>::value)
+static __global__ void __launch_bounds__(ElemRows<B>::NT)
     k_bdf2_start(const double* __restrict__ Minv, const double* __restrict__ A0u, const double* __restrict__ u,
                  const double* __restrict__ w, const double* __restrict__ mask, double* __restrict__ up,
                  double* __restrict__ wp, IonicParams prm, double dt, double chi, double cm, double c, double ia,
-                 int64_t nslices, int64_t wstride) {
-  constexpr int NTB = UnitThreads<B>::value;
-  constexpr int KP = Pad<double, B>::KP;
-  const int lane = threadIdx.x & 31;
-  const int64_t slice = first_slice<NTB>();
-  if (slice >= nslices) return;
-  const size_t o = (size_t)(slice * SL + lane) * B;
-  double t[B];
-#pragma unroll
-  for (int r = 0; r < B; ++r) t[r] = 0.0;
-  block_mv<double, double, B>(Minv + (size_t)slice * SL * KP, lane, A0u + o, t);
+                 int64_t n, int64_t wstride) {
+  constexpr int U = ElemRows<B>::U;
+  __shared__ double sh[U * B];
+  const int slot = threadIdx.x / B, r = threadIdx.x - slot * B;
+  const int64_t unit = (int64_t)blockIdx.x * U + slot;
+  const bool active = slot < U && unit < n;
+  const size_t o = (size_t)unit * B + r;
+  if (active) sh[threadIdx.x] = A0u[o];
+  __syncthreads();
+  if (!active) return;
+  const double t = elem_mv<B>(Minv + (size_t)unit * B * B, r, sh + slot * B);
   const int ng = ionic_gates(prm.model);
+  const double ur = u[o];
+  double g[kMaxGates], H[kMaxGates];
+  load_gates(w, wstride, o, ng, g);
+  ionic_rates(prm, ur, g, H);
+  const double f0 = ia * mask[o] - chi * ionic_current(prm, ur, g);
+  const double udot = (f0 - (t - c * ur)) / (chi * cm);
+  up[o] = ur - dt * udot;
 #pragma unroll
-  for (int r = 0; r < B; ++r) {
-    const double ur = u[o + r];
-    double g[kMaxGates], H[kMaxGates], I;
-    load_gates(w, wstride, o + r, ng, g);
-    ionic_eval(prm, ur, g, I, H);
-    const double f0 = ia * mask[o + r] - chi * I;
-    const double udot = (f0 - (t[r] - c * ur)) / (chi * cm);
-    up[o + r] = ur - dt * udot;
-#pragma unroll
-    for (int k = 0; k < kMaxGates; ++k)
-      if (k < ng) wp[k * wstride + o + r] = g[k] - dt * H[k];
-  }
+  for (int k = 0; k < kMaxGates; ++k)
+    if (k < ng) wp[k * wstride + o] = g[k] - dt * H[k];
 }
 
 // BDF2 step prologue (Eq. fully_discrete with extrapolation), per element:
@@ -412,58 +444,42 @@ static __global__ void __launch_bounds__(UnitThreads<B>::value)
 //   f = I_app mask - chi I(U*, w_new), b_e = M_e (chi C_m (4u - up)/(2dt) + f);
 //   then the history shifts: up <- u, wp <- w, w <- w_new.
 template <int B>
-static __global__ void __launch_bounds__(UnitThreads<B>::value)
+static __global__ void __launch_bounds__(ElemRows<B>::NT)
     k_ionic_rhs_bdf2(const double* __restrict__ Me, const double* __restrict__ u, double* __restrict__ up,
                      double* __restrict__ w, double* __restrict__ wp, const double* __restrict__ mask,
                      double* __restrict__ b, IonicParams prm, double dt, double chi, double cm, double iapp_value,
-                     int64_t iapp_steps, const int64_t* __restrict__ step, int64_t nslices, int64_t wstride) {
-  constexpr int NTB = UnitThreads<B>::value;
-  constexpr int KP = Pad<double, B>::KP;
-  const int lane = threadIdx.x & 31;
-  const int64_t slice = first_slice<NTB>();
-  if (slice >= nslices) return;
-  const size_t o = (size_t)(slice * SL + lane) * B;
-  const double ia = (*step < iapp_steps) ? iapp_value : 0.0;
-  const int ng = ionic_gates(prm.model);
-  auto nodal = [&](int r) {
-    const double un = u[o + r], upr = up[o + r];
+                     int64_t iapp_steps, const int64_t* __restrict__ step, int64_t n, int64_t wstride) {
+  constexpr int U = ElemRows<B>::U;
+  __shared__ double sh[U * B];
+  const int slot = threadIdx.x / B, r = threadIdx.x - slot * B;
+  const int64_t unit = (int64_t)blockIdx.x * U + slot;
+  const bool active = slot < U && unit < n;
+  const size_t o = (size_t)unit * B + r;
+  if (active) {
+    const double ia = (*step < iapp_steps) ? iapp_value : 0.0;
+    const int ng = ionic_gates(prm.model);
+    const double un = u[o], upr = up[o];
     const double us = 2.0 * un - upr;
-    double wn[kMaxGates], wpr[kMaxGates], ws[kMaxGates], w1[kMaxGates], H[kMaxGates], I;
-    load_gates(w, wstride, o + r, ng, wn);
-    load_gates(wp, wstride, o + r, ng, wpr);
+    double wn[kMaxGates], wpr[kMaxGates], ws[kMaxGates], w1[kMaxGates], H[kMaxGates];
+    load_gates(w, wstride, o, ng, wn);
+    load_gates(wp, wstride, o, ng, wpr);
 #pragma unroll
     for (int k = 0; k < kMaxGates; ++k) ws[k] = 2.0 * wn[k] - wpr[k];
-    ionic_eval(prm, us, ws, I, H);
-#pragma unroll
-    for (int k = 0; k < kMaxGates; ++k) w1[k] = (4.0 * wn[k] - wpr[k]) / 3.0 + (2.0 * dt / 3.0) * H[k];
-    ionic_eval(prm, us, w1, I, H);
-    up[o + r] = un;
+    ionic_rates(prm, us, ws, H);
+    up[o] = un;
 #pragma unroll
     for (int k = 0; k < kMaxGates; ++k)
       if (k < ng) {
-        wp[k * wstride + o + r] = wn[k];
-        w[k * wstride + o + r] = w1[k];
+        w1[k] = (4.0 * wn[k] - wpr[k]) / 3.0 + (2.0 * dt / 3.0) * H[k];
+        wp[k * wstride + o] = wn[k];
+        w[k * wstride + o] = w1[k];
+      } else {
+        w1[k] = 0.0;
       }
-    return chi * cm / (2.0 * dt) * (4.0 * un - upr) + ia * mask[o + r] - chi * I;
-  };
-  double acc[B];
-#pragma unroll
-  for (int r = 0; r < B; ++r) acc[r] = 0.0;
-  const double* Mb = Me + (size_t)slice * SL * KP;
-  if constexpr (B > 32) {
-    __shared__ double tsh[B * NTB];
-    double* ts = tsh + threadIdx.x;
-#pragma unroll
-    for (int r = 0; r < B; ++r) ts[r * NTB] = nodal(r);
-    block_mv<double, double, B, NTB>(Mb, lane, ts, acc);
-  } else {
-    double tv[B];
-#pragma unroll
-    for (int r = 0; r < B; ++r) tv[r] = nodal(r);
-    block_mv<double, double, B>(Mb, lane, tv, acc);
+    sh[threadIdx.x] = chi * cm / (2.0 * dt) * (4.0 * un - upr) + ia * mask[o] - chi * ionic_current(prm, us, w1);
   }
-#pragma unroll
-  for (int r = 0; r < B; ++r) b[o + r] = acc[r];
+  __syncthreads();
+  if (active) b[o] = elem_mv<B>(Me + (size_t)unit * B * B, r, sh + slot * B);
 }
 
 // Partial derivatives of the ionic model at one DoF (I_u, I_w, H_u, H_w).
@@ -488,49 +504,36 @@ __device__ __forceinline__ void ionic_jac(const IonicParams& p, double u, double
   }
 }
 
-// Reverse of one time step, pointwise part, for the thread's element
+// Reverse of one time step, pointwise part
 // (discrete adjoint of the step; lambda = K^{-1} ubar is the input):
 //   q = M_e lambda_e,  w~ = wbar - chi I_w(u_n, w_np1) q,
 //   ubar_n = q (c - chi I_u(u_n, w_np1)) + dt H_u(u_n, w_n) w~,
 //   wbar_n = w~ (1 + dt H_w(u_n, w_n)),   with w_np1 = w_n + dt H(u_n, w_n).
 template <int B>
-static __global__ void __launch_bounds__(UnitThreads<B>::value)
+static __global__ void __launch_bounds__(ElemRows<B>::NT)
     k_adj_pointwise(const double* __restrict__ Me, const double* __restrict__ lam, const double* __restrict__ u_n,
                     const double* __restrict__ w_n, double* __restrict__ ubar, double* __restrict__ wbar,
-                    IonicParams prm, double dt, double chi, double c, int64_t nslices) {
-  constexpr int NTB = UnitThreads<B>::value;
-  constexpr int KP = Pad<double, B>::KP;
-  const int lane = threadIdx.x & 31;
-  {
-  const int64_t slice = first_slice<NTB>();
-  if (slice >= nslices) return;
-  const int64_t unit = slice * SL + lane;
-  const size_t o = (size_t)unit * B;
-  double q[B];
-#pragma unroll
-  for (int r = 0; r < B; ++r) q[r] = 0.0;
-  if constexpr (B > 32) {
-    block_mv<double, double, B>(Me + (size_t)slice * SL * KP, lane, lam + o, q);
-  } else {
-    double lv[B];
-#pragma unroll
-    for (int r = 0; r < B; ++r) lv[r] = lam[o + r];
-    block_mv<double, double, B>(Me + (size_t)slice * SL * KP, lane, lv, q);
-  }
-#pragma unroll
-  for (int r = 0; r < B; ++r) {
-    const double un = u_n[o + r], wn = w_n[o + r];
-    double I, H[kMaxGates], Iu, Iw, Hu, Hw, Iu1, Iw1, Hu1, Hw1;
-    const double wg[kMaxGates] = {wn, 0.0, 0.0};
-    ionic_eval(prm, un, wg, I, H);                 // one-gate models only
-    const double w1 = wn + dt * H[0];
-    ionic_jac(prm, un, w1, Iu1, Iw1, Hu1, Hw1);
-    ionic_jac(prm, un, wn, Iu, Iw, Hu, Hw);
-    const double wt = wbar[o + r] - chi * Iw1 * q[r];
-    ubar[o + r] = q[r] * (c - chi * Iu1) + dt * Hu * wt;
-    wbar[o + r] = wt * (1.0 + dt * Hw);
-  }
-  }
+                    IonicParams prm, double dt, double chi, double c, int64_t n) {
+  constexpr int U = ElemRows<B>::U;
+  __shared__ double sh[U * B];
+  const int slot = threadIdx.x / B, r = threadIdx.x - slot * B;
+  const int64_t unit = (int64_t)blockIdx.x * U + slot;
+  const bool active = slot < U && unit < n;
+  const size_t o = (size_t)unit * B + r;
+  if (active) sh[threadIdx.x] = lam[o];
+  __syncthreads();
+  if (!active) return;
+  const double q = elem_mv<B>(Me + (size_t)unit * B * B, r, sh + slot * B);
+  const double un = u_n[o], wn = w_n[o];
+  double H[kMaxGates], Iu, Iw, Hu, Hw, Iu1, Iw1, Hu1, Hw1;
+  const double wg[kMaxGates] = {wn, 0.0, 0.0};
+  ionic_rates(prm, un, wg, H);                        // one-gate models only
+  const double w1 = wn + dt * H[0];
+  ionic_jac(prm, un, w1, Iu1, Iw1, Hu1, Hw1);
+  ionic_jac(prm, un, wn, Iu, Iw, Hu, Hw);
+  const double wt = wbar[o] - chi * Iw1 * q;
+  ubar[o] = q * (c - chi * Iu1) + dt * Hu * wt;
+  wbar[o] = wt * (1.0 + dt * Hw);
 }
 
 // Layout of the adjoint face parts on the device: per slice and local face,

@@ -1041,16 +1041,16 @@ class Engine : public EngineBase {
   }
 
   void launch_step_prologue(cudaStream_t s) {
-    IonicParams ip{sp_.model, sp_.k, sp_.a, sp_.eps, sp_.gamma, sp_.mu1, sp_.mu2, sp_.bo};
+    const IonicParams ip = make_ionic(sp_.model, sp_.k, sp_.a, sp_.eps, sp_.gamma, sp_.mu1, sp_.mu2, sp_.bo);
+    const int64_t n = lev_[0].n;
     if (sp_.scheme == 1) {
-      k_ionic_rhs_bdf2<B><<<bgrid(0, lev_[0].nsl), NTB, 0, s>>>(Me_, x_, up_, w_, wp_, mask_, b_, ip, sp_.dt, sp_.chi,
-                                                              sp_.cm, sp_.iapp_value, sp_.iapp_steps, step_,
-                                                              lev_[0].nsl, N0());
+      k_ionic_rhs_bdf2<B><<<cdiv(n, ElemRows<B>::U), ElemRows<B>::NT, 0, s>>>(
+          Me_, x_, up_, w_, wp_, mask_, b_, ip, sp_.dt, sp_.chi, sp_.cm, sp_.iapp_value, sp_.iapp_steps, step_, n, N0());
       return;
     }
     const double c = sp_.chi * sp_.cm / sp_.dt;
-    k_ionic_rhs<B><<<bgrid(0, lev_[0].nsl), NTB, 0, s>>>(Me_, x_, w_, mask_, b_, ip, sp_.dt, sp_.chi, c,
-                                                         sp_.iapp_value, sp_.iapp_steps, step_, lev_[0].nsl, N0());
+    k_ionic_rhs<B><<<cdiv(n, ElemRows<B>::U), ElemRows<B>::NT, 0, s>>>(
+        Me_, x_, w_, mask_, b_, ip, sp_.dt, sp_.chi, c, sp_.iapp_value, sp_.iapp_steps, step_, n, N0());
   }
 
   // Builds [prologue] -> WHILE(body) -> [epilogue]; prologue/epilogue are
@@ -1309,7 +1309,7 @@ class Engine : public EngineBase {
       std::vector<double> me((size_t)m.ne * B * B);
       for (int64_t r = 0; r < m.ne; ++r)
         std::memcpy(&me[(size_t)r * B * B], &m.Me[(size_t)h.lev[0].perm[r] * B * B], sizeof(double) * B * B);
-      if ((rc = upload_blocks<double>(me, m.ne, lev_[0].nsl, &Me_, err))) return rc;
+      if ((rc = upload_colmajor<double>(me.data(), m.ne, &Me_, err))) return rc;
       me_int_.swap(me);
     }
     // adjoint data: volume forms and per-slot face parts in the fine operator's slot order
@@ -1565,7 +1565,7 @@ class Engine : public EngineBase {
       if ((rc = dalloc(&wp_, kMaxGates * N, err))) return rc;
       std::vector<double> minv(me_int_.size());
       if (!spd_inverse_blocks(me_int_.data(), v0.n, B, minv.data())) { err = "element mass block not SPD"; return AGG_ENOTSPD; }
-      if ((rc = upload_blocks<double>(minv, v0.n, v0.nsl, &Minv_, err))) return rc;
+      if ((rc = upload_colmajor<double>(minv.data(), v0.n, &Minv_, err))) return rc;
     }
     hist_valid_ = false;
     if (mask_user)
@@ -1604,12 +1604,12 @@ class Engine : public EngineBase {
     AGG_CK(cudaMemsetAsync(sim_status_, 0, sizeof(int), s));
     if (sp_.scheme == 1 && !hist_valid_) {
       // second-order start of the BDF2 history from the current state
-      IonicParams ip{sp_.model, sp_.k, sp_.a, sp_.eps, sp_.gamma, sp_.mu1, sp_.mu2, sp_.bo};
+      const IonicParams ip = make_ionic(sp_.model, sp_.k, sp_.a, sp_.eps, sp_.gamma, sp_.mu1, sp_.mu2, sp_.bo);
       const double c = 1.5 * sp_.chi * sp_.cm / sp_.dt;
       const double ia = (clock < sp_.iapp_steps) ? sp_.iapp_value : 0.0;
       spmv0<0>(x_, nullptr, q_, nullptr, s);
-      k_bdf2_start<B><<<bgrid(0, v0.nsl), NTB, 0, s>>>(Minv_, q_, x_, w_, mask_, up_, wp_, ip, sp_.dt, sp_.chi, sp_.cm,
-                                                       c, ia, v0.nsl, N0());
+      k_bdf2_start<B><<<cdiv(v0.n, ElemRows<B>::U), ElemRows<B>::NT, 0, s>>>(Minv_, q_, x_, w_, mask_, up_, wp_, ip, sp_.dt,
+                                                                             sp_.chi, sp_.cm, c, ia, v0.n, N0());
       hist_valid_ = true;
     }
     k_set_opts<<<1, 1, 0, s>>>(st_, sp_.pcg.rtol, sp_.pcg.atol, sp_.pcg.max_it, sp_.pcg.flexible);
@@ -1803,9 +1803,10 @@ class Engine : public EngineBase {
     k_gather_units<double, double><<<g, 256, 0, s>>>(w_n, wa_, v0.perm, v0.n, B);
     k_gather_units<double, double><<<g, 256, 0, s>>>(u_np1, ub_, v0.perm, v0.n, B);
     k_gather_units<double, double><<<g, 256, 0, s>>>(wbar, wb_, v0.perm, v0.n, B);
-    IonicParams ip{sp_.model, sp_.k, sp_.a, sp_.eps, sp_.gamma, sp_.mu1, sp_.mu2, sp_.bo};
+    const IonicParams ip = make_ionic(sp_.model, sp_.k, sp_.a, sp_.eps, sp_.gamma, sp_.mu1, sp_.mu2, sp_.bo);
     const double c = sp_.chi * sp_.cm / sp_.dt;
-    k_adj_pointwise<B><<<bgrid(k_adj_pointwise<B>, v0.nsl), NTB, 0, s>>>(Me_, x_, ua_, wa_, b_, wb_, ip, sp_.dt, sp_.chi, c, v0.nsl);
+    k_adj_pointwise<B><<<cdiv(v0.n, ElemRows<B>::U), ElemRows<B>::NT, 0, s>>>(Me_, x_, ua_, wa_, b_, wb_, ip, sp_.dt,
+                                                                             sp_.chi, c, v0.n);
     k_grad_logD<B><<<bgrid(0, v0.nsl), NTB, 0, s>>>(A0f_.V, Ke_, Y_, x_, ub_, v0.perm, grad, v0.n);
     k_scatter_units<double, double><<<g, 256, 0, s>>>(b_, ubar, v0.perm, v0.n, B);
     k_scatter_units<double, double><<<g, 256, 0, s>>>(wb_, wbar, v0.perm, v0.n, B);
