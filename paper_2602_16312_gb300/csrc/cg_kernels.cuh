@@ -536,79 +536,92 @@ static __global__ void __launch_bounds__(ElemRows<B>::NT)
   wbar[o] = wt * (1.0 + dt * Hw);
 }
 
-// Layout of the adjoint face parts on the device: per slice and local face,
-// five row-major parts (the structure of Mesh::Yc), each padded to whole
-// double2 chunks, in the sliced chunk order [chunk][lane][2].
-template <int B> struct AdjFaceLayout {
-  static constexpr int NF = FaceIdx<FaceShape<B>::D, FaceShape<B>::N>::NF;
-  static constexpr int P1 = (NF * B + 1) / 2 * 2, P2 = ((B - NF) * NF + 1) / 2 * 2, P3 = (B * NF + 1) / 2 * 2;
-  static constexpr int P4 = P1, P5 = (NF * NF + 1) / 2 * 2;
-  static constexpr int YS = P1 + P2 + P3 + P4 + P5;      // doubles per lane and face
-};
-
-// sum_{r, c} y(r) M[r][c] x(c) over one R x C part starting at chunk ch0
-template <int R, int C, typename YF, typename XF>
-__device__ __forceinline__ double part_bilinear(const double2* yb, int ch0, YF y, XF x) {
-  double s = 0.0;
-#pragma unroll 1
-  for (int ch = 0; ch < (R * C + 1) / 2; ++ch) {
-    const double2 v = __ldg(yb + (size_t)(ch0 + ch) * SL);
-    const int k = 2 * ch;
-    s += v.x * y(k / C) * x(k % C);
-    if (k + 1 < R * C) s += v.y * y((k + 1) / C) * x((k + 1) % C);
-  }
-  return s;
-}
-
 // Per-element log-conductivity gradient, accumulated in the caller's order:
 //   grad[e] -= lam_e^T Ke u_e + sum_faces [lam_e; lam_n]^T Y_e,F [u_e; u_n]
 // with Ke the volume form and Y_e,F the face terms built with D_e, of which
-// only the trace-structured parts are stored (AdjFaceLayout): ee on e's face
-// rows and face columns, en on n's face columns, ne on n's face rows, nn.
+// only the trace-structured parts are stored (the row-major parts of Mesh::Yc,
+// one after the other, per element and local face): ee on e's face rows, ee on
+// face columns of the other rows, en on n's face columns, ne on n's face rows, nn.
+// One thread per (element, DoF), U elements per block: the threads read B
+// consecutive entries per step, hold a column each (the parts with NF columns:
+// N rows per step) and sum over the rows, one FMA per entry; HBM bounds it
+// (one thread per element walked 28,672 entries in sequence for Q3 hexahedra).
 template <int B>
-static __global__ void __launch_bounds__(UnitThreads<B>::value)
+static __global__ void __launch_bounds__(ElemRows<B>::NT)
     k_grad_logD(FaceView<double, B> F, const double* __restrict__ Ke, const double* __restrict__ Yc,
                 const double* __restrict__ lam, const double* __restrict__ u, const int64_t* __restrict__ perm,
                 double* __restrict__ grad, int64_t n) {
-  constexpr int NTB = UnitThreads<B>::value;
-  constexpr int KP = Pad<double, B>::KP;
   using FI = FaceIdx<FaceShape<B>::D, FaceShape<B>::N>;
-  using YL = AdjFaceLayout<B>;
-  constexpr int NF = YL::NF, NFACE = 2 * FaceShape<B>::D;
-  const int lane = threadIdx.x & 31;
-  const int64_t slice = first_slice<NTB>();
-  if (slice >= F.nslices) return;
-  const int64_t unit = slice * SL + lane;
-  const size_t o = (size_t)unit * B;
-  double t[B];
-#pragma unroll
-  for (int r = 0; r < B; ++r) t[r] = 0.0;
-  block_mv<double, double, B>(Ke + (size_t)slice * SL * KP, lane, u + o, t);
-  double g = 0.0;
-#pragma unroll
-  for (int r = 0; r < B; ++r) g += lam[o + r] * t[r];
-  const double* lu = lam + o;
-  const double* uu = u + o;
-#pragma unroll 1
-  for (int f = 0; f < NFACE; ++f) {
-    const size_t fi = ((size_t)slice * NFACE + f) * SL + lane;
-    const int nb = F.nbr[fi];
-    if (nb < 0) continue;
-    const int fn = F.code[fi];
-    const double* ln = lam + (size_t)nb * B;
-    const double* un = u + (size_t)nb * B;
-    const double2* yb = reinterpret_cast<const double2*>(Yc) + ((size_t)(slice * NFACE + f) * (YL::YS / 2)) * SL + lane;
-    g += part_bilinear<NF, B>(yb, 0, [&](int r) { return lu[FI::face(f, r)]; }, [&](int c) { return uu[c]; });
-    g += part_bilinear<B - NF, NF>(yb, YL::P1 / 2, [&](int r) { return lu[FI::off(f, r)]; },
-                                   [&](int c) { return uu[FI::face(f, c)]; });
-    g += part_bilinear<B, NF>(yb, (YL::P1 + YL::P2) / 2, [&](int r) { return lu[r]; },
-                              [&](int c) { return un[FI::face(fn, c)]; });
-    g += part_bilinear<NF, B>(yb, (YL::P1 + YL::P2 + YL::P3) / 2, [&](int r) { return ln[FI::face(fn, r)]; },
-                              [&](int c) { return uu[c]; });
-    g += part_bilinear<NF, NF>(yb, (YL::P1 + YL::P2 + YL::P3 + YL::P4) / 2,
-                               [&](int r) { return ln[FI::face(fn, r)]; }, [&](int c) { return un[FI::face(fn, c)]; });
+  constexpr int N = FaceShape<B>::N, NF = FI::NF, NFACE = 2 * FaceShape<B>::D, U = ElemRows<B>::U;
+  constexpr int S2 = (B - NF) * NF / B, S5 = NF * NF / B;     // steps of the parts with NF columns
+  __shared__ double sl[U * B], su[U * B], sln[U * NFACE * NF], sun[U * NFACE * NF];
+  const int slot = threadIdx.x / B, r = threadIdx.x - slot * B;
+  const int64_t unit = (int64_t)blockIdx.x * U + slot;
+  const bool active = slot < U && unit < n;
+  const int64_t f0 = unit / SL * NFACE * SL + unit % SL;      // (slice, face 0, lane)
+  double* lu = sl + slot * B;
+  double* uu = su + slot * B;
+  double* ln = sln + slot * NFACE * NF;
+  double* un = sun + slot * NFACE * NF;
+  if (active) {
+    lu[r] = lam[(size_t)unit * B + r];
+    uu[r] = u[(size_t)unit * B + r];
+    for (int k = r; k < NFACE * NF; k += B) {
+      const int f = k / NF;
+      const int nb = F.nbr[f0 + f * SL];
+      if (nb < 0) continue;
+      const size_t o = (size_t)nb * B + FI::face(F.code[f0 + f * SL], k % NF);
+      ln[k] = lam[o];
+      un[k] = u[o];
+    }
   }
-  if (unit < n) grad[perm[unit]] -= g;
+  __syncthreads();
+  double g = 0.0;
+  if (active) {
+    const int q = r / NF, cf = r % NF;
+    // sum over steps of M[step B + r] y(step)
+    auto col = [&](const double* M, auto steps, auto y) {
+      constexpr int kSteps = decltype(steps)::value;
+      double s = 0.0;
+#pragma unroll 8
+      for (int i = 0; i < kSteps; ++i) s += __ldcs(M + i * B + r) * y(i);
+      return s;
+    };
+    using std::integral_constant;
+    g = col(Ke + (size_t)unit * B * B, integral_constant<int, B>{}, [&](int i) { return lu[i]; }) * uu[r];
+#pragma unroll 1
+    for (int f = 0; f < NFACE; ++f) {
+      if (F.nbr[f0 + f * SL] < 0) continue;
+      const double* M = Yc + ((size_t)unit * NFACE + f) * 4 * NF * B;
+      const double* lnf = ln + f * NF;
+      const double* unf = un + f * NF;
+      g += col(M, integral_constant<int, NF>{}, [&](int i) { return lu[FI::face(f, i)]; }) * uu[r];
+      M += NF * B;
+      g += col(M, integral_constant<int, S2>{}, [&](int i) { return lu[FI::off(f, i * N + q)]; }) * uu[FI::face(f, cf)];
+      M += (B - NF) * NF;
+      g += col(M, integral_constant<int, NF>{}, [&](int i) { return lu[i * N + q]; }) * unf[cf];
+      M += B * NF;
+      g += col(M, integral_constant<int, NF>{}, [&](int i) { return lnf[i]; }) * uu[r];
+      M += NF * B;
+      g += col(M, integral_constant<int, S5>{}, [&](int i) { return lnf[i * N + q]; }) * unf[cf];
+    }
+  }
+  __syncthreads();
+  if (active) lu[r] = g;                              // summed in a fixed order
+  __syncthreads();
+  if (active && r < NF) {
+    double s = 0.0;
+#pragma unroll
+    for (int a = 0; a < N; ++a) s += lu[a * NF + r];
+    uu[r] = s;
+  }
+  __syncthreads();
+  if (active && r == 0) {
+    double s = 0.0;
+#pragma unroll
+    for (int j = 0; j < NF; ++j) s += uu[j];
+    grad[perm[unit]] -= s;
+  }
 }
 
 // end of a time step: record the iteration count, advance the clock

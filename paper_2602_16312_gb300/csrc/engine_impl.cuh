@@ -1318,40 +1318,20 @@ class Engine : public EngineBase {
       std::vector<double> ke((size_t)m.ne * B * B);
       for (int64_t r = 0; r < m.ne; ++r)
         std::memcpy(&ke[(size_t)r * B * B], &m.Ke[(size_t)l0.perm[r] * B * B], sizeof(double) * B * B);
-      if ((rc = upload_blocks<double>(ke, m.ne, lev_[0].nsl, &Ke_, err))) return rc;
-      // face parts per (slice, local face), the five parts padded to whole
-      // double2 chunks, in the chunk layout (see k_grad_logD); copied in
-      // pieces of 1024 slices so the host needs no full-size staging copy
-      using YL = AdjFaceLayout<B>;
-      const int nf = 2 * FaceShape<B>::D, NF = YL::NF;
-      const int64_t nsl = lev_[0].nsl;
-      const size_t per_slice = (size_t)nf * YL::YS * SL;
-      if ((rc = dalloc(&Y_, (size_t)nsl * per_slice, err))) return rc;
-      const int sizes[5] = {NF * B, (B - NF) * NF, B * NF, NF * B, NF * NF};
-      const int offs[5] = {0, YL::P1, YL::P1 + YL::P2, YL::P1 + YL::P2 + YL::P3, YL::P1 + YL::P2 + YL::P3 + YL::P4};
-      const int64_t piece = 1024;
+      if ((rc = upload(&Ke_, ke.data(), ke.size(), err))) return rc;
+      // face parts per element in internal order, copied in pieces so that the
+      // host needs no full-size staging copy
+      const size_t per = (size_t)2 * FaceShape<B>::D * 4 * FaceIdx<FaceShape<B>::D, FaceShape<B>::N>::NF * B;
+      if ((rc = dalloc(&Y_, (size_t)m.ne * per, err))) return rc;
+      const int64_t piece = 16384;
       std::vector<double> hy;
-      for (int64_t s0 = 0; s0 < nsl; s0 += piece) {
-        const int64_t s1 = std::min(nsl, s0 + piece);
-        hy.assign((size_t)(s1 - s0) * per_slice, 0.0);
-        for (int64_t r = s0 * SL; r < std::min<int64_t>(m.ne, s1 * SL); ++r) {
-          const int64_t e = l0.perm[r], sl = r / SL - s0;
-          const int lane = (int)(r % SL);
-          for (int f = 0; f < nf; ++f) {
-            const double* src = &m.Yc[((size_t)e * nf + f) * 4 * NF * B];
-            double* dst = &hy[((size_t)sl * nf + f) * YL::YS * SL];
-            int so = 0;
-            for (int pt = 0; pt < 5; ++pt) {
-              for (int k = 0; k < sizes[pt]; ++k) {
-                const int kk = offs[pt] + k;
-                dst[((size_t)(kk / 2) * SL + lane) * 2 + (kk % 2)] = src[so + k];
-              }
-              so += sizes[pt];
-            }
-          }
-        }
-        AGG_CK(cudaMemcpy(Y_ + (size_t)s0 * per_slice, hy.data(), sizeof(double) * hy.size(),
-                          cudaMemcpyHostToDevice));
+      for (int64_t r0 = 0; r0 < m.ne; r0 += piece) {
+        const int64_t r1 = std::min<int64_t>(m.ne, r0 + piece);
+        hy.resize((size_t)(r1 - r0) * per);
+#pragma omp parallel for schedule(static)
+        for (int64_t r = r0; r < r1; ++r)
+          std::memcpy(&hy[(size_t)(r - r0) * per], &m.Yc[(size_t)l0.perm[r] * per], sizeof(double) * per);
+        AGG_CK(cudaMemcpy(Y_ + (size_t)r0 * per, hy.data(), sizeof(double) * hy.size(), cudaMemcpyHostToDevice));
       }
     }
     // matrix-free fine operator for the float32 V-cycle
@@ -1807,7 +1787,7 @@ class Engine : public EngineBase {
     const double c = sp_.chi * sp_.cm / sp_.dt;
     k_adj_pointwise<B><<<cdiv(v0.n, ElemRows<B>::U), ElemRows<B>::NT, 0, s>>>(Me_, x_, ua_, wa_, b_, wb_, ip, sp_.dt,
                                                                              sp_.chi, c, v0.n);
-    k_grad_logD<B><<<bgrid(0, v0.nsl), NTB, 0, s>>>(A0f_.V, Ke_, Y_, x_, ub_, v0.perm, grad, v0.n);
+    k_grad_logD<B><<<cdiv(v0.n, ElemRows<B>::U), ElemRows<B>::NT, 0, s>>>(A0f_.V, Ke_, Y_, x_, ub_, v0.perm, grad, v0.n);
     k_scatter_units<double, double><<<g, 256, 0, s>>>(b_, ubar, v0.perm, v0.n, B);
     k_scatter_units<double, double><<<g, 256, 0, s>>>(wb_, wbar, v0.perm, v0.n, B);
     AGG_CK(cudaMemcpyAsync(st_host_, st_, sizeof(CGState), cudaMemcpyDeviceToHost, s));
