@@ -21,6 +21,7 @@ static __global__ void k_loop_ctl(CGState* st) {
     st->done = 1;
     if (st->use_cond) cudaGraphSetConditional((cudaGraphConditionalHandle)st->cond, 0u);
   }
+  st->rho = st->rz;
   st->guard += 1;
 }
 
@@ -37,7 +38,7 @@ static __global__ void k_cg_reset(CGState* st, GridBar* bar) {
   st->done = 0;
   st->status = 0;
   st->rho = st->alpha = st->beta = st->pq = st->rr = st->r0 = 0.0;
-  st->rz_old = 0.0;
+  st->rz = 0.0;
 }
 
 // Start of a solve: reset (with the coarse-level kernel's grid barrier, if
@@ -51,7 +52,7 @@ static __global__ void k_cg_begin(CGState* st, unsigned long long cond, int use_
   st->done = 0;
   st->status = 0;
   st->rho = st->alpha = st->beta = st->pq = st->rr = st->r0 = 0.0;
-  st->rz_old = 0.0;
+  st->rz = 0.0;
   st->guard = 0;
   st->cond = cond;
   st->use_cond = use_cond;
@@ -90,21 +91,27 @@ static __global__ void __launch_bounds__(RED_NT) k_r0(const double* __restrict__
 
 // x += alpha p; r -= alpha q; ||r||; convergence test. Fused with the
 // V-cycle's input cast (r32 = (float) r, when r32 is given) and, for the
-// flexible variant, the (r_new, z_old) product of the Polak-Ribiere beta
-// (z_old: the previous preconditioned residual). Both sums use the fixed
-// grid and block order of the other reductions (second sum in
-// partials[gridDim.x ..]).
+// flexible variant, the (r_new, z_old) product of the Polak-Ribiere beta (z_old:
+// the previous V-cycle's result, still in its buffer). alpha = rho / (p, q) from
+// the float64 product's npq partials. Both sums use the fixed grid and block
+// order of the other reductions; the partials of (r, z_old) go to the p update.
+// HBM bounds it, with the float64 pipe (4 FMAs per entry) close behind.
+template <typename TZ>
 static __global__ void __launch_bounds__(RED_NT) k_cg_update(double* __restrict__ x, double* __restrict__ r,
                                                       const double* __restrict__ p, const double* __restrict__ q,
-                                                      float* __restrict__ r32, const double* __restrict__ zold,
-                                                      int64_t n, double* partials, CGState* st) {
+                                                      float* __restrict__ r32, const TZ* __restrict__ zold, int64_t n,
+                                                      const double* pq_partials, int npq, double* partials,
+                                                      double* rz_partials, CGState* st) {
   if (st->done) return;
-  const double alpha = st->alpha;
+  const double pq = all_sum_partials<RED_NT>(pq_partials, npq);
+  const double alpha = st->rho / pq;
   const bool flex = st->flexible != 0;
+  using Z2 = typename std::conditional<std::is_same<TZ, float>::value, float2, double2>::type;
   double s = 0.0, sz = 0.0;
   // pairs of entries per 16-byte access (n is even: whole 32-unit slices),
   // a scalar tail otherwise
   const int64_t n2 = n >> 1;
+#pragma unroll 2
   for (int64_t i = (int64_t)blockIdx.x * RED_NT + threadIdx.x; i < n2; i += (int64_t)gridDim.x * RED_NT) {
     double2 xv = reinterpret_cast<double2*>(x)[i];
     double2 rv = reinterpret_cast<double2*>(r)[i];
@@ -119,9 +126,9 @@ static __global__ void __launch_bounds__(RED_NT) k_cg_update(double* __restrict_
     s += rv.x * rv.x;
     s += rv.y * rv.y;
     if (flex) {
-      const double2 zv = reinterpret_cast<const double2*>(zold)[i];
-      sz += rv.x * zv.x;
-      sz += rv.y * zv.y;
+      const Z2 zv = reinterpret_cast<const Z2*>(zold)[i];
+      sz += rv.x * (double)zv.x;
+      sz += rv.y * (double)zv.y;
     }
     if (r32) reinterpret_cast<float2*>(r32)[i] = make_float2((float)rv.x, (float)rv.y);
   }
@@ -131,17 +138,19 @@ static __global__ void __launch_bounds__(RED_NT) k_cg_update(double* __restrict_
     const double ri = r[i] - alpha * q[i];
     r[i] = ri;
     s += ri * ri;
-    if (flex) sz += ri * zold[i];
+    if (flex) sz += ri * (double)zold[i];
     if (r32) r32[i] = (float)ri;
   }
-  const double bz = block_sum<RED_NT>(sz);
-  if (threadIdx.x == 0) partials[gridDim.x + blockIdx.x] = bz;
+  if (flex) {
+    const double bz = block_sum<RED_NT>(sz);
+    if (threadIdx.x == 0) rz_partials[blockIdx.x] = bz;
+  }
   if (partial_and_last<RED_NT>(s, partials, &st->ticket[TK_R])) {
     double rr = sum_partials<RED_NT>(partials, gridDim.x);
-    double rz = sum_partials<RED_NT>(partials + gridDim.x, gridDim.x);
     if (threadIdx.x == 0) {
       st->ticket[TK_R] = 0;
-      if (flex) st->rz_old = rz;
+      st->pq = pq;
+      st->alpha = alpha;
       st->rr = rr;
       st->iter += 1;
       double rn = sqrt(rr);
@@ -158,61 +167,47 @@ static __global__ void __launch_bounds__(RED_NT) k_cg_update(double* __restrict_
   }
 }
 
-// z64 <- zin (V-cycle output, any precision); rz = (r, z_new).
-// INIT: rho = rz.  Otherwise beta = rz / rho (Fletcher-Reeves form) or, for
-// the flexible variant, beta = (rz - (r, z_old)) / rho (Polak-Ribiere, with
-// (r, z_old) from k_cg_update), then rho = rz.
-template <typename TZ, bool INIT>
-static __global__ void __launch_bounds__(RED_NT) k_zdot(const TZ* __restrict__ zin, double* __restrict__ z64,
-                                                 const double* __restrict__ r, int64_t n, double* partials,
-                                                 CGState* st) {
+// per-block partials of (r, z), z the V-cycle's result in its own precision
+template <typename TZ>
+static __global__ void __launch_bounds__(RED_NT) k_zdot(const TZ* __restrict__ z, const double* __restrict__ r, int64_t n,
+                                                 double* partials, const CGState* st) {
   if (st->done) return;
   double s = 0.0;
   using Z2 = typename std::conditional<std::is_same<TZ, float>::value, float2, double2>::type;
   const int64_t n2 = n >> 1;
+#pragma unroll 2
   for (int64_t i = (int64_t)blockIdx.x * RED_NT + threadIdx.x; i < n2; i += (int64_t)gridDim.x * RED_NT) {
-    const Z2 zv = reinterpret_cast<const Z2*>(zin)[i];
+    const Z2 zv = reinterpret_cast<const Z2*>(z)[i];
     const double2 rv = reinterpret_cast<const double2*>(r)[i];
-    const double2 zn = make_double2((double)zv.x, (double)zv.y);
-    reinterpret_cast<double2*>(z64)[i] = zn;
-    s += rv.x * zn.x;
-    s += rv.y * zn.y;
+    s += rv.x * (double)zv.x;
+    s += rv.y * (double)zv.y;
   }
-  if ((n & 1) && blockIdx.x == 0 && threadIdx.x == 0) {
-    const double zn = (double)zin[n - 1];
-    z64[n - 1] = zn;
-    s += r[n - 1] * zn;
-  }
-  if (partial_and_last<RED_NT>(s, partials, &st->ticket[TK_Z])) {
-    const double rz = sum_partials<RED_NT>(partials, gridDim.x);
-    if (threadIdx.x == 0) {
-      st->ticket[TK_Z] = 0;
-      if (INIT) st->beta = 0.0;
-      else st->beta = (st->flexible ? rz - st->rz_old : rz) / st->rho;
-      st->rho = rz;
-    }
-  }
+  if ((n & 1) && blockIdx.x == 0 && threadIdx.x == 0) s += r[n - 1] * (double)z[n - 1];
+  const double b = block_sum<RED_NT>(s);
+  if (threadIdx.x == 0) partials[blockIdx.x] = b;
 }
 
-// p = z + beta p (INIT: p = z)
-template <bool INIT>
-static __global__ void __launch_bounds__(RED_NT) k_pupd(const double* __restrict__ z, double* __restrict__ p, int64_t n,
-                                                 const CGState* st) {
+// p = z + beta p (INIT: p = z), beta from the partials (cg_beta); rho follows in k_loop_ctl
+template <typename TZ, bool INIT>
+static __global__ void __launch_bounds__(RED_NT) k_pupd(const TZ* __restrict__ z, double* __restrict__ p, int64_t n,
+                                                 const double* partials, int np, CGState* st) {
   if (st->done) return;
-  const double beta = st->beta;
+  const double beta = cg_beta<RED_NT, INIT>(partials, np, st);
+  using Z2 = typename std::conditional<std::is_same<TZ, float>::value, float2, double2>::type;
   const int64_t n2 = n >> 1;
+#pragma unroll 2
   for (int64_t i = (int64_t)blockIdx.x * RED_NT + threadIdx.x; i < n2; i += (int64_t)gridDim.x * RED_NT) {
-    const double2 zv = reinterpret_cast<const double2*>(z)[i];
-    if (INIT) {
-      reinterpret_cast<double2*>(p)[i] = zv;
-    } else {
-      double2 pv = reinterpret_cast<double2*>(p)[i];
-      pv.x = zv.x + beta * pv.x;
-      pv.y = zv.y + beta * pv.y;
-      reinterpret_cast<double2*>(p)[i] = pv;
+    const Z2 zv = reinterpret_cast<const Z2*>(z)[i];
+    double2 pv = make_double2((double)zv.x, (double)zv.y);
+    if (!INIT) {
+      const double2 po = reinterpret_cast<const double2*>(p)[i];
+      pv.x += beta * po.x;
+      pv.y += beta * po.y;
     }
+    reinterpret_cast<double2*>(p)[i] = pv;
   }
-  if ((n & 1) && blockIdx.x == 0 && threadIdx.x == 0) p[n - 1] = INIT ? z[n - 1] : z[n - 1] + beta * p[n - 1];
+  if ((n & 1) && blockIdx.x == 0 && threadIdx.x == 0)
+    p[n - 1] = INIT ? (double)z[n - 1] : (double)z[n - 1] + beta * p[n - 1];
 }
 
 template <typename TO, typename TI>

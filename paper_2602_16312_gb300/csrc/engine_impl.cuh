@@ -199,7 +199,7 @@ class Engine : public EngineBase {
   double* Me_ = nullptr;
   double *Linv_ = nullptr, *U_ = nullptr, *yc_ = nullptr;
   int64_t nc_ = 0;
-  double *b_ = nullptr, *x_ = nullptr, *r_ = nullptr, *p_ = nullptr, *q_ = nullptr, *z_ = nullptr;
+  double *b_ = nullptr, *x_ = nullptr, *r_ = nullptr, *p_ = nullptr, *q_ = nullptr;
   double* partials_ = nullptr;
   float* r32_ = nullptr;
   CGState* st_ = nullptr;
@@ -646,22 +646,30 @@ class Engine : public EngineBase {
     if ((rc = prepare_sym<T, TD, SYM_CHEB, 2>(6, err))) return rc;
     return prepare_sym<T, TD, SYM_RESTRICT, 0>(7, err);
   }
+  template <int OP, int KIND, typename TT, typename TDD>
+  int64_t sym_grid(int slot, int64_t n) const {
+    if constexpr (kStream) {
+      using M = SymRing<TT, TDD, BS, OP, KIND>;
+      return std::min<int64_t>(cdiv(n, M::EPW * M::NWARP), sym_blocks_[slot]);
+    } else {
+      return std::min<int64_t>(cdiv(n, SymSmem<TT, TDD, B, OP, KIND>::U), sym_blocks_[slot]);
+    }
+  }
   // One k_sym launch: a block per U elements, at most the resident ones (each
   // then loops over the element groups, a group per step, so that the groups
   // in flight stay neighbours and share face blocks through the L2).
   template <int OP, int KIND, typename TT, typename TDD, typename SD>
   void launch_sym(int slot, const SymView<TT, B>& A, SymBlk<SD> ext, SymVec<TT> xv, const TT* rhs, const TT* x, TT* out,
                   TT* d, FxVec fo, TT c1, TT c2, CGState* st, cudaStream_t s) {
+    const int64_t g = sym_grid<OP, KIND, TT, TDD>(slot, A.n);
     if constexpr (kStream) {
       using M = SymRing<TT, TDD, BS, OP, KIND>;
-      const int64_t g = std::min<int64_t>(cdiv(A.n, M::EPW * M::NWARP), sym_blocks_[slot]);
-      k_symw<TT, TDD, BS, OP, KIND><<<g, M::NTH, M::bytes, s>>>(A, ext, xv, rhs, x, out, d, fo.X, fo.E, c1, c2, partials_,
-                                                              st);
+      k_symw<TT, TDD, BS, OP, KIND><<<g, M::NTH, M::bytes, s>>>(A, ext, xv, rhs, x, out, d, fo.X, fo.E, c1, c2,
+                                                              partials_ + kPQ, st);
     } else {
       using M = SymSmem<TT, TDD, B, OP, KIND>;
-      const int64_t g = std::min<int64_t>(cdiv(A.n, M::U), sym_blocks_[slot]);
-      k_sym<TT, TDD, B, OP, KIND><<<g, M::NTH, M::bytes, s>>>(A, ext, xv, rhs, x, out, d, fo.X, fo.E, c1, c2, partials_,
-                                                            st);
+      k_sym<TT, TDD, B, OP, KIND><<<g, M::NTH, M::bytes, s>>>(A, ext, xv, rhs, x, out, d, fo.X, fo.E, c1, c2,
+                                                            partials_ + kPQ, st);
     }
   }
   // Float64 level-0 product (MODE as in k_spmv)
@@ -673,7 +681,7 @@ class Engine : public EngineBase {
                                                  nullptr, FxVec{}, 0.0, 0.0, st, s);
     }
     else
-      k_spmv<double, B, MODE, A0Op><<<bgrid(0, lev_[0].nsl), NTB, 0, s>>>(A0f_, x, rhs, y, partials_, st);
+      k_spmv<double, B, MODE, A0Op><<<bgrid(0, lev_[0].nsl), NTB, 0, s>>>(A0f_, x, rhs, y, partials_ + kPQ, st);
   }
   // Level-0 Chebyshev step, residual + restriction and prolongation on the
   // symmetric blocks in the V-cycle precision
@@ -999,43 +1007,56 @@ class Engine : public EngineBase {
   bool use_mf0() const { return kMf && mf_; }
   int64_t g0() const { return cdiv(lev_[0].nsl * SL, NTB); }
 
+  // Grid of the vector kernels over n entries: up to 2 blocks per SM, at least
+  // two pairs of entries per thread (small problems: one block, whose sums need
+  // no second one).
+  static int red_grid(int64_t n) { return (int)std::min<int64_t>(RED_BLOCKS, std::max<int64_t>(1, cdiv(n, 4 * RED_NT))); }
+  // partials_: (r, r), (r, z), (r, z_old), and (p, q) from kPQ on
+  static constexpr int kRR = 0, kRZ = kPartials, kPQ = 3 * kPartials;
+  // blocks of the float64 product that writes (p, q)
+  int pq_blocks() const {
+    if (!osym_) return (int)bgrid(0, lev_[0].nsl);
+    return (int)sym_grid<SYM_SPMV, 2, double, double>(2, lev_[0].n);
+  }
+  // the buffer that holds the V-cycle's result: 2 degree - 1 swaps of the iterates
+  T* vcycle_result() const { return nlev_ == 1 ? lev_[0].xa : (((2 * degree_ - 1) & 1) ? lev_[0].xb : lev_[0].xa); }
+
   // z = V(r), beta, p. In the iteration body the float32 cast of r and the
   // flexible-beta product (r, z_old) come fused in k_cg_update.
   void launch_precond(cudaStream_t s, bool init) {
     const int64_t N = N0();
     if (init && !std::is_same<T, double>::value)
-      k_cast<float, double><<<RED_BLOCKS, RED_NT, 0, s>>>(r_, r32_, N, st_);
-    T* out = vc(0, s);
-    if (init) {
-      k_zdot<T, true><<<RED_BLOCKS, RED_NT, 0, s>>>(out, z_, r_, N, partials_, st_);
-      launch_pupd<true>(s);
-    } else {
-      k_zdot<T, false><<<RED_BLOCKS, RED_NT, 0, s>>>(out, z_, r_, N, partials_, st_);
-      launch_pupd<false>(s);
-    }
+      k_cast<float, double><<<2 * RED_BLOCKS, 256, 0, s>>>(r_, r32_, N, st_);
+    const T* z = vc(0, s);
+    k_zdot<T><<<red_grid(N), RED_NT, 0, s>>>(z, r_, N, partials_ + kRZ, st_);
+    if (init) launch_pupd<true>(z, s);
+    else launch_pupd<false>(z, s);
   }
   // p = z + beta p, with p's fixed-point copy where the operator takes it
   template <bool INIT>
-  void launch_pupd(cudaStream_t s) {
-    if (osym_)
-      k_pupd_fx<B, INIT><<<cdiv(lev_[0].n, SymRows<B>::U), SymRows<B>::NT, 0, s>>>(z_, p_, lev_[0].n, A0s_.sc, fxp_.X,
-                                                                                  fxp_.E, st_);
-    else
-      k_pupd<INIT><<<RED_BLOCKS, RED_NT, 0, s>>>(z_, p_, N0(), st_);
+  void launch_pupd(const T* z, cudaStream_t s) {
+    const int np = red_grid(N0());
+    if (osym_) {
+      const int64_t g = std::min<int64_t>(cdiv(lev_[0].n, SymRows<B>::U), 12 * num_sms_);
+      k_pupd_fx<T, B, INIT><<<g, SymRows<B>::NT, 0, s>>>(z, p_, lev_[0].n, partials_ + kRZ, np, A0s_.sc, fxp_.X, fxp_.E, st_);
+    } else {
+      k_pupd<T, INIT><<<np, RED_NT, 0, s>>>(z, p_, N0(), partials_ + kRZ, np, st_);
+    }
   }
 
   void launch_init(cudaStream_t s, unsigned long long cond, int use_cond) {
     k_cg_begin<<<1, 1, 0, s>>>(st_, cond, use_cond, persist_ ? bar_ : nullptr);
     spmv0<1>(x_, b_, r_, nullptr, s);
-    k_r0<<<RED_BLOCKS, RED_NT, 0, s>>>(r_, N0(), partials_, st_);
+    k_r0<<<red_grid(N0()), RED_NT, 0, s>>>(r_, N0(), partials_ + kRR, st_);
     launch_precond(s, true);
     k_loop_ctl<<<1, 1, 0, s>>>(st_);
   }
 
   void launch_body(cudaStream_t s) {
     spmv0<2>(p_, nullptr, q_, st_, s);
-    k_cg_update<<<RED_BLOCKS, RED_NT, 0, s>>>(x_, r_, p_, q_, std::is_same<T, double>::value ? nullptr : r32_, z_,
-                                              N0(), partials_, st_);
+    k_cg_update<T><<<red_grid(N0()), RED_NT, 0, s>>>(x_, r_, p_, q_, std::is_same<T, double>::value ? nullptr : r32_,
+                                                     vcycle_result(), N0(), partials_ + kPQ, pq_blocks(), partials_ + kRR,
+                                                     partials_ + kRZ + kPartials, st_);
     launch_precond(s, false);
     k_loop_ctl<<<1, 1, 0, s>>>(st_);
   }
@@ -1384,13 +1405,11 @@ class Engine : public EngineBase {
       if ((rc = dalloc(&yc_, nc_, err))) return rc;
     }
     const int64_t N = N0();
-    for (double** pp : {&b_, &x_, &r_, &p_, &q_, &z_})
+    for (double** pp : {&b_, &x_, &r_, &p_, &q_})
       if ((rc = dalloc(pp, N, err))) return rc;
     if (!std::is_same<T, double>::value)
       if ((rc = dalloc(&r32_, N, err))) return rc;
-    int64_t nparts = std::max<int64_t>(2 * RED_BLOCKS, 2 * g0() + 64);
-    for (int nb : sym_blocks_) nparts = std::max<int64_t>(nparts, nb);
-    if ((rc = dalloc(&partials_, nparts, err))) return rc;
+    if ((rc = dalloc(&partials_, kPQ + std::max<int64_t>(pq_blocks(), 1), err))) return rc;
     lev_[0].rhs = std::is_same<T, double>::value ? reinterpret_cast<T*>(r_) : reinterpret_cast<T*>(r32_);
     AGG_CK(cudaDeviceSynchronize());
     // graphs: conditional WHILE solve, with the batch fallback prepared as
@@ -1492,7 +1511,7 @@ class Engine : public EngineBase {
     k_cg_reset<<<1, 1, 0, s>>>(st_, persist_ ? bar_ : nullptr);
     k_gather_units<double, double><<<g, 256, 0, s>>>(r_user, r_, v.perm, v.n, B);
     if (!std::is_same<T, double>::value)
-      k_cast<float, double><<<RED_BLOCKS, RED_NT, 0, s>>>(r_, r32_, N0(), st_);
+      k_cast<float, double><<<2 * RED_BLOCKS, 256, 0, s>>>(r_, r32_, N0(), st_);
     T* out = vc(0, s);
     k_scatter_units<double, T><<<g, 256, 0, s>>>(out, z_user, v.perm, v.n, B);
     AGG_CK(cudaGetLastError());

@@ -24,13 +24,13 @@ namespace aggmg {
 
 constexpr int SL = 32;          // units per slice
 constexpr int NT = 128;         // threads per block of the unit kernels (B <= 32)
-constexpr int RED_BLOCKS = 1216; // fixed grid of the reduction kernels (152 SMs x 8)
-constexpr int RED_NT = 256;
+constexpr int RED_BLOCKS = 304;  // largest grid of the vector kernels (152 SMs x 2)
+constexpr int RED_NT = 512;
 
 // ---------------------------------------------------------------- PCG state
 struct CGState {
   double rho, alpha, beta, pq, rr, r0, tol, rtol, atol;
-  double rz_old;              // (r_{k+1}, z_k) for the flexible variant
+  double rz;                  // (r, z) of the last preconditioned residual; rho follows it at the iteration's end
   int iter, done, status, max_it, flexible, use_cond;
   int guard;                  // WHILE-body executions of this solve (hard stop)
   unsigned long long cond;    // cudaGraphConditionalHandle of the WHILE node
@@ -307,18 +307,19 @@ __device__ __forceinline__ double warp_sum(double v) {
   return v;
 }
 
-// Sum over the block; result valid in thread 0.
+// Sum over the block; result valid in warp 0. The values meet in shared memory
+// and one warp adds them: NTH / 32 + 4 float64 adds per lane of one warp instead of
+// five in every warp (an add occupies the SM's float64 pipe for 16 clocks a warp).
 template <int NTH>
 __device__ __forceinline__ double block_sum(double v) {
-  __shared__ double sh[NTH / 32];
-  v = warp_sum(v);
-  const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
+  __shared__ double sh[NTH];
   __syncthreads();
-  if (l == 0) sh[w] = v;
+  sh[threadIdx.x] = v;
   __syncthreads();
   double s = 0.0;
-  if (w == 0) {
-    s = (l < NTH / 32) ? sh[l] : 0.0;
+  if (threadIdx.x < 32) {
+#pragma unroll
+    for (int k = 0; k < NTH / 32; ++k) s += sh[k * 32 + threadIdx.x];
     s = warp_sum(s);
   }
   return s;
@@ -344,12 +345,41 @@ __device__ __forceinline__ bool partial_and_last(double v, double* partials, uns
 template <int NTH>
 __device__ __forceinline__ double sum_partials(const double* partials, int n) {
   double s = 0.0;
-  for (int i = threadIdx.x; i < n; i += NTH) s += ((volatile const double*)partials)[i];
+#pragma unroll 4
+  for (int i = threadIdx.x; i < n; i += NTH) s += __ldcg(partials + i);
   return block_sum<NTH>(s);
+}
+// The same for a kernel that uses the sum of an earlier kernel's partials: every
+// thread of the block gets it (each block sums them itself, in the same order).
+// The producer then needs no last block, whose tickets cost it 5 ns a block
+// (2,048 blocks of the float64 product: 10 us).
+template <int NTH>
+__device__ __forceinline__ double all_sum_partials(const double* partials, int n) {
+  __shared__ double all;
+  const double s = sum_partials<NTH>(partials, n);    // (its barriers order this call after an earlier one's read)
+  if (threadIdx.x == 0) all = s;
+  __syncthreads();
+  return all;
+}
+
+// beta of the p update from k_zdot's partials of (r, z) (np of them, followed in
+// the flexible variant by k_cg_update's of (r, z_old) at partials + kPartials):
+// (r, z) / rho or, flexible (Polak-Ribiere), ((r, z) - (r, z_old)) / rho.
+constexpr int kPartials = 1024;     // entries kept for the partials of one sum of the vector kernels
+template <int NTH, bool INIT>
+__device__ __forceinline__ double cg_beta(const double* partials, int np, CGState* st) {
+  const double rz = all_sum_partials<NTH>(partials, np);
+  double beta = 0.0;
+  if (!INIT) beta = (st->flexible ? rz - all_sum_partials<NTH>(partials + kPartials, np) : rz) / st->rho;
+  if (blockIdx.x == 0 && threadIdx.x == 0) {
+    st->rz = rz;
+    st->beta = beta;
+  }
+  return beta;
 }
 
 // ---------------------------------------------------------------- SpMV
-// MODE 0: y = A x;  MODE 1: y = rhs - A x;  MODE 2: y = A x and (x, y) -> alpha
+// MODE 0: y = A x;  MODE 1: y = rhs - A x;  MODE 2: y = A x and per-block partials of (x, y)
 template <typename T, int B, int MODE, typename Op>
 static __global__ void __launch_bounds__(UnitThreads<B>::value, OpMinBlocks<Op>::value)
     k_spmv(Op A, const T* __restrict__ x, const T* __restrict__ rhs, T* __restrict__ y, double* partials,
@@ -377,14 +407,8 @@ static __global__ void __launch_bounds__(UnitThreads<B>::value, OpMinBlocks<Op>:
     }
   }
   if (MODE == 2) {
-    if (partial_and_last<NTB>(part, partials, &st->ticket[0])) {
-      double pq = sum_partials<NTB>(partials, gridDim.x);
-      if (threadIdx.x == 0) {
-        st->pq = pq;
-        st->alpha = st->rho / pq;
-        st->ticket[0] = 0;
-      }
-    }
+    const double s = block_sum<NTB>(part);
+    if (threadIdx.x == 0) partials[blockIdx.x] = s;
   }
 }
 

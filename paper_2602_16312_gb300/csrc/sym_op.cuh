@@ -371,7 +371,7 @@ __device__ __forceinline__ void fx_store(double v, bool active, int slot, int64_
 }
 
 // One level-0 step, y = A0 x inside.
-//   SYM_SPMV, KIND 0: out = y; 1: out = rhs - y; 2: out = y and (x, y) -> alpha
+//   SYM_SPMV, KIND 0: out = y; 1: out = rhs - y; 2: out = y and per-block partials of (x, y)
 //   SYM_CHEB, KIND as in k_cheb: Chebyshev step with the block inverses `ext`;
 //     float64: also writes the new iterate's fixed-point copy (Xo, Eo)
 //   SYM_RESTRICT: out = P^T (rhs - y) with the transfer blocks `ext`
@@ -651,14 +651,8 @@ static __global__ void __launch_bounds__(SymSmem<T, TD, B, OP, KIND>::NTH)
   }
   asm volatile("cp.async.wait_group 0;" ::: "memory");
   if constexpr (OP == SYM_SPMV && KIND == 2) {
-    if (partial_and_last<M::NTH>(part, partials, &st->ticket[0])) {
-      const double pq = sum_partials<M::NTH>(partials, gridDim.x);
-      if (threadIdx.x == 0) {
-        st->pq = pq;
-        st->alpha = st->rho / pq;
-        st->ticket[0] = 0;
-      }
-    }
+    const double s = block_sum<M::NTH>(part);
+    if (threadIdx.x == 0) partials[blockIdx.x] = s;
   }
 }
 
@@ -933,14 +927,8 @@ static __global__ void __launch_bounds__(SymRing<T, TD, B, OP, KIND>::NTH, SymRi
   }
   asm volatile("cp.async.wait_group 0;" ::: "memory");
   if constexpr (OP == SYM_SPMV && KIND == 2) {
-    if (partial_and_last<M::NTH>(dot, partials, &st->ticket[0])) {
-      const double pq = sum_partials<M::NTH>(partials, gridDim.x);
-      if (threadIdx.x == 0) {
-        st->pq = pq;
-        st->alpha = st->rho / pq;
-        st->ticket[0] = 0;
-      }
-    }
+    const double s = block_sum<M::NTH>(dot);
+    if (threadIdx.x == 0) partials[blockIdx.x] = s;
   }
 }
 
@@ -1012,22 +1000,26 @@ static __global__ void __launch_bounds__(SymRows<B>::NT)
   fx_store<B>(active ? x[(size_t)unit * B + r] : 0.0, active, slot, unit, r, sc, X, E, se, SymRows<B>::U);
 }
 // p = z + beta p (INIT: p = z), as k_pupd, with p's fixed-point copy
-template <int B, bool INIT>
+template <typename TZ, int B, bool INIT>
 static __global__ void __launch_bounds__(SymRows<B>::NT)
-    k_pupd_fx(const double* __restrict__ z, double* __restrict__ p, int64_t n, const int16_t* __restrict__ sc,
-              int2* __restrict__ X, int* __restrict__ E, const CGState* st) {
+    k_pupd_fx(const TZ* __restrict__ z, double* __restrict__ p, int64_t n, const double* partials, int np,
+              const int16_t* __restrict__ sc, int2* __restrict__ X, int* __restrict__ E, CGState* st) {
   if (st->done) return;
   __shared__ int se[SymRows<B>::U];
+  const double beta = cg_beta<SymRows<B>::NT, INIT>(partials, np, st);
   const int slot = threadIdx.x / B, r = threadIdx.x - slot * B;
-  const int64_t unit = (int64_t)blockIdx.x * SymRows<B>::U + slot;
-  const bool active = slot < SymRows<B>::U && unit < n;
-  const size_t o = (size_t)unit * B + r;
-  double v = 0.0;
-  if (active) {
-    v = INIT ? z[o] : z[o] + st->beta * p[o];
-    p[o] = v;
+  for (int64_t u0 = (int64_t)blockIdx.x * SymRows<B>::U; u0 < n; u0 += (int64_t)gridDim.x * SymRows<B>::U) {
+    const int64_t unit = u0 + slot;
+    const bool active = slot < SymRows<B>::U && unit < n;
+    const size_t o = (size_t)unit * B + r;
+    double v = 0.0;
+    if (active) {
+      v = INIT ? (double)z[o] : (double)z[o] + beta * p[o];
+      p[o] = v;
+    }
+    fx_store<B>(v, active, slot, unit, r, sc, X, E, se, SymRows<B>::U);
+    __syncthreads();
   }
-  fx_store<B>(v, active, slot, unit, r, sc, X, E, se, SymRows<B>::U);
 }
 
 }  // namespace aggmg
