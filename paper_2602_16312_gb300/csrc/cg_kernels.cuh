@@ -127,10 +127,10 @@ static __global__ void __launch_bounds__(RED_NT) k_cg_update(double* __restrict_
     s += rv.y * rv.y;
     if (flex) {
       const Z2 zv = reinterpret_cast<const Z2*>(zold)[i];
-      sz += rv.x * (double)zv.x;
-      sz += rv.y * (double)zv.y;
+      sz += rv.x * to_double(zv.x);
+      sz += rv.y * to_double(zv.y);
     }
-    if (r32) reinterpret_cast<float2*>(r32)[i] = make_float2((float)rv.x, (float)rv.y);
+    if (r32) reinterpret_cast<float2*>(r32)[i] = make_float2(to_float(rv.x), to_float(rv.y));
   }
   if ((n & 1) && blockIdx.x == 0 && threadIdx.x == 0) {
     const int64_t i = n - 1;
@@ -179,8 +179,8 @@ static __global__ void __launch_bounds__(RED_NT) k_zdot(const TZ* __restrict__ z
   for (int64_t i = (int64_t)blockIdx.x * RED_NT + threadIdx.x; i < n2; i += (int64_t)gridDim.x * RED_NT) {
     const Z2 zv = reinterpret_cast<const Z2*>(z)[i];
     const double2 rv = reinterpret_cast<const double2*>(r)[i];
-    s += rv.x * (double)zv.x;
-    s += rv.y * (double)zv.y;
+    s += rv.x * to_double(zv.x);
+    s += rv.y * to_double(zv.y);
   }
   if ((n & 1) && blockIdx.x == 0 && threadIdx.x == 0) s += r[n - 1] * (double)z[n - 1];
   const double b = block_sum<RED_NT>(s);
@@ -198,7 +198,7 @@ static __global__ void __launch_bounds__(RED_NT) k_pupd(const TZ* __restrict__ z
 #pragma unroll 2
   for (int64_t i = (int64_t)blockIdx.x * RED_NT + threadIdx.x; i < n2; i += (int64_t)gridDim.x * RED_NT) {
     const Z2 zv = reinterpret_cast<const Z2*>(z)[i];
-    double2 pv = make_double2((double)zv.x, (double)zv.y);
+    double2 pv = make_double2(to_double(zv.x), to_double(zv.y));
     if (!INIT) {
       const double2 po = reinterpret_cast<const double2*>(p)[i];
       pv.x += beta * po.x;

@@ -969,10 +969,21 @@ class Engine : public EngineBase {
     return xo;
   }
 
-  // Chebyshev step KIND 1 or 2 on level v with operator op
+  // Chebyshev step (KIND as in k_cheb) on level v with operator op
   template <int KIND, typename Op>
   void cheb_step(const Op& op, Lev& v, const T* xo, T* xn, T c1, T c2, cudaStream_t s, const CGState* st) {
-    k_cheb<T, TD, B, KIND, Op><<<bgrid(0, v.nsl), NTB, 0, s>>>(op, v.Dinv, v.rhs, xo, xn, v.d, c1, c2, v.nsl, st);
+    if constexpr (kMf && std::is_same<Op, MfOpT>::value)
+      k_mf_cheb<T, TD, B, KIND, Op><<<bgrid(0, v.nsl), NTB, 0, s>>>(op, v.Dinv, v.rhs, xo, xn, v.d, c1, c2, v.nsl, st);
+    else
+      k_cheb<T, TD, B, KIND, Op><<<bgrid(0, v.nsl), NTB, 0, s>>>(op, v.Dinv, v.rhs, xo, xn, v.d, c1, c2, v.nsl, st);
+  }
+
+  template <typename Op>
+  void resid_restrict(const Op& op, Lev& v, const T* x, cudaStream_t s, const CGState* st) {
+    if constexpr (kMf && std::is_same<Op, MfOpT>::value)
+      k_mf_restrict<T, B, Op><<<bgrid(0, v.nsl), NTB, 0, s>>>(op, v.P, v.rhs, x, v.S, v.nsl, st);
+    else
+      k_resid_restrict<T, B, Op><<<bgrid(0, v.nsl), NTB, 0, s>>>(op, v.P, v.rhs, x, v.S, st);
   }
 
   // One level of the V-cycle with the level operator `op` (assembled blocks
@@ -983,13 +994,13 @@ class Engine : public EngineBase {
     T* xo = v.xa;
     T* xn = v.xb;
     const int64_t g = bgrid(0, v.nsl);
-    k_cheb<T, TD, B, 0, Op><<<g, NTB, 0, s>>>(op, v.Dinv, v.rhs, nullptr, xo, v.d, T(0), v.c2[0], v.nsl, st_);
+    cheb_step<0>(op, v, nullptr, xo, T(0), v.c2[0], s, st_);
     for (int k = 1; k < degree_; ++k) {
       cheb_step<2>(op, v, xo, xn, v.c1[k], v.c2[k], s, st_);
       std::swap(xo, xn);
     }
     Lev& c = lev_[l + 1];
-    k_resid_restrict<T, B, Op><<<g, NTB, 0, s>>>(op, v.P, v.rhs, xo, v.S, st_);
+    resid_restrict(op, v, xo, s, st_);
     if (!fused_restrict(l + 1))
       k_segsum<T, B><<<cdiv(c.n * B, 256), 256, 0, s>>>(c.child_ptr, v.S, c.rhs, c.n, st_);
     T* ec = vc(l + 1, s);
@@ -1670,7 +1681,7 @@ class Engine : public EngineBase {
           break;
         case 2:
           if (use_mf0())
-            k_resid_restrict<T, B, MfOpT><<<bgrid(0, n), NTB, 0, s>>>(mfop_, v.P, v.rhs, v.xa, v.S, nullptr);
+            resid_restrict(mfop_, v, v.xa, s, nullptr);
           else if (sym_)
             sym_restrict(v, v.xa, s, nullptr);
           else

@@ -300,6 +300,26 @@ __device__ __forceinline__ void sell_row(const SellView<T>& A, int64_t slice, in
   }
 }
 
+// ---------------------------------------------------------------- conversions
+// float <-> double on the integer pipe (a cvt occupies the float64 pipe as long
+// as an FMA, 16 clocks per warp and SM): the same values, round to nearest even.
+// Zeros, subnormals, infinities, NaN and results outside float's normal range
+// take the instruction.
+__device__ __forceinline__ double to_double(float f) {
+  const unsigned u = __float_as_uint(f), e = (u >> 23) & 0xff;
+  if (e == 0 || e == 255) return (double)f;
+  return __hiloint2double((int)((u & 0x80000000u) | (((u & 0x7fffffffu) >> 3) + 0x38000000u)), (int)(u << 29));
+}
+__device__ __forceinline__ double to_double(double d) { return d; }
+__device__ __forceinline__ float to_float(double d) {
+  const unsigned hi = (unsigned)__double2hiint(d), lo = (unsigned)__double2loint(d), e = (hi >> 20) & 0x7ff;
+  if (e < 897 || e > 1149) return (float)d;
+  const unsigned b = (((hi & 0x7fffffffu) << 3) | (lo >> 29)) - (896u << 23);
+  const unsigned rem = lo & 0x1fffffffu;
+  const unsigned up = (rem > 0x10000000u || (rem == 0x10000000u && (b & 1u))) ? 1u : 0u;
+  return __uint_as_float((hi & 0x80000000u) | (b + up));
+}
+
 // ---------------------------------------------------------------- reductions
 __device__ __forceinline__ double warp_sum(double v) {
 #pragma unroll

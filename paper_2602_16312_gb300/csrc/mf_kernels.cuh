@@ -11,9 +11,111 @@
 // normal, + = e, - = neighbour; wdS folded into a, b, s):
 //   -1/2 phi_i (a.grad u+ + b.grad u-) - 1/2 (a.grad phi_i) (u+ - u-) + s (u+ - u-) phi_i
 #pragma once
+#include "face_op.cuh"
 #include "kernels.cuh"
 
 namespace aggmg {
+
+// How a thread reads its element's and its neighbours' DoFs of a unit-major
+// vector: straight from memory, or through the warp's stage in shared memory.
+// Straight, the lanes of a load lie B entries apart and touch up to 32 cache
+// lines: for Q2 hexahedra these loads bound the smoothing step (345 us on the
+// 64^3 cube, against 253 us for its bytes; 304 us now). The stage is filled by coalesced
+// loads (an element's entries by consecutive lanes): own values for the whole
+// slice at once, a neighbour per fetch.
+template <typename R, int B>
+struct DirectDofs {
+  const R* x;
+  int64_t unit;
+  __device__ __forceinline__ R own(int i) const { return x[(size_t)unit * B + i]; }
+  __device__ __forceinline__ void fetch(int) const {}
+  __device__ __forceinline__ R nbr(int nb, int i) const { return x[(size_t)nb * B + i]; }
+};
+// Position of entry i of lane `el` in a stage: neither the lanes of one entry nor
+// the entries of one element share a bank. Rows of 33 need no address
+// arithmetic for constant i; 64-DoF blocks swizzle rows of 32 instead, to stay
+// within 48 KB of shared memory.
+template <int B> constexpr int kStageSize = B * (B > 32 ? SL : SL + 1);
+template <int B>
+__device__ __forceinline__ int stage_at(int i, int el) {
+  return B > 32 ? i * SL + (el ^ (i & (SL - 1))) : i * (SL + 1) + el;
+}
+// a slice's B x 32 consecutive entries into a stage, and back
+template <int B, typename R>
+__device__ __forceinline__ void stage_in(R* st, const R* __restrict__ g, int lane) {
+#pragma unroll 9
+  for (int k = 0; k < B; ++k) {
+    const int id = k * SL + lane, el = id / B;
+    st[stage_at<B>(id - el * B, el)] = g[id];
+  }
+}
+// the same with copies that complete in the background (one commit group)
+template <int B, typename R>
+__device__ __forceinline__ void stage_in_async(R* st, const R* __restrict__ g, int lane) {
+  static_assert(sizeof(R) == 4, "4-byte copies");
+#pragma unroll 9
+  for (int k = 0; k < B; ++k) {
+    const int id = k * SL + lane, el = id / B;
+    const unsigned dst = (unsigned)__cvta_generic_to_shared(st + stage_at<B>(id - el * B, el));
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(dst), "l"(g + id) : "memory");
+  }
+  asm volatile("cp.async.commit_group;" ::: "memory");
+}
+template <int PENDING>
+__device__ __forceinline__ void stage_wait() {
+  asm volatile("cp.async.wait_group %0;" ::"n"(PENDING) : "memory");
+  __syncwarp();
+}
+template <int B, typename R>
+__device__ __forceinline__ void stage_out(const R* st, R* __restrict__ g, int lane) {
+#pragma unroll 9
+  for (int k = 0; k < B; ++k) {
+    const int id = k * SL + lane, el = id / B;
+    g[id] = st[stage_at<B>(id - el * B, el)];
+  }
+}
+// Neighbours of 27-DoF blocks are read straight from memory: staged, a fetch's
+// latency is exposed once per face to the 12 warps that the registers of the
+// Q2 hexahedron leave on an SM (smoothing step on the 64^3 cube 385 us staged, 304 us straight).
+#ifndef AGG_MF_DIRECT_NBR
+#define AGG_MF_DIRECT_NBR (B == 27)
+#endif
+template <typename R, int B>
+struct StagedDofs {
+  static constexpr bool kDirect = AGG_MF_DIRECT_NBR;
+  const R* x;
+  const R* xs;             // the slice's own values
+  R* ns;                   // a neighbour's values per lane
+  int lane;
+  __device__ __forceinline__ R own(int i) const { return xs[stage_at<B>(i, lane)]; }
+  // every lane of the warp calls this with its neighbour (-1: none)
+  __device__ __forceinline__ void fetch(int nb) const {
+    if constexpr (kDirect) return;
+    __syncwarp();
+    if constexpr (B <= 32) {
+      constexpr int EPI = 32 / B, kIt = (32 + EPI - 1) / EPI;
+      const int sub = lane / B, c = lane - sub * B;
+#pragma unroll 8
+      for (int it = 0; it < kIt; ++it) {
+        const int j = it * EPI + sub;
+        const int n = __shfl_sync(0xffffffffu, nb, j & 31);
+        if (sub < EPI && j < 32 && n >= 0) ns[stage_at<B>(c, j)] = x[(size_t)n * B + c];
+      }
+    } else {
+#pragma unroll 4
+      for (int j = 0; j < 32; ++j) {
+        const int n = __shfl_sync(0xffffffffu, nb, j);
+        if (n < 0) continue;
+#pragma unroll
+        for (int c = lane; c < B; c += 32) ns[stage_at<B>(c, j)] = x[(size_t)n * B + c];
+      }
+    }
+    __syncwarp();
+  }
+  __device__ __forceinline__ R nbr(int nb, int i) const {
+    return kDirect ? x[(size_t)nb * B + i] : ns[stage_at<B>(i, lane)];
+  }
+};
 
 template <int B> struct MfDegree;
 template <> struct MfDegree<4> { static constexpr int value = 1; };
@@ -95,13 +197,17 @@ struct MfOpV {
 
   // acc += ((c M + A) x)_e for the thread's element
   __device__ __forceinline__ void apply(int64_t slice, int lane, const R* __restrict__ x, R* acc) const {
+    apply_with(slice, lane, DirectDofs<R, B>{x, slice * SL + lane}, acc);
+  }
+  // the same, the DoFs read through `dofs` (DirectDofs or StagedDofs)
+  template <typename Dofs>
+  __device__ __forceinline__ void apply_with(int64_t slice, int lane, const Dofs& dofs, R* acc) const {
     constexpr int N = MfDegree<B>::value + 1;
-    const int64_t unit = slice * SL + lane;
     R u[N * N];
 #pragma unroll
-    for (int i = 0; i < N * N; ++i) u[i] = x[(size_t)unit * B + i];
+    for (int i = 0; i < N * N; ++i) u[i] = dofs.own(i);
     cell(slice, lane, u, acc);
-    faces(slice, lane, x, u, acc);
+    faces(slice, lane, dofs, u, acc);
   }
 
   // acc += the cell (volume and mass) terms of the element whose DoFs are u;
@@ -233,14 +339,15 @@ struct MfOpV {
     }
   }
 
-  // acc += the face terms of the element whose DoFs are u (x: all DoFs, for
-  // the neighbours)
-  __device__ __forceinline__ void faces(int64_t slice, int lane, const R* __restrict__ x, const R* u, R* acc) const {
+  // acc += the face terms of the element whose DoFs are u
+  template <typename Dofs>
+  __device__ __forceinline__ void faces(int64_t slice, int lane, const Dofs& dofs, const R* u, R* acc) const {
     constexpr int P = MfDegree<B>::value, N = P + 1, Q = P + 2;
 #pragma unroll
     for (int f = 0; f < 4; ++f) {
       const size_t fi = ((size_t)slice * 4 + f) * SL + lane;
       const int nb = V.nbr[fi];
+      dofs.fetch(nb);
       if (nb < 0) continue;
       const int code = V.code[fi];
       const int fn = code >> 1, rev = code & 1;
@@ -257,7 +364,7 @@ struct MfOpV {
       }
       R xn[N * N];
 #pragma unroll
-      for (int i = 0; i < N * N; ++i) xn[i] = x[(size_t)nb * B + i];
+      for (int i = 0; i < N * N; ++i) xn[i] = dofs.nbr(nb, i);
       R un[Q], gn0[Q], gn1[Q];
       switch (fn) {
         case 0: mf_nbr_face<R, P, 0, 0>(T, xn, un, gn0, gn1); break;
@@ -331,11 +438,15 @@ struct MfOp3V {
   __device__ __forceinline__ int64_t nslices() const { return V.nslices; }
 
   __device__ __forceinline__ void apply(int64_t slice, int lane, const R* __restrict__ x, R* acc) const {
+    apply_with(slice, lane, DirectDofs<R, B>{x, slice * SL + lane}, acc);
+  }
+  // the same, the DoFs read through `dofs` (DirectDofs or StagedDofs)
+  template <typename Dofs>
+  __device__ __forceinline__ void apply_with(int64_t slice, int lane, const Dofs& dofs, R* acc) const {
     constexpr int P = kDegree, N = P + 1, Q = P + 2, NN = N * N, QQ = Q * Q;
-    const int64_t unit = slice * SL + lane;
     R u[B];
 #pragma unroll
-    for (int i = 0; i < B; ++i) u[i] = x[(size_t)unit * B + i];
+    for (int i = 0; i < B; ++i) u[i] = dofs.own(i);
     const R* cd = V.cell + (size_t)slice * QQ * Q * 7 * SL + lane;
     // The test-side sums of the face terms (and for B = 64 those of the cell
     // term too) go to the thread's column of a shared array: no register
@@ -443,16 +554,16 @@ struct MfOp3V {
     }
     // ---- face terms: one pass per face at run time; both sides' traces are
     // read from memory through strides
-    const R* xe = x + (size_t)unit * B;
 #pragma unroll 1
     for (int f = 0; f < 6; ++f) {
       const size_t fi = ((size_t)slice * 6 + f) * SL + lane;
       const int nb = V.nbr[fi];
+      dofs.fetch(nb);
       if (nb < 0) continue;
       const int fnb = V.code[fi];
       R sU[N][Q], sT[N][Q], sN[N][Q], nU[N][Q], nT[N][Q], nN[N][Q];
-      face_trace(xe, f, sU, sT, sN);
-      face_trace(x + (size_t)nb * B, fnb, nU, nT, nN);
+      face_trace([&](int i) { return dofs.own(i); }, f, sU, sT, sN);
+      face_trace([&](int i) { return dofs.nbr(nb, i); }, fnb, nU, nT, nN);
       R rF[N][Q], rT[N][Q], rN[N][Q];
 #pragma unroll
       for (int j2 = 0; j2 < N; ++j2)
@@ -519,17 +630,18 @@ struct MfOp3V {
   }
 
   // Trace (U), derivative along the first tangential axis (Tn) and normal
-  // derivative (Nr) on local face f of the element whose DoFs start at xb,
+  // derivative (Nr) on local face f of the element with DoFs x(i),
   // interpolated to the Gauss points along the first tangential axis and
   // kept at the nodes along the second: [j2][q1].
-  __device__ __forceinline__ void face_trace(const R* __restrict__ xb, int f, R (&U)[kDegree + 1][kDegree + 2],
+  template <typename X>
+  __device__ __forceinline__ void face_trace(X x, int f, R (&U)[kDegree + 1][kDegree + 2],
                                              R (&Tn)[kDegree + 1][kDegree + 2],
                                              R (&Nr)[kDegree + 1][kDegree + 2]) const {
     constexpr int P = kDegree, N = P + 1, Q = P + 2, NN = N * N;
     const int k = f >> 1, sd = f & 1;
     const int SK = (k == 0) ? 1 : (k == 1 ? N : NN);
     const int S0 = (k == 0) ? N : 1, S1 = (k == 2) ? N : NN;
-    const R* xf = xb + sd * P * SK;
+    const int f0 = sd * P * SK;
 #pragma unroll
     for (int j2 = 0; j2 < N; ++j2) {
       R tr[N], dn[N];
@@ -539,10 +651,10 @@ struct MfOp3V {
 #pragma unroll
         for (int i = 0; i < N; ++i) {
           const R de = sd ? T.Dend[1][i] : T.Dend[0][i];
-          s += de * xb[i * SK + j1 * S0 + j2 * S1];
+          s += de * x(i * SK + j1 * S0 + j2 * S1);
         }
         dn[j1] = s;
-        tr[j1] = xf[j1 * S0 + j2 * S1];
+        tr[j1] = x(f0 + j1 * S0 + j2 * S1);
       }
 #pragma unroll
       for (int q1 = 0; q1 < Q; ++q1) {
@@ -569,6 +681,147 @@ template <typename R> struct MfOpForT<R, 8> { using type = MfOp3V<R, 8>; };
 template <typename R> struct MfOpForT<R, 27> { using type = MfOp3V<R, 27>; };
 template <typename R> struct MfOpForT<R, 64> { using type = MfOp3V<R, 64>; };
 template <int B> struct MfOpFor { using type = typename MfOpForT<float, B>::type; };
+
+// ---------------------------------------------------------------- level-0 kernels, staged vectors
+// Stages of a warp: own values, a neighbour's values, and rhs and d, whose copies
+// run behind the operator and the block inverse. 27-DoF blocks, which do not stage
+// neighbours, and 64-DoF ones (48 KB of shared memory) have no third stage.
+template <int B> struct MfStages {
+  static constexpr int value = (B <= 16) ? 3 : 2;
+  static constexpr bool kEarly = (B <= 27);           // rhs is staged before the operator
+};
+// Chebyshev step as k_cheb with a matrix-free operator; every vector goes
+// through the warp's stages. 512^2 Q2 square: 54.4 -> 44.9 us.
+template <typename T, typename TD, int B, int KIND, typename Op>
+static __global__ void __launch_bounds__(UnitThreads<B>::value, OpMinBlocks<Op>::value)
+    k_mf_cheb(Op A, const TD* __restrict__ Dinv, const T* __restrict__ rhs, const T* __restrict__ x_old,
+              T* __restrict__ x_new, T* __restrict__ d, T c1, T c2, int64_t nslices, const CGState* st) {
+  constexpr int NTB = UnitThreads<B>::value, KPD = DinvPad<TD, B>::KP;
+  constexpr int kStages = MfStages<B>::value;
+  constexpr bool kEarly = MfStages<B>::kEarly;
+  __shared__ T stage[NTB / 32][kStages][kStageSize<B>];
+  if (st && st->done) return;
+  const int lane = threadIdx.x & 31;
+  const int64_t slice = first_slice<NTB>();
+  if (slice >= nslices) return;
+  T* xs = stage[threadIdx.x >> 5][0];
+  T* ns = stage[threadIdx.x >> 5][1];
+  T* rs = stage[threadIdx.x >> 5][kStages - 1];      // rhs, d (with two stages: where the neighbours' were)
+  const size_t o = (size_t)slice * SL * B;
+  const TD* Db = Dinv + (size_t)slice * SL * KPD;
+  T t[B];
+  if (KIND == 0) {
+    stage_in<B>(xs, rhs + o, lane);
+    __syncwarp();
+#pragma unroll
+    for (int r = 0; r < B; ++r) t[r] = xs[stage_at<B>(r, lane)];
+  } else {
+    stage_in_async<B>(xs, x_old + o, lane);
+    if (kEarly) stage_in_async<B>(rs, rhs + o, lane);
+    stage_wait<kEarly ? 1 : 0>();
+#pragma unroll
+    for (int r = 0; r < B; ++r) t[r] = T(0);
+    A.apply_with(slice, lane, StagedDofs<T, B>{x_old, xs, ns, lane}, t);
+    if (!kEarly) {
+      __syncwarp();
+      stage_in_async<B>(rs, rhs + o, lane);
+    }
+    stage_wait<0>();
+#pragma unroll
+    for (int r = 0; r < B; ++r) t[r] = rs[stage_at<B>(r, lane)] - t[r];
+    if (KIND == 2 && B <= 32) {
+      __syncwarp();
+      stage_in_async<B>(rs, d + o, lane);
+    }
+  }
+  T s[B];
+#pragma unroll
+  for (int r = 0; r < B; ++r) s[r] = T(0);
+  if constexpr (B > 32) {
+    // (the column loop reads t at run-time indices: from the lane's own stage slots)
+#pragma unroll
+    for (int r = 0; r < B; ++r) ns[stage_at<B>(r, lane)] = t[r];
+    __syncwarp();
+    rect_mv<TD, T, B, B>(Db, lane, [&](int c) { return ns[stage_at<B>(c, lane)]; }, [](int r) { return r; }, s);
+  } else {
+    sym_block_mv<TD, T, B>(Db, lane, t, s);
+  }
+  if (KIND == 2) {
+    if (B > 32) {
+      __syncwarp();
+      stage_in_async<B>(rs, d + o, lane);
+    }
+    stage_wait<0>();
+  } else {
+    __syncwarp();
+  }
+#pragma unroll
+  for (int r = 0; r < B; ++r) {
+    const T dn = (KIND == 2) ? c1 * rs[stage_at<B>(r, lane)] + c2 * s[r] : c2 * s[r];
+    rs[stage_at<B>(r, lane)] = dn;
+    if (KIND != 0) xs[stage_at<B>(r, lane)] += dn;
+  }
+  __syncwarp();
+  stage_out<B>(rs, d + o, lane);
+  stage_out<B>(KIND == 0 ? rs : xs, x_new + o, lane);
+}
+
+// S_u = P_u^T (rhs_u - (A x)_u), as k_resid_restrict
+template <typename T, int B, typename Op>
+static __global__ void __launch_bounds__(UnitThreads<B>::value, OpMinBlocks<Op>::value)
+    k_mf_restrict(Op A, const T* __restrict__ P, const T* __restrict__ rhs, const T* __restrict__ x, T* __restrict__ S,
+                  int64_t nslices, const CGState* st) {
+  constexpr int NTB = UnitThreads<B>::value, KP = Pad<T, B>::KP, VW = Vec<T>::W;
+  constexpr int kStages = MfStages<B>::value;
+  constexpr bool kEarly = MfStages<B>::kEarly;
+  __shared__ T stage[NTB / 32][kStages][kStageSize<B>];
+  if (st && st->done) return;
+  const int lane = threadIdx.x & 31;
+  const int64_t slice = first_slice<NTB>();
+  if (slice >= nslices) return;
+  T* xs = stage[threadIdx.x >> 5][0];
+  T* ns = stage[threadIdx.x >> 5][1];
+  T* rs = stage[threadIdx.x >> 5][kStages - 1];      // rhs, d (with two stages: where the neighbours' were)
+  const size_t o = (size_t)slice * SL * B;
+  const T* Pb = P + (size_t)slice * SL * KP;
+  stage_in_async<B>(xs, x + o, lane);
+  if (kEarly) stage_in_async<B>(rs, rhs + o, lane);
+  stage_wait<kEarly ? 1 : 0>();
+  T t[B];
+#pragma unroll
+  for (int r = 0; r < B; ++r) t[r] = T(0);
+  A.apply_with(slice, lane, StagedDofs<T, B>{x, xs, ns, lane}, t);
+  if (!kEarly) {
+    __syncwarp();
+    stage_in_async<B>(rs, rhs + o, lane);
+  }
+  stage_wait<0>();
+#pragma unroll
+  for (int r = 0; r < B; ++r) t[r] = rs[stage_at<B>(r, lane)] - t[r];
+  if constexpr (B > 32) {
+#pragma unroll 1
+    for (int c = 0; c < B; ++c) {
+      T s = T(0);
+#pragma unroll
+      for (int rr = 0; rr < B / VW; ++rr) {
+        T v[VW];
+        ChunkLoad<T, T>::load(Pb, c * (B / VW) + rr, lane, v);
+#pragma unroll
+        for (int k = 0; k < VW; ++k) s += v[k] * t[rr * VW + k];
+      }
+      xs[stage_at<B>(c, lane)] = s;
+    }
+  } else {
+    T s[B];
+#pragma unroll
+    for (int r = 0; r < B; ++r) s[r] = T(0);
+    block_mtv<T, T, B>(Pb, lane, t, s);
+#pragma unroll
+    for (int r = 0; r < B; ++r) xs[stage_at<B>(r, lane)] = s[r];
+  }
+  __syncwarp();
+  stage_out<B>(xs, S + o, lane);
+}
 
 // Sliced block-sparse operator in the same interface.
 template <typename T, int B>

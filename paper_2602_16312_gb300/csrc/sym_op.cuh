@@ -1014,7 +1014,7 @@ static __global__ void __launch_bounds__(SymRows<B>::NT)
     const size_t o = (size_t)unit * B + r;
     double v = 0.0;
     if (active) {
-      v = INIT ? (double)z[o] : (double)z[o] + beta * p[o];
+      v = INIT ? to_double(z[o]) : to_double(z[o]) + beta * p[o];
       p[o] = v;
     }
     fx_store<B>(v, active, slot, unit, r, sc, X, E, se, SymRows<B>::U);
