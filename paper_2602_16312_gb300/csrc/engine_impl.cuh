@@ -632,13 +632,14 @@ class Engine : public EngineBase {
     sym_blocks_[slot] = nb * num_sms_;
     return AGG_OK;
   }
-  int prepare_sym_kernels(std::string& err) {
+  int prepare_sym_kernels(bool matrix_free, std::string& err) {
     int rc;
     if (osym_) {
       if ((rc = prepare_sym<double, double, SYM_SPMV, 0>(0, err))) return rc;
       if ((rc = prepare_sym<double, double, SYM_SPMV, 1>(1, err))) return rc;
       if ((rc = prepare_sym<double, double, SYM_SPMV, 2>(2, err))) return rc;
     }
+    if (matrix_free && B == 64 && (rc = prepare_sym<T, TD, SYM_CHEB, 0>(4, err))) return rc;
     if (!sym_) return AGG_OK;
     if ((rc = prepare_sym<T, TD, SYM_SPMV, 0>(3, err))) return rc;
     if ((rc = prepare_sym<T, TD, SYM_CHEB, 0>(4, err))) return rc;
@@ -994,7 +995,8 @@ class Engine : public EngineBase {
     T* xo = v.xa;
     T* xn = v.xb;
     const int64_t g = bgrid(0, v.nsl);
-    cheb_step<0>(op, v, nullptr, xo, T(0), v.c2[0], s, st_);
+    if (B == 64 && l == 0 && use_mf0()) sym_cheb<0>(v, nullptr, xo, T(0), v.c2[0], s, st_);
+    else cheb_step<0>(op, v, nullptr, xo, T(0), v.c2[0], s, st_);
     for (int k = 1; k < degree_; ++k) {
       cheb_step<2>(op, v, xo, xn, v.c1[k], v.c2[k], s, st_);
       std::swap(xo, xn);
@@ -1004,7 +1006,8 @@ class Engine : public EngineBase {
     if (!fused_restrict(l + 1))
       k_segsum<T, B><<<cdiv(c.n * B, 256), 256, 0, s>>>(c.child_ptr, v.S, c.rhs, c.n, st_);
     T* ec = vc(l + 1, s);
-    k_prolong<T, B, OpStreams<Op>::value><<<g, NTB, 0, s>>>(v.P, v.parent, ec, xo, v.nsl, st_);
+    if (B >= 27 && l == 0 && use_mf0()) sym_prolong(v, ec, xo, s, st_);
+    else k_prolong<T, B, OpStreams<Op>::value><<<g, NTB, 0, s>>>(v.P, v.parent, ec, xo, v.nsl, st_);
     cheb_step<1>(op, v, xo, xn, T(0), v.c2[0], s, st_);
     std::swap(xo, xn);
     for (int k = 1; k < degree_; ++k) {
@@ -1313,7 +1316,17 @@ class Engine : public EngineBase {
           if (kStream && (rc = upload_sym_blocks<false, true>(h.lev[0].P, m.ne, sPT_, err))) return rc;
         }
       }
-      if ((rc = prepare_sym_kernels(err))) return rc;
+      if (B >= 27 && !assembled && nlev_ > 1) {
+        // matrix-free level 0: its prolongation (and, for 64 DoFs, its first
+        // smoothing step) run one thread per row; one thread per element left
+        // most of the GPU idle below ~100,000 elements
+        if ((rc = upload_sym_blocks<false>(h.lev[0].P, m.ne, sP_, err))) return rc;
+        if (B == 64) {
+          if ((rc = upload_sym_blocks<true>(h.lev[0].Dinv, m.ne, sdinv_, err))) return rc;
+          fs_.n = m.ne;
+        }
+      }
+      if ((rc = prepare_sym_kernels(!assembled, err))) return rc;
       const bool face_cycle = assembled && !sym_;
       // (with osym_ only the neighbours, for the adjoint's gradient kernel)
       if (!osym_ || m.adjoint_data || (kDouble && face_cycle)) {
@@ -1688,7 +1701,7 @@ class Engine : public EngineBase {
             k_resid_restrict<T, B, L0Op><<<bgrid(0, n), NTB, 0, s>>>(fop_, v.P, v.rhs, v.xa, v.S, nullptr);
           break;
         case 3:
-          if (sym_ && !use_mf0())
+          if (sym_ || (B >= 27 && use_mf0()))
             sym_prolong(v, lev_[1].xa, v.xb, s, nullptr);
           else
             k_prolong<T, B><<<bgrid(k_prolong<T, B>, n), NTB, 0, s>>>(v.P, v.parent, lev_[1].xa, v.xb, v.nsl, nullptr);

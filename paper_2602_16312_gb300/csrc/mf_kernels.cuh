@@ -432,7 +432,7 @@ template <> struct Mf3Degree<64> { static constexpr int value = 3; };
 template <typename R, int B>
 struct MfOp3V {
   static constexpr int kDegree = Mf3Degree<B>::value;
-  static constexpr int kMinBlocks = AGG_MF3_MINB;
+  static constexpr int kMinBlocks = (AGG_MF3_MINB > 0) ? AGG_MF3_MINB : ((B == 27 && sizeof(R) == 4) ? 3 : 0);
   MfViewT<R> V;
   MfTablesT<R> T;
   __device__ __forceinline__ int64_t nslices() const { return V.nslices; }
@@ -693,7 +693,7 @@ template <int B> struct MfStages {
 // Chebyshev step as k_cheb with a matrix-free operator; every vector goes
 // through the warp's stages. 512^2 Q2 square: 54.4 -> 44.9 us.
 template <typename T, typename TD, int B, int KIND, typename Op>
-static __global__ void __launch_bounds__(UnitThreads<B>::value, OpMinBlocks<Op>::value)
+static __global__ void __launch_bounds__(UnitThreads<B>::value, KIND == 0 ? 0 : OpMinBlocks<Op>::value)
     k_mf_cheb(Op A, const TD* __restrict__ Dinv, const T* __restrict__ rhs, const T* __restrict__ x_old,
               T* __restrict__ x_new, T* __restrict__ d, T c1, T c2, int64_t nslices, const CGState* st) {
   constexpr int NTB = UnitThreads<B>::value, KPD = DinvPad<TD, B>::KP;
