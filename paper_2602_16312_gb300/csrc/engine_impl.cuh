@@ -187,7 +187,8 @@ class Engine : public EngineBase {
   SymView<double, B> A0s_{};
   SymView<T, B> fs_{};
   SymBlk<SymDinv> sdinv_{};
-  SymBlk<SymP> sP_{}, sPT_{};        // transfer blocks, column by column and (streaming form) row by row
+  SymBlk<SymP> sP_{}, sPT_{};        // transfer blocks, column by column and row by row
+  SymBlk<SymDinv> sdinvm_{};         // 64 DoFs: the block inverses column by column
   static constexpr bool kStream = (B <= 32);
   static constexpr int BS = kStream ? B : 27;
   int sym_blocks_[8] = {};           // resident blocks of the k_sym kernels, by sym_slot
@@ -688,10 +689,10 @@ class Engine : public EngineBase {
   // symmetric blocks in the V-cycle precision
   template <int KIND>
   void sym_cheb(Lev& v, const T* xo, T* xn, T c1, T c2, cudaStream_t s, CGState* st) {
-    launch_sym<SYM_CHEB, KIND, T, TD>(4 + KIND, fs_, sdinv_, sym_vec(xo), v.rhs, xo, xn, v.d, fx_of(xn), c1, c2, st, s);
+    launch_sym<SYM_CHEB, KIND, T, TD>(4 + KIND, fs_, (kStream || KIND == 0) ? sdinv_ : sdinvm_, sym_vec(xo), v.rhs, xo, xn, v.d, fx_of(xn), c1, c2, st, s);
   }
   void sym_restrict(Lev& v, const T* x, cudaStream_t s, CGState* st) {
-    launch_sym<SYM_RESTRICT, 0, T, TD>(7, fs_, kStream ? sPT_ : sP_, sym_vec(x), v.rhs, x, v.S, nullptr, FxVec{}, T(0), T(0), st, s);
+    launch_sym<SYM_RESTRICT, 0, T, TD>(7, fs_, sPT_, sym_vec(x), v.rhs, x, v.S, nullptr, FxVec{}, T(0), T(0), st, s);
   }
   void sym_prolong(Lev& v, const T* ec, T* x, cudaStream_t s, CGState* st) {
     k_sym_prolong<T, B><<<cdiv(v.n, SymRows<B>::U), SymRows<B>::NT, 0, s>>>(sP_, v.parent, ec, x, fs_.sc, fx_of(x).X,
@@ -1313,7 +1314,8 @@ class Engine : public EngineBase {
         if (nlev_ > 1) {
           if ((rc = upload_sym_blocks<true>(h.lev[0].Dinv, m.ne, sdinv_, err))) return rc;
           if ((rc = upload_sym_blocks<false>(h.lev[0].P, m.ne, sP_, err))) return rc;
-          if (kStream && (rc = upload_sym_blocks<false, true>(h.lev[0].P, m.ne, sPT_, err))) return rc;
+          if ((rc = upload_sym_blocks<false, true>(h.lev[0].P, m.ne, sPT_, err))) return rc;
+          if (!kStream && (rc = upload_sym_blocks<false>(h.lev[0].Dinv, m.ne, sdinvm_, err))) return rc;
         }
       }
       if (B >= 27 && !assembled && nlev_ > 1) {

@@ -274,8 +274,12 @@ struct SymSmem {
   static constexpr bool kFx = std::is_same<T, double>::value;
   static constexpr bool kProduct = !(OP == SYM_CHEB && KIND == 0);
   static constexpr int U = C::U, G = kProduct ? C::G : 1;
+  // with an operator product, the block inverse or P^T is read from memory, column
+  // by column, instead of shared memory: two stages fit then
+  static constexpr bool kExtMem = kProduct && OP != SYM_SPMV;
   static constexpr int KE = kProduct ? L::KD + S::NFACE * L::KB : 0;
-  static constexpr int KX = (OP == SYM_SPMV) ? 0 : (OP == SYM_CHEB ? SymLay<SD, B>::KD : L::KP);
+  static constexpr int KX = (OP == SYM_CHEB && !kProduct) ? SymLay<SD, B>::KD : 0;
+  static constexpr int KXM = SymLay<SD, B>::KP, CPG = B / G;   // block entries in memory, columns per group
   static constexpr int NX = kProduct ? 1 + S::NFACE : 0;
   static constexpr int NTH = round_to(U * B * G, 32);
   static constexpr size_t kBlk = (size_t)U * KE * sizeof(ST);
@@ -374,7 +378,8 @@ __device__ __forceinline__ void fx_store(double v, bool active, int slot, int64_
 //   SYM_SPMV, KIND 0: out = y; 1: out = rhs - y; 2: out = y and per-block partials of (x, y)
 //   SYM_CHEB, KIND as in k_cheb: Chebyshev step with the block inverses `ext`;
 //     float64: also writes the new iterate's fixed-point copy (Xo, Eo)
-//   SYM_RESTRICT: out = P^T (rhs - y) with the transfer blocks `ext`
+//   SYM_RESTRICT: out = P^T (rhs - y) with the transposed transfer blocks `ext`
+// (ext: column by column, LDP apart; KIND 0 of SYM_CHEB: packed triangles)
 // x: the vector itself (own values); xv: what the products read. The blocks of
 // a launch loop over tiles of U elements, so that the tiles in flight are
 // neighbours and share face blocks through the L2.
@@ -439,7 +444,7 @@ static __global__ void __launch_bounds__(SymSmem<T, TD, B, OP, KIND>::NTH)
       ST* eb = reinterpret_cast<ST*>(base) + slot * M::KE;
       SX* ex = reinterpret_cast<SX*>(base + M::kBlk + M::kExt) + slot * M::NX * BX;
       int* ee = reinterpret_cast<int*>(base + M::kBlk + M::kExt + M::kXs) + slot * M::NX;
-      if constexpr (OP != SYM_SPMV) {
+      if constexpr (M::KX > 0) {
         constexpr int QD = 16 / (int)sizeof(SD);
         const SD* src = ext.v + (size_t)unit * M::KX;
         SD* dst = reinterpret_cast<SD*>(base + M::kBlk) + slot * M::KX;
@@ -517,6 +522,14 @@ static __global__ void __launch_bounds__(SymSmem<T, TD, B, OP, KIND>::NTH)
     const SX* ex = reinterpret_cast<SX*>(base + M::kBlk + M::kExt) + slot * M::NX * BX;
     const int* ee = reinterpret_cast<int*>(base + M::kBlk + M::kExt + M::kXs) + slot * M::NX;
     T own = T(0), rh = T(0), dv = T(0);               // loaded ahead of their use
+    SD ev[M::kExtMem ? M::CPG : 1];
+    if constexpr (M::kExtMem) {
+      if (active) {
+        const SD* e = ext.v + (size_t)unit * M::KXM + (size_t)(g * M::CPG) * S::LDP + r;
+#pragma unroll
+        for (int c = 0; c < M::CPG; ++c) ev[c] = e[c * S::LDP];
+      }
+    }
     if (lead) {
       if (M::kProduct && (KIND == 2 || OP == SYM_CHEB)) own = x[o];
       if (!(OP == SYM_SPMV && KIND != 1)) rh = rhs[o];
@@ -612,13 +625,25 @@ static __global__ void __launch_bounds__(SymSmem<T, TD, B, OP, KIND>::NTH)
       }
       __syncthreads();
       T res = T(0);
-      if (lead) {
+      Sum es = Sum(0);
+      if (active) {
         Acc acc;
-        if constexpr (OP == SYM_CHEB) sym_tri<T, B>(sext, r, ts, acc);
-        else sym_dot<T, B>(sext + r * S::LDP, 1, ts, acc);
+        if constexpr (M::kExtMem) {
+#pragma unroll
+          for (int c = 0; c < M::CPG; ++c) acc.fma(sym_val(ev[c]), ts[g * M::CPG + c]);
+        } else {
+          sym_tri<T, B>(sext, r, ts, acc);
+        }
+        es = acc.sum();
+        if (G > 1 && g > 0) sred[(g - 1) * U * B + slot * B + r] = es;
+      }
+      if (G > 1) __syncthreads();
+      if (lead) {
+#pragma unroll
+        for (int k = 0; k < G - 1; ++k) es += sred[k * U * B + slot * B + r];
         T sv;
-        if constexpr (kFx) sv = Et == 2047 ? nan("") : fx_scale(acc.sum(), Et + kFxBias - ext.k[unit]);
-        else sv = acc.sum();
+        if constexpr (kFx) sv = Et == 2047 ? nan("") : fx_scale(es, Et + kFxBias - ext.k[unit]);
+        else sv = es;
         if constexpr (OP == SYM_RESTRICT) {
           out[o] = sv;
         } else {
