@@ -77,12 +77,9 @@ __device__ __forceinline__ void stage_out(const R* st, R* __restrict__ g, int la
 // Neighbours of 27-DoF blocks are read straight from memory: staged, a fetch's
 // latency is exposed once per face to the 12 warps that the registers of the
 // Q2 hexahedron leave on an SM (smoothing step on the 64^3 cube 385 us staged, 304 us straight).
-#ifndef AGG_MF_DIRECT_NBR
-#define AGG_MF_DIRECT_NBR (B == 27)
-#endif
 template <typename R, int B>
 struct StagedDofs {
-  static constexpr bool kDirect = AGG_MF_DIRECT_NBR;
+  static constexpr bool kDirect = (B == 27);
   const R* x;
   const R* xs;             // the slice's own values
   R* ns;                   // a neighbour's values per lane

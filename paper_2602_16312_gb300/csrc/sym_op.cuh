@@ -16,9 +16,19 @@
 // bank conflicts in shared memory. 2D Q2: 135 instead of 261 stored entries
 // per element, 3D Q2: 1,593 instead of 3,159, 3D Q3: 7,456 instead of 14,848.
 //
-// A block of threads owns a few elements, copies their blocks to shared memory
-// with cp.async, gathers its own and its neighbours' DoFs (coalesced: the
-// threads of an element read one neighbour's DoFs together) and multiplies.
+// Blocks and the neighbours' DoFs (coalesced: the threads of an element read one
+// neighbour's DoFs together) are copied to shared memory with cp.async and
+// multiplied there: per warp through a ring of slots (k_symw, B <= 32), or per
+// block of threads in two stages (k_sym, 64 DoFs: one element's blocks are 53
+// (float32) or 106 KB, too much per warp).
+//
+// Measured on GB300 against one thread per element on the blocks of both
+// directions (k_spmv / k_cheb with FaceOp), which is FP64-bound in float64 and short
+// of loads in flight in float32:
+//   float64 product, 64^3 Q2 hexahedra: 1,483 -> 990 us (3.3 GB; HBM bound 490 us,
+//     the multiply-adds of three integer products per entry take the rest)
+//   float64 product, 24^3 Q3 hexahedra: 1,340 -> 272 us
+//   float64 smoothing step, 18^3 Q3 hexahedra: 1,475 -> 200 us with one stage
 //
 // Float64 products run on the integer pipe. GB300 issues 2 float64 FMAs per
 // SM and clock against 64 32-bit integer multiply-adds, so a float64 block
@@ -135,35 +145,6 @@ template <typename ST, int B> struct SymLay {
   static constexpr int KP = round_to(B * S::LDP, Q);
 };
 
-// Elements per block (U) and thread groups per element (G: group 0 takes the
-// diagonal block, the others share the faces; their sums are added at the end).
-#ifndef AGG_SYM_D9
-#define AGG_SYM_D9 14, 1
-#endif
-#ifndef AGG_SYM_D16
-#define AGG_SYM_D16 8, 1
-#endif
-#ifndef AGG_SYM_D27
-#define AGG_SYM_D27 1, 4
-#endif
-#ifndef AGG_SYM_F9
-#define AGG_SYM_F9 14, 1
-#endif
-template <int U_, int G_> struct SymCfgOf { static constexpr int U = U_, G = G_; };
-template <typename T, int B> struct SymCfg;
-template <> struct SymCfg<double, 4> : SymCfgOf<32, 1> {};
-template <> struct SymCfg<double, 8> : SymCfgOf<16, 1> {};
-template <> struct SymCfg<double, 9> : SymCfgOf<AGG_SYM_D9> {};
-template <> struct SymCfg<double, 16> : SymCfgOf<AGG_SYM_D16> {};
-template <> struct SymCfg<double, 27> : SymCfgOf<AGG_SYM_D27> {};
-template <> struct SymCfg<double, 64> : SymCfgOf<1, 4> {};
-template <> struct SymCfg<float, 4> : SymCfgOf<32, 1> {};
-template <> struct SymCfg<float, 8> : SymCfgOf<16, 1> {};
-template <> struct SymCfg<float, 9> : SymCfgOf<AGG_SYM_F9> {};
-template <> struct SymCfg<float, 16> : SymCfgOf<8, 1> {};
-template <> struct SymCfg<float, 27> : SymCfgOf<4, 1> {};
-template <> struct SymCfg<float, 64> : SymCfgOf<1, 4> {};
-
 template <typename T, int B>
 struct SymView {
   using ST = typename SymNum<T>::ST;
@@ -258,13 +239,14 @@ template <typename T> struct SymVec {
   const int* E;
 };
 
-// Shared memory of a block. Two stages (of everything a tile reads: operator
-// blocks, Dinv or P blocks, x), so that one tile's copies are in flight while
-// the other one is multiplied: GB300 needs about 100 KB in flight per SM to reach
-// its HBM rate. Then the face rows' partial sums, the groups' sums, exponents.
+// Shared memory of a block of k_sym. Two stages (of everything an element's step
+// copies), so that one element's copies are in flight while the other one is
+// multiplied: GB300 needs about 100 KB in flight per SM to reach its HBM rate. Then
+// the face rows' partial sums, the groups' sums, exponents. G groups of B threads
+// share an element: group 0 takes the diagonal block, the others two faces each;
+// their sums are added at the end.
 template <typename T, typename TD, int B, int OP, int KIND>
 struct SymSmem {
-  using C = SymCfg<T, B>;
   using S = SymShape<B>;
   using ST = typename SymNum<T>::ST;
   using SX = typename SymNum<T>::SX;
@@ -273,9 +255,10 @@ struct SymSmem {
   using L = SymLay<ST, B>;
   static constexpr bool kFx = std::is_same<T, double>::value;
   static constexpr bool kProduct = !(OP == SYM_CHEB && KIND == 0);
-  static constexpr int U = C::U, G = kProduct ? C::G : 1;
+  static constexpr int U = 1, G = kProduct ? 4 : 1;
   // with an operator product, the block inverse or P^T is read from memory, column
-  // by column, instead of shared memory: two stages fit then
+  // by column and a group's columns per thread, instead of shared memory, where only
+  // one stage would fit: adjoint step of the 18^3 Q3 cube 21.3 -> 19.5 ms
   static constexpr bool kExtMem = kProduct && OP != SYM_SPMV;
   static constexpr int KE = kProduct ? L::KD + S::NFACE * L::KB : 0;
   static constexpr int KX = (OP == SYM_CHEB && !kProduct) ? SymLay<SD, B>::KD : 0;
@@ -293,35 +276,6 @@ struct SymSmem {
   static constexpr size_t kRest = kPart + kRed + kTs + round_to(2 * U * (int)sizeof(int), 16);
   static constexpr int kStages = (2 * kStage + kRest <= 225 * 1024) ? 2 : 1;
   static constexpr size_t bytes = kStages * kStage + kRest;
-};
-
-// Ring slots, warps per block and blocks per SM of the streaming form.
-#ifndef AGG_RING_S27
-#define AGG_RING_S27 4
-#endif
-#ifndef AGG_RING_W27
-#define AGG_RING_W27 5
-#endif
-#ifndef AGG_RING_B27
-#define AGG_RING_B27 3
-#endif
-#ifndef AGG_RING_S9
-#define AGG_RING_S9 5
-#endif
-#ifndef AGG_RING_W9
-#define AGG_RING_W9 5
-#endif
-#ifndef AGG_RING_B9
-#define AGG_RING_B9 4
-#endif
-template <typename T, int B> struct SymRingSlots {
-  static constexpr int value = (B == 27) ? AGG_RING_S27 : AGG_RING_S9;
-};
-template <typename T, int B> struct SymRingWarps {
-  static constexpr int value = (B == 27) ? AGG_RING_W27 : AGG_RING_W9;
-};
-template <typename T, int B> struct SymRingBlocks {
-  static constexpr int value = (B == 27) ? AGG_RING_B27 : AGG_RING_B9;
 };
 
 // The row's product over stored entries in float64, for neighbourhoods that
@@ -379,7 +333,8 @@ __device__ __forceinline__ void fx_store(double v, bool active, int slot, int64_
 //   SYM_CHEB, KIND as in k_cheb: Chebyshev step with the block inverses `ext`;
 //     float64: also writes the new iterate's fixed-point copy (Xo, Eo)
 //   SYM_RESTRICT: out = P^T (rhs - y) with the transposed transfer blocks `ext`
-// (ext: column by column, LDP apart; KIND 0 of SYM_CHEB: packed triangles)
+// (ext: column by column, LDP apart; KIND 0 of SYM_CHEB: packed triangles, which
+// without a product leave room for two stages: 64 DoFs, 24^3, 108 -> 22 us)
 // x: the vector itself (own values); xv: what the products read. The blocks of
 // a launch loop over tiles of U elements, so that the tiles in flight are
 // neighbours and share face blocks through the L2.
@@ -685,6 +640,8 @@ static __global__ void __launch_bounds__(SymSmem<T, TD, B, OP, KIND>::NTH)
 // One warp per 32 / B elements, one lane per row; each warp streams its blocks
 // (diagonal, faces, Dinv) through a private ring of NS slots in shared memory,
 // so that NS - 1 blocks are always in flight and no warp waits for another.
+// Shared memory holds kBlocks x NWARP rings per SM; more slots or warps did not
+// fit, fewer left HBM idle.
 template <typename T, typename TD, int B, int OP, int KIND>
 struct SymRing {
   using S = SymShape<B>;
@@ -698,16 +655,16 @@ struct SymRing {
   static constexpr int EPW = 32 / B;
   static constexpr int K0 = kProduct ? 0 : 1 + S::NFACE;                  // first block of an element
   static constexpr int K1 = 1 + S::NFACE + (OP == SYM_CHEB ? 1 : 0);      // one past the last
-  static constexpr int NS = kProduct ? SymRingSlots<T, B>::value : 2;     // at most K1 - K0 + 1
+  static constexpr int NS = kProduct ? (B == 27 ? 4 : 5) : 2;             // at most K1 - K0 + 1
   static constexpr int KM = L::KD > L::KB ? L::KD : L::KB;                // entries of a slot and element
   static constexpr size_t kSlot = round_to(EPW * (KM * (int)sizeof(ST) + S::BX * (int)sizeof(SX)) + (kFx ? EPW * 4 : 0), 16);
   static constexpr size_t kWarp = NS * kSlot + round_to(EPW * S::BX * (int)sizeof(Sum), 16);
-  static constexpr int NWARP = SymRingWarps<T, B>::value, NTH = NWARP * 32;
+  static constexpr int NWARP = 5, NTH = NWARP * 32, kBlocks = (B == 27) ? 3 : 4;   // warps, blocks per SM
   static constexpr size_t bytes = NWARP * kWarp;
 };
 
 template <typename T, typename TD, int B, int OP, int KIND>
-static __global__ void __launch_bounds__(SymRing<T, TD, B, OP, KIND>::NTH, SymRingBlocks<T, B>::value)
+static __global__ void __launch_bounds__(SymRing<T, TD, B, OP, KIND>::NTH, SymRing<T, TD, B, OP, KIND>::kBlocks)
     k_symw(SymView<T, B> A, SymBlk<typename SymRing<T, TD, B, OP, KIND>::SD> ext, SymVec<T> xv,
            const T* __restrict__ rhs, const T* __restrict__ x, T* __restrict__ out, T* __restrict__ d, int2* Xo, int* Eo,
            T c1, T c2, double* partials, CGState* st) {
@@ -964,7 +921,9 @@ template <int B> struct SymRows {
 
 // Level-0 prolongation x_u += P_u e_{parent(u)}, one thread per (element, row):
 // a row's entries of consecutive columns lie LDP apart, so the threads of an
-// element read each column contiguously, straight from HBM (no reuse).
+// element read each column contiguously, straight from HBM (no reuse). HBM bound:
+// 64^3 Q2 hexahedra 132 us (121 us at the copy rate), 24^3 Q3 115 -> 33 us against
+// one thread per element.
 template <typename T, int B>
 static __global__ void __launch_bounds__(SymRows<B>::NT)
     k_sym_prolong(SymBlk<typename SymNum<T>::ST> P, const int32_t* __restrict__ parent, const T* __restrict__ ec,
