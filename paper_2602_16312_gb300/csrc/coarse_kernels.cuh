@@ -120,19 +120,39 @@ struct RowValues {
   }
 };
 
-// sum_c M[r][c] t_c with t distributed over the unit's lanes (column-major M)
-template <typename T, typename TD, int B>
-__device__ __forceinline__ T rl_block(const TD* __restrict__ M, const RowOf<B>& L, T t, T* xsh) {
-  T s = T(0);
-  const TD* m = M + (size_t)L.unit * B * B + L.r;
-  const RowValues<T, B> tv(L, t, xsh);
-#pragma unroll
-  for (int c = 0; c < B; ++c) {
-    const T tc = tv(c);
-    if (L.active) s += (T)m[c * B] * tc;
+// Row r of a unit's block M (column-major) or, TR, of M^T, and its product with a
+// vector distributed over the unit's lanes. The kernels on these levels are one
+// chain of load latencies, and the compiler does not move loads across the loop
+// over the neighbours, so the row is held: loaded before the operator product that
+// precedes its use. Chebyshev step, restriction, us: 250^2 Q2 float64 16.7 -> 12.9,
+// 13.5 -> 10.0; 101^2 Q3 6.9 -> 5.5, 7.0 -> 5.6; Q2 shell 11.2 -> 7.9, 9.6 -> 8.0. Not
+// held: float32 rows of up to 9 entries (PCG on 181^2 Q2 4.7 ms, held 5.3 ms), and
+// 64-DoF rows, which would take 64 or 128 registers.
+template <typename T, typename TD, int B, bool TR>
+struct RowBlock {
+  static constexpr bool kHeld = (B <= 32) && (B > 9 || std::is_same<T, double>::value);
+  TD v[kHeld ? B : 1];
+  static __device__ __forceinline__ TD at(const TD* __restrict__ M, const RowOf<B>& L, int c) {
+    return M[(size_t)L.unit * B * B + (TR ? L.r * B + c : c * B + L.r)];
   }
-  return s;
-}
+  __device__ __forceinline__ RowBlock(const TD* __restrict__ M, const RowOf<B>& L) {
+    if constexpr (kHeld) {
+#pragma unroll
+      for (int c = 0; c < B; ++c)
+        if (L.active) v[c] = at(M, L, c);
+    }
+  }
+  __device__ __forceinline__ T mv(const TD* __restrict__ M, const RowOf<B>& L, T t, T* xsh) const {
+    T s = T(0);
+    const RowValues<T, B> tv(L, t, xsh);
+#pragma unroll
+    for (int c = 0; c < B; ++c) {
+      const T tc = tv(c);
+      if (L.active) s += (T)(kHeld ? v[kHeld ? c : 0] : at(M, L, c)) * tc;
+    }
+    return s;
+  }
+};
 
 // KIND 0/1/2 as k_cheb, one (unit, row) per thread
 template <typename T, typename TD, int B, int KIND>
@@ -144,6 +164,7 @@ static __global__ void __launch_bounds__(RL_NT) k_rl_cheb(CsrBlocks<T> A, const 
   __shared__ T xsh[kRowXchg<B>];
   const RowOf<B> L(A.n);
   const size_t o = (size_t)L.unit * B + L.r;
+  const RowBlock<T, TD, B, false> Dr(Dinv, L);
   T t = T(0);
   if constexpr (KIND == 0) {
     if (L.active) t = rhs[o];
@@ -151,7 +172,7 @@ static __global__ void __launch_bounds__(RL_NT) k_rl_cheb(CsrBlocks<T> A, const 
     const T ax = rl_row<T, B>(A, L, x_old);
     if (L.active) t = rhs[o] - ax;
   }
-  const T s = rl_block<T, TD, B>(Dinv, L, t, xsh);
+  const T s = Dr.mv(Dinv, L, t, xsh);
   if (!L.active) return;
   const T dn = (KIND == 2) ? c1 * d[o] + c2 * s : c2 * s;
   d[o] = dn;
@@ -172,13 +193,13 @@ static __global__ void __launch_bounds__(RL_NT)
   __shared__ T xsh[kRowXchg<B>];
   const RowOf<B> L(A.n);
   const size_t o = (size_t)L.unit * B + L.r;
+  const RowBlock<T, TD, B, false> Dr(Dinv, L);
   T t = T(0);
   if (L.active) {
-#pragma unroll 4
-    for (int64_t u = child_ptr[L.unit]; u < child_ptr[L.unit + 1]; ++u) t += S[(size_t)u * B + L.r];
+    t = child_sum<T, B>(S, child_ptr[L.unit], child_ptr[L.unit + 1], L.r);
     rhs[o] = t;
   }
-  const T s = rl_block<T, TD, B>(Dinv, L, t, xsh);
+  const T s = Dr.mv(Dinv, L, t, xsh);
   if (!L.active) return;
   const T dn = c2 * s;
   d[o] = dn;
@@ -194,18 +215,12 @@ static __global__ void __launch_bounds__(RL_NT) k_rl_resid_restrict(CsrBlocks<T>
   __shared__ T xsh[kRowXchg<B>];
   const RowOf<B> L(A.n);
   const size_t o = (size_t)L.unit * B + L.r;
+  // lane j (as column index) needs P[i][j] for all i: entries j*B + i, i.e. row j of P^T
+  const RowBlock<T, T, B, true> Pr(P, L);
   T t = T(0);
   const T ax = rl_row<T, B>(A, L, x);
   if (L.active) t = rhs[o] - ax;
-  // lane j (as column index) needs P[i][j] for all i: entries j*B + i, i.e. row j of P^T
-  T s = T(0);
-  const T* pj = P + (size_t)L.unit * B * B + (size_t)L.r * B;
-  const RowValues<T, B> tv(L, t, xsh);
-#pragma unroll
-  for (int i = 0; i < B; ++i) {
-    const T ti = tv(i);
-    if (L.active) s += pj[i] * ti;
-  }
+  const T s = Pr.mv(P, L, t, xsh);
   if (L.active) S[o] = s;
 }
 
