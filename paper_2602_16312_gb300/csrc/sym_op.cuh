@@ -28,7 +28,7 @@
 //   float64 product, 64^3 Q2 hexahedra: 1,483 -> 990 us (3.3 GB; HBM bound 490 us,
 //     the multiply-adds of three integer products per entry take the rest)
 //   float64 product, 24^3 Q3 hexahedra: 1,340 -> 272 us
-//   float64 smoothing step, 18^3 Q3 hexahedra: 1,475 -> 200 us with one stage
+//   float64 smoothing step, 18^3 Q3 hexahedra: 1,475 -> 163 us (one stage: 200 us)
 //
 // Float64 products run on the integer pipe. GB300 issues 2 float64 FMAs per
 // SM and clock against 64 32-bit integer multiply-adds, so a float64 block
