@@ -229,11 +229,15 @@ agg_status agg_vcycle_apply(agg_hier_t hier, const double* r_dev, double* z_dev,
  * (same operator, same kernels, same results), for callers that must not
  * allocate device memory at the time of the call, such as an embedding that
  * fixes its device-memory budget at start-up.
- * It has no counterpart in the paper: it only changes where the two
- * temporary, unit-permuted copies of x and y live.
+ * It has no counterpart in the paper: it only changes where the temporary,
+ * unit-permuted copies of x and y and the fixed-point copy of x (products of
+ * level 0 with 16 and more DoFs per element) live. No work buffer of the
+ * hierarchy is written: the call may overlap, on another stream, a call that
+ * uses those (agg_operator_apply, a V-cycle, a solve).
  *
- * Scratch: one file-scope device array of 2 x AGG_STATIC_APPLY_MAX_ENTRIES
- * doubles (16 MiB), which every GPU that loads the library holds until the
+ * Scratch: one file-scope device array of 24.25 MiB (two vectors of
+ * AGG_STATIC_APPLY_MAX_ENTRIES doubles, a fixed-point vector and an exponent
+ * per element), which every GPU that loads the library holds until the
  * process exits. The call calls no cudaMalloc, cudaFree or other allocating
  * routine. Levels 0 .. n_levels-2 only; a level whose padded vector length
  * ((units rounded up to 32) * (p+1)^d) exceeds AGG_STATIC_APPLY_MAX_ENTRIES

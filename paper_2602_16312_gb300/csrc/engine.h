@@ -62,10 +62,12 @@ class EngineBase {
   virtual void launch_counts(int& per_vcycle, int& per_iteration, int& per_setup, int& persistent,
                              int& cluster_level, int& cluster_ctas) const = 0;
   // y = A_l x with the permuted copies of x and y in caller-provided device
-  // scratch (s_in, s_out: at least level_scratch_entries(l) doubles each)
+  // scratch (s_in, s_out: at least level_scratch_entries(l) doubles each; s_fx,
+  // for the fixed-point copy of x that products with 16 and more DoFs per unit
+  // make: 8 bytes per entry and 4 per unit)
   virtual int64_t level_scratch_entries(int level) const = 0;
   virtual int apply_level_scratch(int level, const double* x_user, double* y_user, void* s_in, void* s_out,
-                                  cudaStream_t s, std::string& err) = 0;
+                                  void* s_fx, cudaStream_t s, std::string& err) = 0;
 };
 
 EngineBase* make_engine(int B, int precision);

@@ -674,12 +674,12 @@ class Engine : public EngineBase {
                                                             partials_ + kPQ, st);
     }
   }
-  // Float64 level-0 product (MODE as in k_spmv)
+  // Float64 level-0 product (MODE as in k_spmv); fx: where x's fixed-point copy goes
   template <int MODE>
-  void spmv0(const double* x, const double* rhs, double* y, CGState* st, cudaStream_t s) {
+  void spmv0(const double* x, const double* rhs, double* y, FxVec fx, CGState* st, cudaStream_t s) {
     if (osym_) {
-      if (MODE != 2) make_fx(x, fxp_, st, s);        // MODE 2: written with p
-      launch_sym<SYM_SPMV, MODE, double, double>(MODE, A0s_, SymBlk<int2>{}, SymVec<double>{fxp_.X, fxp_.E}, rhs, x, y,
+      if (MODE != 2) make_fx(x, fx, st, s);          // MODE 2: written with p
+      launch_sym<SYM_SPMV, MODE, double, double>(MODE, A0s_, SymBlk<int2>{}, SymVec<double>{fx.X, fx.E}, rhs, x, y,
                                                  nullptr, FxVec{}, 0.0, 0.0, st, s);
     }
     else
@@ -1061,14 +1061,14 @@ class Engine : public EngineBase {
 
   void launch_init(cudaStream_t s, unsigned long long cond, int use_cond) {
     k_cg_begin<<<1, 1, 0, s>>>(st_, cond, use_cond, persist_ ? bar_ : nullptr);
-    spmv0<1>(x_, b_, r_, nullptr, s);
+    spmv0<1>(x_, b_, r_, fxp_, nullptr, s);
     k_r0<<<red_grid(N0()), RED_NT, 0, s>>>(r_, N0(), partials_ + kRR, st_);
     launch_precond(s, true);
     k_loop_ctl<<<1, 1, 0, s>>>(st_);
   }
 
   void launch_body(cudaStream_t s) {
-    spmv0<2>(p_, nullptr, q_, st_, s);
+    spmv0<2>(p_, nullptr, q_, fxp_, st_, s);
     k_cg_update<T><<<red_grid(N0()), RED_NT, 0, s>>>(x_, r_, p_, q_, std::is_same<T, double>::value ? nullptr : r32_,
                                                      vcycle_result(), N0(), partials_ + kPQ, pq_blocks(), partials_ + kRR,
                                                      partials_ + kRZ + kPartials, st_);
@@ -1490,7 +1490,7 @@ class Engine : public EngineBase {
       if (use_mf0())
         k_op_apply<T, B, MfOpT><<<bgrid(0, v.nsl), NTB, 0, s>>>(mfop_, v.xa, v.xb);
       else if (std::is_same<T, double>::value)
-        spmv0<0>(reinterpret_cast<const double*>(v.xa), nullptr, reinterpret_cast<double*>(v.xb), nullptr, s);
+        spmv0<0>(reinterpret_cast<const double*>(v.xa), nullptr, reinterpret_cast<double*>(v.xb), fxa_, nullptr, s);
       else if (sym_)
         launch_sym<SYM_SPMV, 0, T, TD>(3, fs_, SymBlk<typename SymNum<T>::ST>{}, sym_vec(v.xa), nullptr, v.xa, v.xb, nullptr,
                                        FxVec{}, T(0), T(0), nullptr, s);
@@ -1519,7 +1519,7 @@ class Engine : public EngineBase {
     const int64_t g = cdiv(v.n * B, 256);
     if (l == 0) {
       k_gather_units<double, double><<<g, 256, 0, s>>>(x_user, p_, v.perm, v.n, B);
-      spmv0<0>(p_, nullptr, q_, nullptr, s);
+      spmv0<0>(p_, nullptr, q_, fxp_, nullptr, s);
       k_scatter_units<double, double><<<g, 256, 0, s>>>(q_, y_user, v.perm, v.n, B);
     } else {
       if (l == nlev_ - 1) { err = "the coarsest level is applied through its Cholesky factor only"; return AGG_EUNSUPPORTED; }
@@ -1549,8 +1549,9 @@ class Engine : public EngineBase {
     return lev_[l].nvec;
   }
 
-  int apply_level_scratch(int l, const double* x_user, double* y_user, void* s_in, void* s_out, cudaStream_t s,
-                          std::string& err) override {
+  // s_fx: the fixed-point copy of x, its entries and then an exponent per unit
+  int apply_level_scratch(int l, const double* x_user, double* y_user, void* s_in, void* s_out, void* s_fx,
+                          cudaStream_t s, std::string& err) override {
     if (l < 0 || l >= nlev_ - 1) { err = "level out of range (the coarsest level has no stored operator)"; return AGG_EINVAL; }
     Lev& v = lev_[l];
     const int64_t g = cdiv(v.n * B, 256);
@@ -1558,7 +1559,8 @@ class Engine : public EngineBase {
       double* xi = static_cast<double*>(s_in);
       double* yi = static_cast<double*>(s_out);
       k_gather_units<double, double><<<g, 256, 0, s>>>(x_user, xi, v.perm, v.n, B);
-      spmv0<0>(xi, nullptr, yi, nullptr, s);
+      spmv0<0>(xi, nullptr, yi, FxVec{static_cast<int2*>(s_fx), reinterpret_cast<int*>(static_cast<int2*>(s_fx) + v.nvec)},
+               nullptr, s);
       k_scatter_units<double, double><<<g, 256, 0, s>>>(yi, y_user, v.perm, v.n, B);
     } else {
       T* xi = static_cast<T*>(s_in);
@@ -1632,7 +1634,7 @@ class Engine : public EngineBase {
       const IonicParams ip = make_ionic(sp_.model, sp_.k, sp_.a, sp_.eps, sp_.gamma, sp_.mu1, sp_.mu2, sp_.bo);
       const double c = 1.5 * sp_.chi * sp_.cm / sp_.dt;
       const double ia = (clock < sp_.iapp_steps) ? sp_.iapp_value : 0.0;
-      spmv0<0>(x_, nullptr, q_, nullptr, s);
+      spmv0<0>(x_, nullptr, q_, fxp_, nullptr, s);
       k_bdf2_start<B><<<cdiv(v0.n, ElemRows<B>::U), ElemRows<B>::NT, 0, s>>>(Minv_, q_, x_, w_, mask_, up_, wp_, ip, sp_.dt,
                                                                              sp_.chi, sp_.cm, c, ia, v0.n, N0());
       hist_valid_ = true;
@@ -1683,7 +1685,7 @@ class Engine : public EngineBase {
     for (int i = 0; i < reps; ++i) {
       switch (id) {
         case 0:
-          spmv0<0>(p_, nullptr, q_, nullptr, s);
+          spmv0<0>(p_, nullptr, q_, fxp_, nullptr, s);
           break;
         case 1:
           if (use_mf0())

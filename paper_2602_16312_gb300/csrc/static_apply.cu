@@ -1,7 +1,9 @@
 // agg_operator_apply_static: the level-operator product of agg_operator_apply
 // for callers that must not allocate device memory. The two unit-permuted
-// work vectors live in one file-scope device array instead of the
-// hierarchy's work buffers; the entry point itself calls no allocator.
+// work vectors and the fixed-point copy of x that the float64 product of
+// level 0 reads (engine_impl.cuh, spmv0) live in one file-scope device array;
+// nothing of the hierarchy's own work buffers is written, so that a call may
+// overlap one that works in those. The entry point itself calls no allocator.
 #include <cuda_runtime.h>
 
 #include <mutex>
@@ -13,9 +15,12 @@
 
 namespace {
 
-// Two vectors of up to AGG_STATIC_APPLY_MAX_ENTRIES doubles each (16 MiB in
-// total), held by every GPU that loads the library until the process exits.
-static __device__ __align__(256) double g_static_apply_scratch[2 * AGG_STATIC_APPLY_MAX_ENTRIES];
+// Two vectors of up to AGG_STATIC_APPLY_MAX_ENTRIES doubles each, the fixed-point
+// copy's entries (8 bytes each) and its exponents (4 bytes per unit; units of 16
+// and more entries have them), 24.25 MiB in total, held by every GPU that loads the
+// library until the process exits.
+constexpr int64_t kFxDoubles = AGG_STATIC_APPLY_MAX_ENTRIES + AGG_STATIC_APPLY_MAX_ENTRIES / 32;
+static __device__ __align__(256) double g_static_apply_scratch[2 * AGG_STATIC_APPLY_MAX_ENTRIES + kFxDoubles];
 
 constexpr int kMaxDevices = 64;
 std::mutex g_mu;
@@ -76,8 +81,9 @@ extern "C" agg_status agg_operator_apply_static(agg_hier_t h, int level, const d
   if (s) return s;
   double* s_in = static_cast<double*>(base);
   double* s_out = s_in + AGG_STATIC_APPLY_MAX_ENTRIES;
+  double* s_fx = s_out + AGG_STATIC_APPLY_MAX_ENTRIES;
   std::string err;
-  int rc = h->eng->apply_level_scratch(level, x, y, s_in, s_out, (cudaStream_t)stream, err);
+  int rc = h->eng->apply_level_scratch(level, x, y, s_in, s_out, s_fx, (cudaStream_t)stream, err);
   if (rc) {
     aggmg::set_last_error(err);
     return (agg_status)rc;
