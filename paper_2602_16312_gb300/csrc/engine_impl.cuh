@@ -1489,12 +1489,11 @@ class Engine : public EngineBase {
       k_gather_units<T, double><<<g, 256, 0, s>>>(x_user, v.xa, v.perm, v.n, B);
       if (use_mf0())
         k_op_apply<T, B, MfOpT><<<bgrid(0, v.nsl), NTB, 0, s>>>(mfop_, v.xa, v.xb);
-      else if (std::is_same<T, double>::value)
-        spmv0<0>(reinterpret_cast<const double*>(v.xa), nullptr, reinterpret_cast<double*>(v.xb), fxa_, nullptr, s);
-      else if (sym_)
+      else if (sym_) {
+        if constexpr (std::is_same<T, double>::value) make_fx(v.xa, fxa_, nullptr, s);
         launch_sym<SYM_SPMV, 0, T, TD>(3, fs_, SymBlk<typename SymNum<T>::ST>{}, sym_vec(v.xa), nullptr, v.xa, v.xb, nullptr,
                                        FxVec{}, T(0), T(0), nullptr, s);
-      else
+      } else
         k_op_apply<T, B, L0Op><<<bgrid(0, v.nsl), NTB, 0, s>>>(fop_, v.xa, v.xb);
       k_scatter_units<double, T><<<g, 256, 0, s>>>(v.xb, y_user, v.perm, v.n, B);
       AGG_CK(cudaGetLastError());
