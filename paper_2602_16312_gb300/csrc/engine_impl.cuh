@@ -424,65 +424,74 @@ class Engine : public EngineBase {
     return AGG_OK;
   }
 
-  // Scale exponents s_e (2^{2 s_e} >= the element's largest diagonal entry) and
-  // the global exponent kA of the scaled entries.
-  int sym_scales(const FaceBlocks& fb, int64_t n, std::vector<int16_t>& sc) const {
+  // s with 2^{2 s} >= d, the smallest such
+  static int16_t fx_half_exponent(double d) {
+    int e = 0;
+    if (d > 0.0) std::frexp(d, &e);
+    return (int16_t)(e >= 0 ? (e + 1) / 2 : -((-e) / 2));
+  }
+  // Scale exponents s_i (2^{2 s_i} >= A_ii) and the global exponent kA of the scaled
+  // entries. False if rounding them to fixed point would take more than kFxLoss of
+  // sum_j |A_ij| from some row.
+  bool sym_scales(const FaceBlocks& fb, int64_t n, std::vector<int16_t>& sc, int& kA) const {
     using S = SymShape<B>;
     using FI = FaceIdx<S::D, S::N>;
     const int nf = S::NFACE, NF = S::NF, BO = S::BO;
-    {
-      sc.assign(n, 0);
+    sc.assign((size_t)n * B, 0);
 #pragma omp parallel for schedule(static)
-      for (int64_t u = 0; u < n; ++u) {
-        double m = 0.0;
-        for (int i = 0; i < B; ++i) m = std::max(m, std::fabs(fb.diag[(size_t)u * B * B + (size_t)i * B + i]));
-        int e = 0;
-        if (m > 0.0) std::frexp(m, &e);
-        sc[u] = (int16_t)(e >= 0 ? (e + 1) / 2 : -((-e) / 2));
+    for (int64_t u = 0; u < n; ++u)
+      for (int i = 0; i < B; ++i) sc[(size_t)u * B + i] = fx_half_exponent(fb.diag[(size_t)u * B * B + (size_t)i * B + i]);
+    // calls g(i, |A_ij| 2^{-s_i}, 2^{s_j}) for the entries of element u
+    auto entries = [&](int64_t u, auto&& g) {
+      double p[B], q[B];
+      for (int i = 0; i < B; ++i) {
+        p[i] = std::ldexp(1.0, -sc[(size_t)u * B + i]);
+        q[i] = std::ldexp(1.0, sc[(size_t)u * B + i]);
       }
-      double rs = 0.0, mx = 0.0;                     // largest row sum and entry after scaling
+      for (int i = 0; i < B; ++i)
+        for (int j = 0; j < B; ++j) g(i, std::fabs(fb.diag[(size_t)u * B * B + (size_t)i * B + j]) * p[i], q[j]);
+      for (int f = 0; f < nf; ++f) {
+        const int64_t nb = fb.nbr[(size_t)u * nf + f];
+        if (nb < 0) continue;
+        const int fn = fb.code[(size_t)u * nf + f];
+        for (int i = 0; i < B; ++i) q[i] = std::ldexp(1.0, sc[(size_t)nb * B + i]);
+        const double* R = &fb.R[((size_t)u * nf + f) * NF * B];
+        const double* C = &fb.C[((size_t)u * nf + f) * BO * NF];
+        for (int j = 0; j < NF; ++j) {
+          const int i = FI::face(f, j);
+          for (int c = 0; c < B; ++c) g(i, std::fabs(R[j * B + c]) * p[i], q[c]);
+        }
+        for (int j = 0; j < BO; ++j) {
+          const int i = FI::off(f, j);
+          for (int c = 0; c < NF; ++c) g(i, std::fabs(C[j * NF + c]) * p[i], q[FI::face(fn, c)]);
+        }
+      }
+    };
+    double rs = 0.0, mx = 0.0;                       // largest row sum and entry after scaling
 #pragma omp parallel for schedule(static) reduction(max : rs, mx)
-      for (int64_t u = 0; u < n; ++u) {
-        double row[B];
-        for (int i = 0; i < B; ++i) {
-          row[i] = 0.0;
-          double big = 0.0;
-          for (int j = 0; j < B; ++j) {
-            const double v = std::fabs(fb.diag[(size_t)u * B * B + (size_t)i * B + j]);
-            row[i] += v;
-            big = std::max(big, v);
-          }
-          row[i] = std::ldexp(row[i], -2 * sc[u]);
-          mx = std::max(mx, std::ldexp(big, -2 * sc[u]));
-        }
-        for (int f = 0; f < nf; ++f) {
-          const int64_t nb = fb.nbr[(size_t)u * nf + f];
-          if (nb < 0) continue;
-          for (int j = 0; j < NF; ++j) {
-            double a = 0.0, big = 0.0;
-            for (int c = 0; c < B; ++c) {
-              const double v = std::fabs(fb.R[((size_t)u * nf + f) * NF * B + (size_t)j * B + c]);
-              a += v;
-              big = std::max(big, v);
-            }
-            row[FI::face(f, j)] += std::ldexp(a, -sc[u] - sc[nb]);
-            mx = std::max(mx, std::ldexp(big, -sc[u] - sc[nb]));
-          }
-          for (int j = 0; j < BO; ++j) {
-            double a = 0.0, big = 0.0;
-            for (int c = 0; c < NF; ++c) {
-              const double v = std::fabs(fb.C[((size_t)u * nf + f) * BO * NF + (size_t)j * NF + c]);
-              a += v;
-              big = std::max(big, v);
-            }
-            row[FI::off(f, j)] += std::ldexp(a, -sc[u] - sc[nb]);
-            mx = std::max(mx, std::ldexp(big, -sc[u] - sc[nb]));
-          }
-        }
-        for (int i = 0; i < B; ++i) rs = std::max(rs, row[i]);
-      }
-      return fx_exponent(rs, mx);
+    for (int64_t u = 0; u < n; ++u) {
+      double row[B] = {};
+      entries(u, [&](int i, double a, double q) {
+        row[i] += a / q;
+        mx = std::max(mx, a / q);
+      });
+      for (int i = 0; i < B; ++i) rs = std::max(rs, row[i]);
     }
+    if (!(rs > 0.0)) return false;
+    kA = fx_exponent(rs, mx);
+    const double unit = std::ldexp(1.0, kA);
+    int bad = 0;
+#pragma omp parallel for schedule(static) reduction(+ : bad)
+    for (int64_t u = 0; u < n; ++u) {
+      double lost[B] = {}, sum[B] = {};              // of row i, both times 2^{kA - s_i}
+      entries(u, [&](int i, double a, double q) {
+        const double w = a / q * unit;
+        lost[i] += std::fabs(w - std::rint(w)) * q;
+        sum[i] += a * unit;
+      });
+      for (int i = 0; i < B; ++i) bad += !(lost[i] <= kFxLoss * sum[i]);
+    }
+    return bad == 0;
   }
   // exponent that takes row sums to at most 2^FX_A and entries to at most 2^FX_AE
   static int fx_exponent(double rowsum, double entry) {
@@ -491,7 +500,8 @@ class Engine : public EngineBase {
   }
 
   template <typename TS>
-  int upload_sym(const FaceBlocks& fb, int64_t n, SymView<TS, B>& view, std::string& err) {
+  int upload_sym(const FaceBlocks& fb, int64_t n, const std::vector<int16_t>& sc, int kA, SymView<TS, B>& view,
+                 std::string& err) {
     using S = SymShape<B>;
     using FI = FaceIdx<S::D, S::N>;
     using ST = typename SymNum<TS>::ST;
@@ -503,17 +513,15 @@ class Engine : public EngineBase {
     std::vector<int2> info;
     if ((rc = sym_faces(fb, n, info, nblk, err))) return rc;
     std::vector<int8_t> code(fb.code.begin(), fb.code.end());
-    std::vector<int16_t> sc;
-    const int kA = kFx ? sym_scales(fb, n, sc) : 0;
     std::vector<ST> hd((size_t)n * L::KD, ST{}), hf((size_t)nblk * L::KB, ST{});
 #pragma omp parallel for schedule(static)
     for (int64_t u = 0; u < n; ++u) {
       const double* D = &fb.diag[(size_t)u * B * B];
       ST* d = &hd[(size_t)u * L::KD];
-      const int su = kFx ? sc[u] : 0;
+      auto scale = [&](int64_t e, int i) { return kFx ? (int)sc[(size_t)e * B + i] : 0; };
       for (int i = 0; i < B; ++i)
         for (int j = 0; j <= i; ++j)
-          d[i * (i + 1) / 2 + j] = sym_entry<ST>(0.5 * (D[i * B + j] + D[j * B + i]), kA - 2 * su);
+          d[i * (i + 1) / 2 + j] = sym_entry<ST>(0.5 * (D[i * B + j] + D[j * B + i]), kA - scale(u, i) - scale(u, j));
       for (int f = 0; f < nf; ++f) {
         const int64_t nb = info[(size_t)u * nf + f].x;
         if (nb < u) continue;                        // none, or stored by the neighbour
@@ -522,13 +530,15 @@ class Engine : public EngineBase {
         const double* C = &fb.C[((size_t)u * nf + f) * BO * NF];
         ST* F = &hf[(size_t)info[(size_t)u * nf + f].y * L::KB];
         ST* G = F + NF * S::LDF;
-        const int k = kFx ? kA - su - sc[nb] : 0;
         for (int c = 0; c < NF; ++c) {
-          for (int j = 0; j < NF; ++j) F[c * S::LDF + j] = sym_entry<ST>(R[j * B + FI::face(fn, c)], k);
-          for (int j = 0; j < BO; ++j) F[c * S::LDF + NF + j] = sym_entry<ST>(C[j * NF + c], k);
+          const int k = kA - scale(nb, FI::face(fn, c));
+          for (int j = 0; j < NF; ++j) F[c * S::LDF + j] = sym_entry<ST>(R[j * B + FI::face(fn, c)], k - scale(u, FI::face(f, j)));
+          for (int j = 0; j < BO; ++j) F[c * S::LDF + NF + j] = sym_entry<ST>(C[j * NF + c], k - scale(u, FI::off(f, j)));
         }
-        for (int c = 0; c < BO; ++c)
-          for (int j = 0; j < NF; ++j) G[c * S::LDG + j] = sym_entry<ST>(R[j * B + FI::off(fn, c)], k);
+        for (int c = 0; c < BO; ++c) {
+          const int k = kA - scale(nb, FI::off(fn, c));
+          for (int j = 0; j < NF; ++j) G[c * S::LDG + j] = sym_entry<ST>(R[j * B + FI::off(fn, c)], k - scale(u, FI::face(f, j)));
+        }
       }
     }
     ST *dd, *df;
@@ -544,20 +554,6 @@ class Engine : public EngineBase {
     return AGG_OK;
   }
 
-  // fixed-point exponent of a B x B block (used by rows and by columns)
-  static int fx_block_exponent(const double* m) {
-    double rs = 0.0, mx = 0.0;
-    for (int i = 0; i < B; ++i) {
-      double a = 0.0, b = 0.0;
-      for (int j = 0; j < B; ++j) {
-        a += std::fabs(m[i * B + j]);
-        b += std::fabs(m[j * B + i]);
-        mx = std::max(mx, std::fabs(m[i * B + j]));
-      }
-      rs = std::max(rs, std::max(a, b));
-    }
-    return fx_exponent(rs, mx);
-  }
   int alloc_fx(FxVec& v, std::string& err) {
     int rc = dalloc(&v.X, lev_[0].nvec, err);
     return rc ? rc : dalloc(&v.E, lev_[0].nsl * SL, err);
@@ -573,39 +569,73 @@ class Engine : public EngineBase {
     else return SymVec<T>{x, nullptr};
   }
 
-  // smoother block inverses (TRI) or transfer blocks of level 0, one per
-  // element; the float64 V-cycle keeps them in fixed point
+  // Scale exponents (2^{2 s_i} >= m_ii) and exponents of the SPD blocks m for fixed
+  // point, as sym_scales; false if one cannot take it.
+  static bool block_scales(const std::vector<double>& blk, int64_t n, std::vector<int16_t>& hs, std::vector<int16_t>& hk) {
+    hs.assign((size_t)n * B, 0);
+    hk.assign(n, 0);
+    int bad = 0;
+#pragma omp parallel for schedule(static) reduction(+ : bad)
+    for (int64_t u = 0; u < n; ++u) {
+      const double* m = &blk[(size_t)u * B * B];
+      int16_t* s = &hs[(size_t)u * B];
+      for (int i = 0; i < B; ++i) s[i] = fx_half_exponent(m[i * B + i]);
+      double rs = 0.0, mx = 0.0, w[B * B];
+      for (int i = 0; i < B; ++i) {
+        double row = 0.0;
+        for (int j = 0; j < B; ++j) {
+          w[i * B + j] = std::ldexp(std::fabs(0.5 * (m[i * B + j] + m[j * B + i])), -s[i] - s[j]);
+          row += w[i * B + j];
+          mx = std::max(mx, w[i * B + j]);
+        }
+        rs = std::max(rs, row);
+      }
+      if (!(rs > 0.0)) { bad += 1; continue; }
+      hk[u] = (int16_t)fx_exponent(rs, mx);
+      const double unit = std::ldexp(1.0, hk[u]);
+      for (int i = 0; i < B; ++i) {
+        double lost = 0.0, sum = 0.0;
+        for (int j = 0; j < B; ++j) {
+          const double v = w[i * B + j] * unit, q = std::ldexp(1.0, s[j] - s[i]);
+          lost += std::fabs(v - std::rint(v)) * q;
+          sum += v * q;
+        }
+        bad += !(lost <= kFxLoss * sum);
+      }
+    }
+    return bad == 0;
+  }
+
+  // smoother block inverses (TRI) or transfer blocks of level 0, one per element
+  // (hs, hk: scales of fixed-point entries)
   template <bool TRI, bool ROWS = false, typename ST>
-  int upload_sym_blocks(const std::vector<double>& blk, int64_t n, SymBlk<ST>& out, std::string& err) {
+  int upload_sym_blocks(const std::vector<double>& blk, int64_t n, SymBlk<ST>& out, std::string& err,
+                        const std::vector<int16_t>& hs = {}, const std::vector<int16_t>& hk = {}) {
     using S = SymShape<B>;
     constexpr bool kFx = std::is_same<ST, int2>::value;
     constexpr int K = TRI ? SymLay<ST, B>::KD : SymLay<ST, B>::KP;
     std::vector<ST> hv((size_t)n * K, ST{});
-    std::vector<int16_t> hk(kFx ? n : 0, 0);
 #pragma omp parallel for schedule(static)
     for (int64_t u = 0; u < n; ++u) {
       const double* m = &blk[(size_t)u * B * B];
       ST* o = &hv[(size_t)u * K];
-      int k = 0;
-      if (kFx) {
-        k = fx_block_exponent(m);
-        hk[u] = (int16_t)k;
-      }
+      auto k = [&](int i, int j) { return kFx ? hk[u] - hs[(size_t)u * B + i] - hs[(size_t)u * B + j] : 0; };
       for (int i = 0; i < B; ++i)
         for (int j = 0; j < B; ++j) {
+          const double v = kFx ? 0.5 * (m[i * B + j] + m[j * B + i]) : m[i * B + j];
           if (TRI) {
-            if (j <= i) o[i * (i + 1) / 2 + j] = sym_entry<ST>(0.5 * (m[i * B + j] + m[j * B + i]), k);
+            if (j <= i) o[i * (i + 1) / 2 + j] = sym_entry<ST>(0.5 * (m[i * B + j] + m[j * B + i]), k(i, j));
           } else {
-            o[ROWS ? i * S::LDP + j : j * S::LDP + i] = sym_entry<ST>(m[i * B + j], k);
+            o[ROWS ? i * S::LDP + j : j * S::LDP + i] = sym_entry<ST>(v, k(i, j));
           }
         }
     }
     ST* dv;
-    int16_t* dk = nullptr;
+    int16_t *dk = nullptr, *ds = nullptr;
     int rc;
     if ((rc = upload(&dv, hv.data(), hv.size(), err))) return rc;
-    if (kFx && (rc = upload(&dk, hk.data(), hk.size(), err))) return rc;
-    out = SymBlk<ST>{dv, dk};
+    if (kFx && ((rc = upload(&dk, hk.data(), hk.size(), err)) || (rc = upload(&ds, hs.data(), hs.size(), err)))) return rc;
+    out = SymBlk<ST>{dv, dk, ds};
     return AGG_OK;
   }
 
@@ -679,7 +709,7 @@ class Engine : public EngineBase {
   void spmv0(const double* x, const double* rhs, double* y, FxVec fx, CGState* st, cudaStream_t s) {
     if (osym_) {
       if (MODE != 2) make_fx(x, fx, st, s);          // MODE 2: written with p
-      launch_sym<SYM_SPMV, MODE, double, double>(MODE, A0s_, SymBlk<int2>{}, SymVec<double>{fx.X, fx.E}, rhs, x, y,
+      launch_sym<SYM_SPMV, MODE, double, double>(MODE, A0s_, SymBlk<double>{}, SymVec<double>{fx.X, fx.E}, rhs, x, y,
                                                  nullptr, FxVec{}, 0.0, 0.0, st, s);
     }
     else
@@ -1298,10 +1328,15 @@ class Engine : public EngineBase {
       constexpr bool kDouble = std::is_same<T, double>::value;
       const bool assembled = kDouble || fine_operator != 1;   // the V-cycle's level-0 operator
       const bool symmetric = sym_check(fb, m.ne);
-      osym_ = symmetric && kOuterSym;
+      // float64 forms: where fixed point holds the rows to a double's accuracy
+      std::vector<int16_t> sc, ds, dk;
+      int kA = 0;
+      const bool fixed = symmetric && (kOuterSym || (kCycleSym && kDouble)) && sym_scales(fb, m.ne, sc, kA);
+      osym_ = fixed && kOuterSym;
       sym_ = symmetric && kCycleSym && assembled;
+      if (kDouble) sym_ = sym_ && fixed && (nlev_ == 1 || block_scales(h.lev[0].Dinv, m.ne, ds, dk));
       if (osym_ || (sym_ && kDouble)) {
-        if ((rc = upload_sym<double>(fb, m.ne, A0s_, err))) return rc;
+        if ((rc = upload_sym<double>(fb, m.ne, sc, kA, A0s_, err))) return rc;
       }
       if (osym_ && (rc = alloc_fx(fxp_, err))) return rc;
       if (sym_) {
@@ -1309,13 +1344,13 @@ class Engine : public EngineBase {
           if ((rc = alloc_fx(fxa_, err)) || (rc = alloc_fx(fxb_, err))) return rc;
           fs_ = A0s_;
         } else {
-          if ((rc = upload_sym<T>(fb, m.ne, fs_, err))) return rc;
+          if ((rc = upload_sym<T>(fb, m.ne, {}, 0, fs_, err))) return rc;
         }
         if (nlev_ > 1) {
-          if ((rc = upload_sym_blocks<true>(h.lev[0].Dinv, m.ne, sdinv_, err))) return rc;
+          if ((rc = upload_sym_blocks<true>(h.lev[0].Dinv, m.ne, sdinv_, err, ds, dk))) return rc;
           if ((rc = upload_sym_blocks<false>(h.lev[0].P, m.ne, sP_, err))) return rc;
           if ((rc = upload_sym_blocks<false, true>(h.lev[0].P, m.ne, sPT_, err))) return rc;
-          if (!kStream && (rc = upload_sym_blocks<false>(h.lev[0].Dinv, m.ne, sdinvm_, err))) return rc;
+          if (!kStream && (rc = upload_sym_blocks<false>(h.lev[0].Dinv, m.ne, sdinvm_, err, ds, dk))) return rc;
         }
       }
       if (B >= 27 && !assembled && nlev_ > 1) {
@@ -1491,7 +1526,7 @@ class Engine : public EngineBase {
         k_op_apply<T, B, MfOpT><<<bgrid(0, v.nsl), NTB, 0, s>>>(mfop_, v.xa, v.xb);
       else if (sym_) {
         if constexpr (std::is_same<T, double>::value) make_fx(v.xa, fxa_, nullptr, s);
-        launch_sym<SYM_SPMV, 0, T, TD>(3, fs_, SymBlk<typename SymNum<T>::ST>{}, sym_vec(v.xa), nullptr, v.xa, v.xb, nullptr,
+        launch_sym<SYM_SPMV, 0, T, TD>(3, fs_, SymBlk<T>{}, sym_vec(v.xa), nullptr, v.xa, v.xb, nullptr,
                                        FxVec{}, T(0), T(0), nullptr, s);
       } else
         k_op_apply<T, B, L0Op><<<bgrid(0, v.nsl), NTB, 0, s>>>(fop_, v.xa, v.xb);

@@ -36,9 +36,17 @@
 // 60-bit fixed point and x is converted to 58-bit fixed point with one exponent
 // per element; the sum of the products is formed exactly in 64-bit integers (up
 // to the product of the low halves, 2^-60 of the row's scale) and rounded once.
-// Fixed point needs entries of one magnitude: element e's rows and columns are
-// scaled by 2^-s_e, 2^{2 s_e} >= its largest diagonal entry, after which an SPD
-// operator's entries are at most 1. An entry is a1 2^28 + a0 with |a0| <= 2^27, an
+// Fixed point needs entries of one magnitude: row and column i are scaled by 2^-s_i,
+// 2^{2 s_i} >= A_ii, after which an SPD operator has diagonal entries in (1/4, 1] and
+// no entry above 1 in any row (the scales of x and y are powers of two, added to
+// exponents: they cost nothing and round nothing). What a small entry loses is then
+// 2^-59 sqrt(A_ii A_jj), 1/64 of a double's rounding of the diagonal; the set-up
+// bounds the sum of these losses in every row and keeps the float64 form if one
+// passes kFxLoss of the row (engine_impl.cuh, sym_scales). One exponent per element
+// instead lost the ratio of its diagonal entries: worst row against 80-bit arithmetic,
+// relative to (|A| |x|)_i, Q2 shell 2.4e-15 -> 1.1e-16 (float64 sums: 6e-16), Q3 cube
+// 1.4e-15 -> 1.2e-16 (7e-16), 2D Q3 stiffness with a contrast of 1e-4 in the
+// conductivity 2.6e-13 -> 1.6e-15, there kept in float64 (3.6e-16). An entry is a1 2^28 + a0 with |a0| <= 2^27, an
 // x is x1 2^31 + x0 with |x0| <= 2^30. With sum_j |A_ij| <= 2^60, |A_ij| <= 2^58
 // (global exponent kA) and |x| <= 2^58, and T <= 304 entries in a row:
 //   hi = sum a1 x1 <= 2^32 2^27,  m1 = sum a1 x0 <= 2^32 2^30,
@@ -58,23 +66,26 @@ namespace aggmg {
 constexpr int FX_A = 60, FX_AE = 58, FX_X = 58, FX_P = 28, FX_Q = 31;
 constexpr int kFxNone = -100000;                    // below every exponent
 constexpr int kFxBad = 1 << 20;                     // marks a NaN or an infinity
+// largest loss of a fixed-point row relative to sum_j |A_ij|: 8 roundings of a double
+// (a float64 sum of the row's 135 to 700 products rounds as often as it adds)
+constexpr double kFxLoss = 8.0 / 9007199254740992.0;
 // exponent of the unit of FxAcc::sum() for x with shared biased exponent E, less E
 constexpr int kFxBias = FX_P + FX_Q - 1075 - (FX_X - 53);
 
-// biased exponent of x (1 for zero and subnormals; 2047 for NaN and Inf)
-__device__ __forceinline__ int fx_exp(double x) {
+// biased exponent of x 2^t (as of a subnormal for zero; kFxBad for NaN and Inf)
+__device__ __forceinline__ int fx_exp(double x, int t) {
   const int e = (__double2hiint(x) >> 20) & 0x7ff;
-  return e ? e : 1;
+  return e == 2047 ? kFxBad : (e ? e : 1) + t;
 }
 // x in units of 2^{E - 1075 - (FX_X - 53)} rounded to an integer (at most 2^FX_X for
-// E >= fx_exp(x)), as halves (lo, hi)
+// E >= fx_exp(x, 0)), as halves (lo, hi)
 __device__ __forceinline__ int2 fx_split(double x, int E) {
   const int h = __double2hiint(x);
   int e = (h >> 20) & 0x7ff;
   unsigned long long m = ((unsigned long long)(unsigned)(h & 0xfffff) << 32) | (unsigned)__double2loint(x);
   if (e) m |= 1ull << 52;
   else e = 1;
-  const int sh = min(E - e, 63);
+  const int sh = min(max(E - e, 0), 63);             // (below 0: E of a NaN or infinity)
   long long v = (long long)((((m << (FX_X - 52)) >> sh) + 1) >> 1);
   v = h < 0 ? -v : v;
   const int lo = ((int)v << (32 - FX_Q)) >> (32 - FX_Q);
@@ -106,23 +117,25 @@ __device__ __forceinline__ long long sum_shift(long long S, int sh) {
   return sh > 62 ? 0 : (S + (1ll << (sh - 1))) >> sh;
 }
 __device__ __forceinline__ float sum_shift(float s, int) { return s; }
-struct FlAcc {
-  float s = 0.0f;
-  __device__ __forceinline__ void fma(float a, float x) { s += a * x; }
-  using Sum = float;
-  __device__ __forceinline__ float sum() const { return s; }
+template <typename T>
+struct PlAcc {
+  T s = T(0);
+  __device__ __forceinline__ void fma(T a, T x) { s += a * x; }
+  using Sum = T;
+  __device__ __forceinline__ T sum() const { return s; }
 };
 
 // Stored entry, x entry and accumulator of a value type
 template <typename T> struct SymNum;
 template <> struct SymNum<double> { using ST = int2; using SX = int2; using SX2 = int4; using Acc = FxAcc; };
-template <> struct SymNum<float> { using ST = float; using SX = float; using SX2 = float2; using Acc = FlAcc; };
+template <> struct SymNum<float> { using ST = float; using SX = float; using SX2 = float2; using Acc = PlAcc<float>; };
 __device__ __forceinline__ int2 sx_first(int4 v) { return make_int2(v.x, v.y); }
 __device__ __forceinline__ int2 sx_second(int4 v) { return make_int2(v.z, v.w); }
 __device__ __forceinline__ float sx_first(float2 v) { return v.x; }
 __device__ __forceinline__ float sx_second(float2 v) { return v.y; }
 __device__ __forceinline__ int2 sym_val(int2 v) { return v; }
 __device__ __forceinline__ float sym_val(float v) { return v; }
+__device__ __forceinline__ double sym_val(double v) { return v; }
 __device__ __forceinline__ float sym_val(__nv_bfloat16 v) { return __bfloat162float(v); }
 
 // ---------------------------------------------------------------- layout
@@ -152,17 +165,18 @@ struct SymView {
   const ST* face;         // [face block][KB]
   const int2* info;       // [n][2d] neighbour's internal index (-1 none), face block
   const int8_t* code;     // [n][2d] neighbour's local face
-  const int16_t* sc;      // [n] scale exponents s_e (float64)
+  const int16_t* sc;      // [n][B] scale exponents s_i (float64)
   int kA;                 // global exponent of the fixed-point entries (float64)
   int64_t n;
 };
 
 // smoother block inverses (packed triangles) or transfer blocks of level 0, one
-// per element; float64: fixed point with an exponent per element
+// per element; float64 block inverses: fixed point as the operator's entries, with
+// an exponent per element and scale exponents of their own (from their diagonals)
 template <typename TS>
 struct SymBlk {
   const TS* v;
-  const int16_t* k;
+  const int16_t *k, *s;   // [n], [n][B]
 };
 
 __device__ __forceinline__ void cp_async16(void* dst, const void* src) {
@@ -232,8 +246,8 @@ __device__ __forceinline__ void sym_tri(const ST* m, int r, const typename SymNu
 enum { SYM_SPMV = 0, SYM_CHEB = 1, SYM_RESTRICT = 2 };
 
 // A vector as the kernels read it: T = double: fixed point, X[unit B + i] and one
-// exponent per element (the largest biased exponent of its x plus its scale, kFxBad
-// with a NaN or Inf); T = float: the vector itself.
+// exponent per element (the largest biased exponent of its scaled x, kFxBad with a
+// NaN or Inf); T = float: the vector itself.
 template <typename T> struct SymVec {
   const typename SymNum<T>::SX* X;
   const int* E;
@@ -251,7 +265,8 @@ struct SymSmem {
   using ST = typename SymNum<T>::ST;
   using SX = typename SymNum<T>::SX;
   using Sum = typename SymNum<T>::Acc::Sum;
-  using SD = typename std::conditional<OP != SYM_CHEB || std::is_same<T, double>::value, ST, TD>::type;
+  using SD = typename std::conditional<OP == SYM_CHEB, typename std::conditional<std::is_same<T, double>::value, ST, TD>::type, T>::type;
+  using XAcc = typename std::conditional<OP == SYM_CHEB, typename SymNum<T>::Acc, PlAcc<T>>::type;   // block inverse / transfer sums
   using L = SymLay<ST, B>;
   static constexpr bool kFx = std::is_same<T, double>::value;
   static constexpr bool kProduct = !(OP == SYM_CHEB && KIND == 0);
@@ -285,17 +300,18 @@ __device__ __noinline__ double sym_row_nonfinite(const SymView<double, B>& A, in
   using S = SymShape<B>;
   using L = SymLay<int2, B>;
   using FI = FaceIdx<S::D, S::N>;
-  const int se = A.sc[unit];
+  const int16_t* se = A.sc + (size_t)unit * B;
   double y = 0.0;
-  auto val = [&](int2 a, int s) { return scalbn((double)(((long long)a.y << FX_P) + a.x), se + s - A.kA); };
+  auto val = [&](int2 a, int s) { return scalbn((double)(((long long)a.y << FX_P) + a.x), se[r] + s - A.kA); };
   for (int c = 0; c < B; ++c) {
     const int hi = max(r, c), lo = min(r, c);
-    y += val(A.diag[(size_t)unit * L::KD + hi * (hi + 1) / 2 + lo], se) * x[(size_t)unit * B + c];
+    y += val(A.diag[(size_t)unit * L::KD + hi * (hi + 1) / 2 + lo], se[c]) * x[(size_t)unit * B + c];
   }
   for (int f = 0; f < S::NFACE; ++f) {
     const int2 nf = A.info[unit * S::NFACE + f];
     if (nf.x < 0) continue;
-    const int fn = A.code[unit * S::NFACE + f], sn = A.sc[nf.x];
+    const int fn = A.code[unit * S::NFACE + f];
+    const int16_t* sn = A.sc + (size_t)nf.x * B;
     const bool tr = nf.x < unit;
     bool on;
     const int pos = face_first<B>(f, r, on);
@@ -306,7 +322,7 @@ __device__ __noinline__ double sym_row_nonfinite(const SymView<double, B>& A, in
       const int dof = t < S::NF ? FI::face(fn, t) : FI::off(fn, t - S::NF);
       const int2 a = tr ? (on ? blk[pos * S::LDF + t] : g[(pos - S::NF) * S::LDG + t])
                         : (t < S::NF ? blk[t * S::LDF + pos] : g[(t - S::NF) * S::LDG + pos]);
-      y += val(a, sn) * xn[dof];
+      y += val(a, sn[dof]) * xn[dof];
     }
   }
   return y;
@@ -317,14 +333,15 @@ __device__ __noinline__ double sym_row_nonfinite(const SymView<double, B>& A, in
 template <int B>
 __device__ __forceinline__ void fx_store(double v, bool active, int slot, int64_t unit, int r, const int16_t* sc, int2* X,
                                          int* E, int* se, int U) {
-  if (threadIdx.x < U) se[threadIdx.x] = 1;
+  if (threadIdx.x < U) se[threadIdx.x] = kFxNone;
+  const int t = active ? sc[(size_t)unit * B + r] : 0;
   __syncthreads();
-  if (active) atomicMax(se + slot, fx_exp(v));
+  if (active) atomicMax(se + slot, fx_exp(v, t));
   __syncthreads();
   if (active) {
     const int e = se[slot];
-    X[(size_t)unit * B + r] = fx_split(v, e);
-    if (r == 0) E[unit] = e == 2047 ? kFxBad : e + sc[unit];
+    X[(size_t)unit * B + r] = fx_split(v, e - t);
+    if (r == 0) E[unit] = e;
   }
 }
 
@@ -353,7 +370,10 @@ static __global__ void __launch_bounds__(SymSmem<T, TD, B, OP, KIND>::NTH)
   using SX = typename M::SX;
   using Sum = typename M::Sum;
   using Acc = typename SymNum<T>::Acc;
+  using XAcc = typename M::XAcc;
+  using XSum = typename XAcc::Sum;
   using L = typename M::L;
+  constexpr bool kFxExt = M::kFx && OP == SYM_CHEB;   // the block inverses are in fixed point
   constexpr int U = M::U, G = M::G, NFACE = S::NFACE, BX = S::BX, NF = S::NF, BO = S::BO, N = S::N;
   constexpr bool kFx = M::kFx;
   constexpr int kShare = BO / N;                      // off-face terms of a face row per thread
@@ -469,7 +489,7 @@ static __global__ void __launch_bounds__(SymSmem<T, TD, B, OP, KIND>::NTH)
     } else {
       asm volatile("cp.async.wait_group 0;" ::: "memory");
     }
-    if (OP != SYM_SPMV && tid < 2 * U) smax[tid] = 1;
+    if (OP != SYM_SPMV && tid < 2 * U) smax[tid] = kFxNone;
     __syncthreads();
     unsigned char* base = sym_sm + sg * M::kStage;
     const ST* eb = reinterpret_cast<ST*>(base) + slot * M::KE;
@@ -477,6 +497,7 @@ static __global__ void __launch_bounds__(SymSmem<T, TD, B, OP, KIND>::NTH)
     const SX* ex = reinterpret_cast<SX*>(base + M::kBlk + M::kExt) + slot * M::NX * BX;
     const int* ee = reinterpret_cast<int*>(base + M::kBlk + M::kExt + M::kXs) + slot * M::NX;
     T own = T(0), rh = T(0), dv = T(0);               // loaded ahead of their use
+    int ti = 0, ui = 0;                               // scale exponents of the row and of its block inverse
     SD ev[M::kExtMem ? M::CPG : 1];
     if constexpr (M::kExtMem) {
       if (active) {
@@ -489,6 +510,8 @@ static __global__ void __launch_bounds__(SymSmem<T, TD, B, OP, KIND>::NTH)
       if (M::kProduct && (KIND == 2 || OP == SYM_CHEB)) own = x[o];
       if (!(OP == SYM_SPMV && KIND != 1)) rh = rhs[o];
       if (OP == SYM_CHEB && KIND == 2) dv = d[o];
+      if (kFx) ti = A.sc[o];
+      if (kFxExt) ui = ext.s[o];
     }
 
     // ---- y = (A0 x)_r
@@ -550,7 +573,7 @@ static __global__ void __launch_bounds__(SymSmem<T, TD, B, OP, KIND>::NTH)
           }
         }
         if constexpr (kFx) {
-          if (E != kFxBad) y = fx_scale(sum, A.sc[unit] - A.kA + E + kFxBias);
+          if (E != kFxBad) y = fx_scale(sum, ti - A.kA + E + kFxBias);
           else if (OP == SYM_SPMV) y = sym_row_nonfinite<B>(A, unit, r, x);
           else y = nan("");
         } else {
@@ -568,21 +591,23 @@ static __global__ void __launch_bounds__(SymSmem<T, TD, B, OP, KIND>::NTH)
       // ---- the element's residual t, then its block inverse or P^T
       const T t = rh - y;
       int Et = 0;
-      if constexpr (kFx) {
-        if (lead) atomicMax(smax + slot, fx_exp(t));
+      if constexpr (kFxExt) {
+        if (lead) atomicMax(smax + slot, fx_exp(t, ui));
         __syncthreads();
         if (lead) Et = smax[slot];
       }
-      SX* ts = sts + slot * BX;
+      using TS = typename std::conditional<OP == SYM_CHEB, SX, T>::type;
+      TS* ts = reinterpret_cast<TS*>(sts) + slot * BX;
+      XSum* xred = reinterpret_cast<XSum*>(sred);
       if (lead) {
-        if constexpr (kFx) ts[r] = fx_split(t, Et);
+        if constexpr (kFxExt) ts[r] = fx_split(t, Et - ui);
         else ts[r] = t;
       }
       __syncthreads();
       T res = T(0);
-      Sum es = Sum(0);
+      XSum es = XSum(0);
       if (active) {
-        Acc acc;
+        XAcc acc;
         if constexpr (M::kExtMem) {
 #pragma unroll
           for (int c = 0; c < M::CPG; ++c) acc.fma(sym_val(ev[c]), ts[g * M::CPG + c]);
@@ -590,14 +615,14 @@ static __global__ void __launch_bounds__(SymSmem<T, TD, B, OP, KIND>::NTH)
           sym_tri<T, B>(sext, r, ts, acc);
         }
         es = acc.sum();
-        if (G > 1 && g > 0) sred[(g - 1) * U * B + slot * B + r] = es;
+        if (G > 1 && g > 0) xred[(g - 1) * U * B + slot * B + r] = es;
       }
       if (G > 1) __syncthreads();
       if (lead) {
 #pragma unroll
-        for (int k = 0; k < G - 1; ++k) es += sred[k * U * B + slot * B + r];
+        for (int k = 0; k < G - 1; ++k) es += xred[k * U * B + slot * B + r];
         T sv;
-        if constexpr (kFx) sv = Et == 2047 ? nan("") : fx_scale(es, Et + kFxBias - ext.k[unit]);
+        if constexpr (kFxExt) sv = Et == kFxBad ? nan("") : fx_scale(es, ui + Et + kFxBias - ext.k[unit]);
         else sv = es;
         if constexpr (OP == SYM_RESTRICT) {
           out[o] = sv;
@@ -609,12 +634,12 @@ static __global__ void __launch_bounds__(SymSmem<T, TD, B, OP, KIND>::NTH)
         }
       }
       if constexpr (kFx && OP == SYM_CHEB) {
-        if (lead) atomicMax(smax + U + slot, fx_exp(res));
+        if (lead) atomicMax(smax + U + slot, fx_exp(res, ti));
         __syncthreads();
         if (lead) {
           const int e = smax[U + slot];
-          Xo[o] = fx_split(res, e);
-          if (r == 0) Eo[unit] = e == 2047 ? kFxBad : e + A.sc[unit];
+          Xo[o] = fx_split(res, e - ti);
+          if (r == 0) Eo[unit] = e;
         }
       }
     }
@@ -648,7 +673,8 @@ struct SymRing {
   using ST = typename SymNum<T>::ST;
   using SX = typename SymNum<T>::SX;
   using Sum = typename SymNum<T>::Acc::Sum;
-  using SD = typename std::conditional<OP != SYM_CHEB || std::is_same<T, double>::value, ST, TD>::type;
+  using SD = typename std::conditional<OP == SYM_CHEB, typename std::conditional<std::is_same<T, double>::value, ST, TD>::type, T>::type;
+  using XAcc = typename std::conditional<OP == SYM_CHEB, typename SymNum<T>::Acc, PlAcc<T>>::type;   // block inverse / transfer sums
   using L = SymLay<ST, B>;
   static constexpr bool kFx = std::is_same<T, double>::value;
   static constexpr bool kProduct = !(OP == SYM_CHEB && KIND == 0);
@@ -675,7 +701,9 @@ static __global__ void __launch_bounds__(SymRing<T, TD, B, OP, KIND>::NTH, SymRi
   using SX = typename M::SX;
   using Sum = typename M::Sum;
   using Acc = typename SymNum<T>::Acc;
+  using XAcc = typename M::XAcc;
   using L = typename M::L;
+  constexpr bool kFxExt = M::kFx && OP == SYM_CHEB;   // the block inverses are in fixed point
   constexpr int EPW = M::EPW, NFACE = S::NFACE, BX = S::BX, NF = S::NF, BO = S::BO, N = S::N, NS = M::NS;
   constexpr int K0 = M::K0, K1 = M::K1, NB = K1 - K0;
   constexpr bool kFx = M::kFx;
@@ -765,12 +793,13 @@ static __global__ void __launch_bounds__(SymRing<T, TD, B, OP, KIND>::NTH, SymRi
     const size_t o = (size_t)unit * B + r;
     load_info(tile + 2 * nw, in2, cn2);
     T own = T(0), rh = T(0), dv = T(0);
-    int se = 0;
+    int ti = 0, ui = 0;                               // scale exponents of the row and of its block inverse
     if (active) {
       if (M::kProduct && (KIND == 2 || OP == SYM_CHEB)) own = x[o];
       if (!(OP == SYM_SPMV && KIND != 1)) rh = rhs[o];
       if (OP == SYM_CHEB && KIND == 2) dv = d[o];
-      if (kFx) se = A.sc[unit];
+      if (kFx) ti = A.sc[o];
+      if (kFxExt) ui = ext.s[o];
     }
     Sum sum = Sum(0);
     int E = kFxNone;
@@ -840,7 +869,7 @@ static __global__ void __launch_bounds__(SymRing<T, TD, B, OP, KIND>::NTH, SymRi
         T y = T(0);
         if (M::kProduct && active) {
           if constexpr (kFx) {
-            if (E < kFxBad / 2) y = fx_scale(sum, se - A.kA + E + kFxBias);
+            if (E < kFxBad / 2) y = fx_scale(sum, ti - A.kA + E + kFxBias);
             else if (OP == SYM_SPMV) y = sym_row_nonfinite<B>(A, unit, r, x);
             else y = nan("");
           } else {
@@ -860,28 +889,29 @@ static __global__ void __launch_bounds__(SymRing<T, TD, B, OP, KIND>::NTH, SymRi
         if (k == K1 - 1) {
           const T t = res;
           int Et = 0;
-          SX* ts = reinterpret_cast<SX*>(part);
+          using TS = typename std::conditional<OP == SYM_CHEB, SX, T>::type;
+          TS* ts = reinterpret_cast<TS*>(part);
           __syncwarp();
           if (active) {
-            if constexpr (kFx) {
-              Et = __reduce_max_sync(emask, fx_exp(t));
-              ts[r] = fx_split(t, Et);
+            if constexpr (kFxExt) {
+              Et = __reduce_max_sync(emask, fx_exp(t, ui));
+              ts[r] = fx_split(t, Et - ui);
             } else {
               ts[r] = t;
             }
           }
           __syncwarp();
           if (active) {
-            Acc acc;
+            XAcc acc;
             if constexpr (OP == SYM_CHEB) {
               sym_tri<T, B>(reinterpret_cast<const SD*>(blk), r, ts, acc);
             } else {
-              const ST* p = ext.v + (size_t)unit * L::KP + r;
+              const SD* p = ext.v + (size_t)unit * SymLay<SD, B>::KP + r;
 #pragma unroll
               for (int i = 0; i < B; ++i) acc.fma(__ldcs(p + i * S::LDP), ts[i]);
             }
             T sv;
-            if constexpr (kFx) sv = Et == 2047 ? nan("") : fx_scale(acc.sum(), Et + kFxBias - ext.k[unit]);
+            if constexpr (kFxExt) sv = Et == kFxBad ? nan("") : fx_scale(acc.sum(), ui + Et + kFxBias - ext.k[unit]);
             else sv = acc.sum();
             if constexpr (OP == SYM_RESTRICT) {
               out[o] = sv;
@@ -891,9 +921,9 @@ static __global__ void __launch_bounds__(SymRing<T, TD, B, OP, KIND>::NTH, SymRi
               const T xn = M::kProduct ? own + dn : dn;
               out[o] = xn;
               if constexpr (kFx) {
-                const int e = __reduce_max_sync(emask, fx_exp(xn));
-                Xo[o] = fx_split(xn, e);
-                if (r == 0) Eo[unit] = e == 2047 ? kFxBad : e + se;
+                const int e = __reduce_max_sync(emask, fx_exp(xn, ti));
+                Xo[o] = fx_split(xn, e - ti);
+                if (r == 0) Eo[unit] = e;
               }
             }
           }
@@ -926,45 +956,26 @@ template <int B> struct SymRows {
 // one thread per element.
 template <typename T, int B>
 static __global__ void __launch_bounds__(SymRows<B>::NT)
-    k_sym_prolong(SymBlk<typename SymNum<T>::ST> P, const int32_t* __restrict__ parent, const T* __restrict__ ec,
+    k_sym_prolong(SymBlk<T> P, const int32_t* __restrict__ parent, const T* __restrict__ ec,
                   T* __restrict__ x, const int16_t* __restrict__ sc, int2* Xo, int* Eo, int64_t n, const CGState* st) {
   if (st && st->done) return;
   using S = SymShape<B>;
-  using ST = typename SymNum<T>::ST;
-  using SX = typename SymNum<T>::SX;
-  constexpr int KP = SymLay<ST, B>::KP, U = SymRows<B>::U, BX = (B + 1) / 2 * 2;
+  constexpr int KP = SymLay<T, B>::KP, U = SymRows<B>::U, BX = (B + 1) / 2 * 2;
   constexpr bool kFx = std::is_same<T, double>::value;
-  __shared__ __align__(16) SX sx[U * BX];
+  __shared__ T sx[U * BX];
   __shared__ int smax[U];
   const int slot = threadIdx.x / B, r = threadIdx.x - slot * B;
   const int64_t unit = (int64_t)blockIdx.x * U + slot;
   const bool active = slot < U && unit < n;
-  T e = T(0);
-  if (active) e = ec[(size_t)parent[unit] * B + r];
-  int E = 0;
-  if constexpr (kFx) {
-    if (threadIdx.x < U) smax[threadIdx.x] = 1;
-    __syncthreads();
-    if (active) atomicMax(smax + slot, fx_exp(e));
-    __syncthreads();
-    if (active) {
-      E = smax[slot];
-      sx[slot * BX + r] = fx_split(e, E);
-    }
-  } else {
-    if (active) sx[slot * BX + r] = e;
-  }
+  if (active) sx[slot * BX + r] = ec[(size_t)parent[unit] * B + r];
   __syncthreads();
   T v = T(0);
   if (active) {
-    const ST* p = P.v + (size_t)unit * KP + r;
-    typename SymNum<T>::Acc acc;
+    const T* p = P.v + (size_t)unit * KP + r;
+    T s = T(0);
     constexpr int kUnroll = (B <= 27) ? B : 16;
 #pragma unroll kUnroll
-    for (int j = 0; j < B; ++j) acc.fma(__ldcs(p + j * S::LDP), sx[slot * BX + j]);
-    T s;
-    if constexpr (kFx) s = E == 2047 ? nan("") : fx_scale(acc.sum(), E + kFxBias - P.k[unit]);
-    else s = acc.sum();
+    for (int j = 0; j < B; ++j) s += __ldcs(p + j * S::LDP) * sx[slot * BX + j];
     v = x[(size_t)unit * B + r] + s;
     x[(size_t)unit * B + r] = v;
   }
