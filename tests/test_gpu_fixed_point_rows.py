@@ -83,3 +83,27 @@ def test_rows_with_contrast(kind, dt, contrast):
             err = float((np.abs(_apply(hier, x, level) - y) / size).max())
             assert err <= (ref.terms + 8) * 2.0 ** -53, (level, err)
     hier.close()
+
+
+@pytest.mark.parametrize("contrast,dt", [(1.0, None), (1e-8, 1000.0)])
+@pytest.mark.parametrize("kind", sorted(WORKLOADS))
+def test_vcycle_with_contrast(kind, contrast, dt):
+    """One float64 V-cycle (products with A_0, its block inverses and transfers)
+    against the oracle's: 12 products of at most T terms between r and z."""
+    from oracle import multigrid as omg
+    from oracle import sipg as osipg
+    from paper_2602_16312_gb300 import aggmg
+    wl = WORKLOADS[kind]()
+    D = wl.conductivity.copy()
+    D[np.random.default_rng(1).random(len(D)) < 0.3] *= contrast
+    c = 1.0 / (wl.dt if dt is None else dt)
+    disc = osipg.assemble(wl.mesh.vertices, wl.mesh.elements, D, wl.degree, wl.penalty_mode, wl.penalty_coeff)
+    mesh = _mesh(wl, contrast)
+    hier = aggmg.Hierarchy(mesh, c, wl.maps, precision="f64")
+    r = np.random.default_rng(3).standard_normal(wl.n_dofs)
+    z = torch.empty(wl.n_dofs, dtype=torch.float64, device="cuda")
+    hier.vcycle_apply(torch.tensor(r, device="cuda"), z)
+    ref = omg.vcycle(omg.build_hierarchy(disc, c, wl.maps), r)
+    err = float(np.abs(z.cpu().numpy() - ref).max() / np.abs(ref).max())
+    assert err <= 12 * mesh.B * (1 + 2 * mesh.dim) * 2.0 ** -53, err
+    hier.close()
