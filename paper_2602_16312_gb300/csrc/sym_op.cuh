@@ -52,8 +52,7 @@
 //   hi = sum a1 x1 <= 2^32 2^27,  m1 = sum a1 x0 <= 2^32 2^30,
 //   m2 = sum a0 x1 <= T 2^27 2^27 < 2^62.3,
 // so none overflows, and every a1 and x1 fits 32 bits. A NaN or infinity in the
-// neighbourhood takes a float64 path over the same entries (products) or gives
-// NaN (smoother).
+// neighbourhood takes a float64 path over the same entries.
 #pragma once
 #include "face_op.cuh"
 #include "kernels.cuh"
@@ -64,18 +63,23 @@ namespace aggmg {
 // bits of a row's entries in sum, of a single entry, of x; of the low halves of
 // an entry and of x
 constexpr int FX_A = 60, FX_AE = 58, FX_X = 58, FX_P = 28, FX_Q = 31;
-constexpr int kFxNone = -100000;                    // below every exponent
-constexpr int kFxBad = 1 << 20;                     // marks a NaN or an infinity
+constexpr int kFxNone = -100000;                    // exponent of zero
+constexpr int kFxInf = 2600;                        // of a NaN or an infinity, above every other scaled one
+constexpr int kFxSpan = 6;                          // see SymVec
+constexpr int kFxWide = -(1 << 20);                 // added to the exponent of an element kept as doubles
+constexpr int kFxRaw = 1823;                        // biased exponent of such an element's largest double
 // largest loss of a fixed-point row relative to sum_j |A_ij|: 8 roundings of a double
 // (a float64 sum of the row's 135 to 700 products rounds as often as it adds)
 constexpr double kFxLoss = 8.0 / 9007199254740992.0;
 // exponent of the unit of FxAcc::sum() for x with shared biased exponent E, less E
 constexpr int kFxBias = FX_P + FX_Q - 1075 - (FX_X - 53);
 
-// biased exponent of x 2^t (as of a subnormal for zero; kFxBad for NaN and Inf)
+// biased exponent of x 2^t
 __device__ __forceinline__ int fx_exp(double x, int t) {
-  const int e = (__double2hiint(x) >> 20) & 0x7ff;
-  return e == 2047 ? kFxBad : (e ? e : 1) + t;
+  const int h = __double2hiint(x), e = (h >> 20) & 0x7ff;
+  if (e == 2047) return kFxInf;
+  if (e == 0) return ((h << 1) | __double2loint(x)) ? 1 + t : kFxNone;
+  return e + t;
 }
 // x in units of 2^{E - 1075 - (FX_X - 53)} rounded to an integer (at most 2^FX_X for
 // E >= fx_exp(x, 0)), as halves (lo, hi)
@@ -85,7 +89,7 @@ __device__ __forceinline__ int2 fx_split(double x, int E) {
   unsigned long long m = ((unsigned long long)(unsigned)(h & 0xfffff) << 32) | (unsigned)__double2loint(x);
   if (e) m |= 1ull << 52;
   else e = 1;
-  const int sh = min(max(E - e, 0), 63);             // (below 0: E of a NaN or infinity)
+  const int sh = min(max(E - e, 0), 63);             // (below 0: x = 0)
   long long v = (long long)((((m << (FX_X - 52)) >> sh) + 1) >> 1);
   v = h < 0 ? -v : v;
   const int lo = ((int)v << (32 - FX_Q)) >> (32 - FX_Q);
@@ -246,8 +250,19 @@ __device__ __forceinline__ void sym_tri(const ST* m, int r, const typename SymNu
 enum { SYM_SPMV = 0, SYM_CHEB = 1, SYM_RESTRICT = 2 };
 
 // A vector as the kernels read it: T = double: fixed point, X[unit B + i] and one
-// exponent per element (the largest biased exponent of its scaled x, kFxBad with a
-// NaN or Inf); T = float: the vector itself.
+// exponent per element (the largest biased exponent of its scaled x); T = float: the
+// vector itself.
+// One exponent per element (and one per row: the largest of the row's blocks) rounds a
+// row that sees nothing but an element's small values, as a neighbour's row sees only
+// its face, to 2^-57 of the large ones. So an element with a face whose largest value
+// is below 2^-kFxSpan of the element's is kept as doubles (E + kFxWide; X the bits
+// of x 2^{s_i} over its power of two), as is one with a NaN or an infinity, and its
+// blocks are multiplied in float64 (sym_wide_row). Every row that an element takes
+// part in then holds a term of 2^-kFxSpan of its largest value, and rounds to about
+// 2^-50 of (|A| |x|)_i, for vectors of any range. (A unit vector over noise of 1e-12: rows
+// beside the unit off by 6e-5 of (|A| |x|)_i before.) Of random vectors and CG
+// directions (from stimuli and fronts) at most 0.4% of the elements were kept as
+// doubles, mostly none; 4% of a first direction from a front on the thin shell.
 template <typename T> struct SymVec {
   const typename SymNum<T>::SX* X;
   const int* E;
@@ -288,60 +303,129 @@ struct SymSmem {
   static constexpr size_t kPart = kProduct ? round_to(U * S::NFACE * B * (int)sizeof(Sum), 16) : 0;
   static constexpr size_t kRed = round_to((G - 1) * U * B * (int)sizeof(Sum), 16);
   static constexpr size_t kTs = (OP == SYM_SPMV) ? 0 : round_to(U * S::BX * (int)sizeof(SX), 16);
-  static constexpr size_t kRest = kPart + kRed + kTs + round_to(2 * U * (int)sizeof(int), 16);
+  static constexpr size_t kRest = kPart + kRed + kTs + round_to((1 + 2 * (1 + S::NFACE)) * (int)sizeof(int), 16);
   static constexpr int kStages = (2 * kStage + kRest <= 225 * 1024) ? 2 : 1;
   static constexpr size_t bytes = kStages * kStage + kRest;
 };
 
-// The row's product over stored entries in float64, for neighbourhoods that
-// hold a NaN or an infinity (agg_operator_apply passes those on as before).
+// y plus row r's products with those of its blocks whose element is kept as doubles
+// (SymVec), in float64 over the stored entries. The integer sums that the kernels
+// form of such blocks carry exponents so low that they are shifted out.
 template <int B>
-__device__ __noinline__ double sym_row_nonfinite(const SymView<double, B>& A, int64_t unit, int r, const double* x) {
+__device__ __forceinline__ double sym_wide_row(const SymView<double, B>& A, int64_t unit, int r, double y, const int2* X,
+                                               const int* E) {
   using S = SymShape<B>;
   using L = SymLay<int2, B>;
   using FI = FaceIdx<S::D, S::N>;
-  const int16_t* se = A.sc + (size_t)unit * B;
-  double y = 0.0;
-  auto val = [&](int2 a, int s) { return scalbn((double)(((long long)a.y << FX_P) + a.x), se[r] + s - A.kA); };
-  for (int c = 0; c < B; ++c) {
-    const int hi = max(r, c), lo = min(r, c);
-    y += val(A.diag[(size_t)unit * L::KD + hi * (hi + 1) / 2 + lo], se[c]) * x[(size_t)unit * B + c];
+  auto term = [](int2 a, int2 x) {
+    return (double)(((long long)a.y << FX_P) + a.x) * __hiloint2double(x.y, x.x);
+  };
+  const int q = A.sc[(size_t)unit * B + r] - A.kA - kFxWide - kFxRaw;
+  if (E[unit] < kFxWide / 2) {
+    const int2 *m = A.diag + (size_t)unit * L::KD, *x = X + (size_t)unit * B;
+    double s = 0.0;
+#pragma unroll 4
+    for (int c = 0; c < B; ++c) s += term(m[c <= r ? r * (r + 1) / 2 + c : c * (c + 1) / 2 + r], x[c]);
+    y += scalbn(s, q + E[unit]);
   }
   for (int f = 0; f < S::NFACE; ++f) {
     const int2 nf = A.info[unit * S::NFACE + f];
-    if (nf.x < 0) continue;
+    if (nf.x < 0 || E[nf.x] >= kFxWide / 2) continue;
     const int fn = A.code[unit * S::NFACE + f];
-    const int16_t* sn = A.sc + (size_t)nf.x * B;
-    const bool tr = nf.x < unit;
+    const bool tr = nf.x < unit;                      // the block is the neighbour's: row of K^T
     bool on;
     const int pos = face_first<B>(f, r, on);
-    const int2* blk = A.face + (size_t)nf.y * L::KB;
-    const int2* g = blk + S::NF * S::LDF;
-    const double* xn = x + (size_t)nf.x * B;
-    for (int t = 0; t < (on ? B : S::NF); ++t) {
-      const int dof = t < S::NF ? FI::face(fn, t) : FI::off(fn, t - S::NF);
-      const int2 a = tr ? (on ? blk[pos * S::LDF + t] : g[(pos - S::NF) * S::LDG + t])
-                        : (t < S::NF ? blk[t * S::LDF + pos] : g[(t - S::NF) * S::LDG + pos]);
-      y += val(a, sn[dof]) * xn[dof];
+    const int2 *F = A.face + (size_t)nf.y * L::KB, *Gb = F + S::NF * S::LDF, *x = X + (size_t)nf.x * B;
+    const int2* p = tr ? (on ? F + pos * S::LDF : Gb + (pos - S::NF) * S::LDG) : F + pos;
+    double s = 0.0;
+#pragma unroll 3
+    for (int t = 0; t < S::NF; ++t) s += term(p[tr ? t : t * S::LDF], x[FI::face(fn, t)]);
+    if (on) {
+      p = tr ? F + pos * S::LDF + S::NF : Gb + pos;
+#pragma unroll 3
+      for (int t = 0; t < S::BO; ++t) s += term(p[tr ? t : t * S::LDG], x[FI::off(fn, t)]);
     }
+    y += scalbn(s, q + E[nf.x]);
   }
   return y;
 }
+// The same as a call: k_sym is faster with it (V-cycle of the 18^3 Q3 cube 2,288 inline,
+// 2,272 us), k_symw<9> inline (V-cycle on 250^2 Q2 556, 542 us).
+template <int B>
+__device__ __noinline__ double sym_wide_row_call(SymView<double, B> A, int64_t unit, int r, double y, const int2* X,
+                                                 const int* E) {
+  return sym_wide_row<B>(A, unit, r, y, X, E);
+}
+
+// An element's vector copy (SymVec): E the largest scaled exponent of its values, mn
+// the least of its faces' largest ones.
+__device__ __forceinline__ bool fx_raw(int E, int mn) { return E == kFxInf || mn < E - kFxSpan; }
+static __device__ __noinline__ int2 fx_double(double v, int q) {
+  const double w = scalbn(v, q);
+  return make_int2(__double2loint(w), __double2hiint(w));
+}
+__device__ __forceinline__ int2 fx_copy(double v, int t, int E, bool raw) {
+  return raw ? fx_double(v, t + kFxRaw - E) : fx_split(v, E - t);
+}
+template <int B>
+__device__ __forceinline__ bool on_face(int f, int r) {
+  bool on;
+  face_first<B>(f, r, on);
+  return on;
+}
+// lanes (r) of the DoFs of each face, B <= 32
+template <int B>
+struct FaceLanes {
+  unsigned v[6] = {};
+  constexpr FaceLanes() {
+    constexpr int N = SymShape<B>::N;
+    for (int f = 0; f < SymShape<B>::NFACE; ++f)
+      for (int r = 0; r < B; ++r) {
+        const int i = f < 2 ? r % N : (f < 4 ? r / N % N : r / (N * N));
+        if (i == (f & 1) * (N - 1)) v[f] |= 1u << (r & 31);
+      }
+  }
+};
 
 // Fixed-point copy of one value per thread, a block of threads holding whole
-// elements (thread = slot B + r): X and E of SymVec. se: shared int per slot.
-template <int B>
+// elements (thread = slot B + r): X and E of SymVec.
+template <int B, int U>
+struct FxShared {
+  int mx[U], mn[U], ex[U * B];
+};
+template <int B, int U>
 __device__ __forceinline__ void fx_store(double v, bool active, int slot, int64_t unit, int r, const int16_t* sc, int2* X,
-                                         int* E, int* se, int U) {
-  if (threadIdx.x < U) se[threadIdx.x] = kFxNone;
-  const int t = active ? sc[(size_t)unit * B + r] : 0;
-  __syncthreads();
-  if (active) atomicMax(se + slot, fx_exp(v, t));
+                                         int* E, FxShared<B, U>& sh) {
+  using S = SymShape<B>;
+  using FI = FaceIdx<S::D, S::N>;
+  if (threadIdx.x < U) {
+    sh.mx[threadIdx.x] = kFxNone;
+    sh.mn[threadIdx.x] = kFxInf;
+  }
+  const size_t o = (size_t)unit * B + r;
+  const int t = active ? sc[o] : 0;
+  const int e = fx_exp(v, t);
+  if (active) sh.ex[slot * B + r] = e;
   __syncthreads();
   if (active) {
-    const int e = se[slot];
-    X[(size_t)unit * B + r] = fx_split(v, e - t);
-    if (r == 0) E[unit] = e;
+    if (r < S::NFACE) {                               // face r's
+      int m = kFxNone;
+#pragma unroll
+      for (int j = 0; j < S::NF; ++j) m = max(m, sh.ex[slot * B + FI::face(r, j)]);
+      atomicMax(sh.mx + slot, m);
+      atomicMin(sh.mn + slot, m);
+    }
+    bool inner = true;
+#pragma unroll
+    for (int f = 0; f < S::NFACE; ++f) inner = inner && !on_face<B>(f, r);
+    if (inner) atomicMax(sh.mx + slot, e);
+  }
+  __syncthreads();
+  if (active) {
+    const int em = sh.mx[slot];
+    const bool raw = fx_raw(em, sh.mn[slot]);
+    X[o] = fx_copy(v, t, em, raw);
+    if (r == 0) E[unit] = raw ? em + kFxWide : em;
   }
 }
 
@@ -378,6 +462,7 @@ static __global__ void __launch_bounds__(SymSmem<T, TD, B, OP, KIND>::NTH)
   constexpr bool kFx = M::kFx;
   constexpr int kShare = BO / N;                      // off-face terms of a face row per thread
   constexpr int FPG = (G == 1) ? NFACE : (NFACE + G - 2) / (G - 1);   // faces per group
+  static_assert(U == 1 && B == 64, "two warps hold an element's rows");
   if (st && st->done) return;
   extern __shared__ __align__(16) unsigned char sym_sm[];
   Sum* spart = reinterpret_cast<Sum*>(sym_sm + M::kStages * M::kStage);
@@ -489,7 +574,7 @@ static __global__ void __launch_bounds__(SymSmem<T, TD, B, OP, KIND>::NTH)
     } else {
       asm volatile("cp.async.wait_group 0;" ::: "memory");
     }
-    if (OP != SYM_SPMV && tid < 2 * U) smax[tid] = kFxNone;
+    if (OP != SYM_SPMV && tid == 0) smax[0] = kFxNone;
     __syncthreads();
     unsigned char* base = sym_sm + sg * M::kStage;
     const ST* eb = reinterpret_cast<ST*>(base) + slot * M::KE;
@@ -519,12 +604,16 @@ static __global__ void __launch_bounds__(SymSmem<T, TD, B, OP, KIND>::NTH)
     int E = kFxNone;
     if constexpr (M::kProduct) {
       Sum sum = Sum(0);
-      if (active) {
-        if constexpr (kFx) {
-          E = ee[0];
+      int lo = kFxNone;                               // largest (E) and least exponent of the blocks
+      if constexpr (kFx) {
+        E = lo = ee[0];
 #pragma unroll
-          for (int f = 0; f < NFACE; ++f) E = max(E, ee[f + 1]);
+        for (int k = 1; k <= NFACE; ++k) {
+          E = max(E, ee[k]);
+          lo = min(lo, ee[k]);
         }
+      }
+      if (active) {
         if (g == 0) {
           Acc acc;
           sym_tri<T, B>(eb, r, ex, acc);
@@ -573,9 +662,8 @@ static __global__ void __launch_bounds__(SymSmem<T, TD, B, OP, KIND>::NTH)
           }
         }
         if constexpr (kFx) {
-          if (E != kFxBad) y = fx_scale(sum, ti - A.kA + E + kFxBias);
-          else if (OP == SYM_SPMV) y = sym_row_nonfinite<B>(A, unit, r, x);
-          else y = nan("");
+          y = fx_scale(sum, ti - A.kA + E + kFxBias);
+          if (lo < kFxWide / 2) y = sym_wide_row_call<B>(A, unit, r, E < kFxWide / 2 ? 0.0 : y, xv.X, xv.E);
         } else {
           y = sum;
         }
@@ -622,7 +710,7 @@ static __global__ void __launch_bounds__(SymSmem<T, TD, B, OP, KIND>::NTH)
 #pragma unroll
         for (int k = 0; k < G - 1; ++k) es += xred[k * U * B + slot * B + r];
         T sv;
-        if constexpr (kFxExt) sv = Et == kFxBad ? nan("") : fx_scale(es, ui + Et + kFxBias - ext.k[unit]);
+        if constexpr (kFxExt) sv = Et == kFxInf ? nan("") : fx_scale(es, ui + Et + kFxBias - ext.k[unit]);
         else sv = es;
         if constexpr (OP == SYM_RESTRICT) {
           out[o] = sv;
@@ -634,12 +722,28 @@ static __global__ void __launch_bounds__(SymSmem<T, TD, B, OP, KIND>::NTH)
         }
       }
       if constexpr (kFx && OP == SYM_CHEB) {
-        if (lead) atomicMax(smax + U + slot, fx_exp(res, ti));
+        // largest exponents of the two warps that hold the rows: all values, face by face
+        int* wmax = smax + 1;
+        if (lead) {
+          const int e = fx_exp(res, ti);
+#pragma unroll
+          for (int f = -1; f < NFACE; ++f) {
+            const int m = __reduce_max_sync(0xffffffffu, f < 0 || on_face<B>(f, r) ? e : kFxNone);
+            if ((tid & 31) == 0) wmax[(tid >> 5) * (1 + NFACE) + f + 1] = m;
+          }
+        }
         __syncthreads();
         if (lead) {
-          const int e = smax[U + slot];
-          Xo[o] = fx_split(res, e - ti);
-          if (r == 0) Eo[unit] = e;
+          int mn = kFxInf;
+#pragma unroll
+          for (int f = 0; f < NFACE; ++f) {
+            const int m = max(wmax[f + 1], wmax[1 + NFACE + f + 1]);
+            mn = min(mn, m);
+          }
+          const int em = max(wmax[0], wmax[1 + NFACE]);
+          const bool raw = fx_raw(em, mn);
+          Xo[o] = fx_copy(res, ti, em, raw);
+          if (r == 0) Eo[unit] = raw ? em + kFxWide : em;
         }
       }
     }
@@ -802,7 +906,7 @@ static __global__ void __launch_bounds__(SymRing<T, TD, B, OP, KIND>::NTH, SymRi
       if (kFxExt) ui = ext.s[o];
     }
     Sum sum = Sum(0);
-    int E = kFxNone;
+    int E = kFxNone, lo = kFxNone;                    // largest and least exponent of the blocks
     T res = T(0);
     constexpr int kBlkUnroll = (S::D == 2) ? NB : 1;
 #pragma unroll kBlkUnroll
@@ -822,7 +926,7 @@ static __global__ void __launch_bounds__(SymRing<T, TD, B, OP, KIND>::NTH, SymRi
           Acc acc;
           sym_tri<T, B>(blk, r, xs, acc);
           sum = acc.sum();
-          if constexpr (kFx) E = *slot_e(slot);
+          if constexpr (kFx) E = lo = *slot_e(slot);
         }
       } else if (k <= NFACE) {
         const int f = k - 1;
@@ -853,6 +957,7 @@ static __global__ void __launch_bounds__(SymRing<T, TD, B, OP, KIND>::NTH, SymRi
           }
           if constexpr (kFx) {
             const int e = *slot_e(slot);
+            lo = min(lo, e);
             if (e > E) {
               sum = sum_shift(sum, e - E) + s;
               E = e;
@@ -869,9 +974,8 @@ static __global__ void __launch_bounds__(SymRing<T, TD, B, OP, KIND>::NTH, SymRi
         T y = T(0);
         if (M::kProduct && active) {
           if constexpr (kFx) {
-            if (E < kFxBad / 2) y = fx_scale(sum, ti - A.kA + E + kFxBias);
-            else if (OP == SYM_SPMV) y = sym_row_nonfinite<B>(A, unit, r, x);
-            else y = nan("");
+            y = fx_scale(sum, ti - A.kA + E + kFxBias);
+            if (lo < kFxWide / 2) y = sym_wide_row<B>(A, unit, r, E < kFxWide / 2 ? 0.0 : y, xv.X, xv.E);
           } else {
             y = sum;
           }
@@ -911,7 +1015,7 @@ static __global__ void __launch_bounds__(SymRing<T, TD, B, OP, KIND>::NTH, SymRi
               for (int i = 0; i < B; ++i) acc.fma(__ldcs(p + i * S::LDP), ts[i]);
             }
             T sv;
-            if constexpr (kFxExt) sv = Et == kFxBad ? nan("") : fx_scale(acc.sum(), ui + Et + kFxBias - ext.k[unit]);
+            if constexpr (kFxExt) sv = Et == kFxInf ? nan("") : fx_scale(acc.sum(), ui + Et + kFxBias - ext.k[unit]);
             else sv = acc.sum();
             if constexpr (OP == SYM_RESTRICT) {
               out[o] = sv;
@@ -921,9 +1025,14 @@ static __global__ void __launch_bounds__(SymRing<T, TD, B, OP, KIND>::NTH, SymRi
               const T xn = M::kProduct ? own + dn : dn;
               out[o] = xn;
               if constexpr (kFx) {
-                const int e = __reduce_max_sync(emask, fx_exp(xn, ti));
-                Xo[o] = fx_split(xn, e - ti);
-                if (r == 0) Eo[unit] = e;
+                const int e = fx_exp(xn, ti), em = __reduce_max_sync(emask, e);
+                const unsigned big = __ballot_sync(emask, e >= em - kFxSpan) >> (sub * B);
+                constexpr FaceLanes<B> kLanes;
+                bool raw = em == kFxInf;
+#pragma unroll
+                for (int f = 0; f < NFACE; ++f) raw = raw || !(big & kLanes.v[f]);
+                Xo[o] = fx_copy(xn, ti, em, raw);
+                if (r == 0) Eo[unit] = raw ? em + kFxWide : em;
               }
             }
           }
@@ -963,7 +1072,7 @@ static __global__ void __launch_bounds__(SymRows<B>::NT)
   constexpr int KP = SymLay<T, B>::KP, U = SymRows<B>::U, BX = (B + 1) / 2 * 2;
   constexpr bool kFx = std::is_same<T, double>::value;
   __shared__ T sx[U * BX];
-  __shared__ int smax[U];
+  __shared__ FxShared<B, U> sh;
   const int slot = threadIdx.x / B, r = threadIdx.x - slot * B;
   const int64_t unit = (int64_t)blockIdx.x * U + slot;
   const bool active = slot < U && unit < n;
@@ -979,7 +1088,7 @@ static __global__ void __launch_bounds__(SymRows<B>::NT)
     v = x[(size_t)unit * B + r] + s;
     x[(size_t)unit * B + r] = v;
   }
-  if constexpr (kFx) fx_store<B>(v, active, slot, unit, r, sc, Xo, Eo, smax, U);
+  if constexpr (kFx) fx_store<B, U>(v, active, slot, unit, r, sc, Xo, Eo, sh);
 }
 
 // x's fixed-point copy
@@ -988,11 +1097,11 @@ static __global__ void __launch_bounds__(SymRows<B>::NT)
     k_fx(const double* __restrict__ x, int64_t n, const int16_t* __restrict__ sc, int2* __restrict__ X,
          int* __restrict__ E, const CGState* st) {
   if (st && st->done) return;
-  __shared__ int se[SymRows<B>::U];
+  __shared__ FxShared<B, SymRows<B>::U> sh;
   const int slot = threadIdx.x / B, r = threadIdx.x - slot * B;
   const int64_t unit = (int64_t)blockIdx.x * SymRows<B>::U + slot;
   const bool active = slot < SymRows<B>::U && unit < n;
-  fx_store<B>(active ? x[(size_t)unit * B + r] : 0.0, active, slot, unit, r, sc, X, E, se, SymRows<B>::U);
+  fx_store<B, SymRows<B>::U>(active ? x[(size_t)unit * B + r] : 0.0, active, slot, unit, r, sc, X, E, sh);
 }
 // p = z + beta p (INIT: p = z), as k_pupd, with p's fixed-point copy
 template <typename TZ, int B, bool INIT>
@@ -1000,7 +1109,7 @@ static __global__ void __launch_bounds__(SymRows<B>::NT)
     k_pupd_fx(const TZ* __restrict__ z, double* __restrict__ p, int64_t n, const double* partials, int np,
               const int16_t* __restrict__ sc, int2* __restrict__ X, int* __restrict__ E, CGState* st) {
   if (st->done) return;
-  __shared__ int se[SymRows<B>::U];
+  __shared__ FxShared<B, SymRows<B>::U> sh;
   const double beta = cg_beta<SymRows<B>::NT, INIT>(partials, np, st);
   const int slot = threadIdx.x / B, r = threadIdx.x - slot * B;
   for (int64_t u0 = (int64_t)blockIdx.x * SymRows<B>::U; u0 < n; u0 += (int64_t)gridDim.x * SymRows<B>::U) {
@@ -1012,7 +1121,7 @@ static __global__ void __launch_bounds__(SymRows<B>::NT)
       v = INIT ? to_double(z[o]) : to_double(z[o]) + beta * p[o];
       p[o] = v;
     }
-    fx_store<B>(v, active, slot, unit, r, sc, X, E, se, SymRows<B>::U);
+    fx_store<B, SymRows<B>::U>(v, active, slot, unit, r, sc, X, E, sh);
     __syncthreads();
   }
 }

@@ -107,3 +107,60 @@ def test_vcycle_with_contrast(kind, contrast, dt):
     err = float(np.abs(z.cpu().numpy() - ref).max() / np.abs(ref).max())
     assert err <= 12 * mesh.B * (1 + 2 * mesh.dim) * 2.0 ** -53, err
     hier.close()
+
+
+def _vectors(wl, rng):
+    """Vectors whose values differ by many orders of magnitude, within elements
+    and from element to element."""
+    n, B = wl.n_dofs, (wl.degree + 1) ** wl.mesh.dim
+    N = wl.degree + 1
+    index = np.arange(B)
+    inner = np.ones(B, bool)
+    for k in range(wl.mesh.dim):
+        i = index // N ** k % N
+        inner &= (i > 0) & (i < N - 1)
+    noise = rng.standard_normal(n)
+    centre = wl.mesh.vertices[wl.mesh.elements].mean(1)
+    dist = np.linalg.norm(centre - centre[0], axis=1)
+    steps = dist / np.sort(dist)[1]
+    out = {}
+    mid = n // B // 2 * B
+    for name, dof in (("corner", 0), ("inner", int(index[inner][0]))):
+        out["unit_" + name] = np.eye(1, n, mid + dof)[0]
+        for tiny in (1e-2, 1e-4, 1e-12, 1e-30):
+            out[f"unit_{name}_over_{tiny}"] = np.eye(1, n, mid + dof)[0] + tiny * noise
+    out["decay"] = noise * 10.0 ** (-3.0 * np.repeat(steps, B))
+    out["by_element"] = noise * np.repeat(10.0 ** rng.uniform(-30, 30, n // B), B)
+    out["by_dof"] = noise * 10.0 ** rng.uniform(-30, 30, n)
+    out["bubbles"] = noise * np.where(np.tile(inner, n // B), 1.0, 1e-9)
+    out["sparse"] = np.where(np.repeat(rng.random(n // B) < 0.2, B), noise, 0.0)
+    return out
+
+
+@pytest.mark.parametrize("contrast", [1.0, 1e-4])
+@pytest.mark.parametrize("kind", sorted(WORKLOADS))
+def test_rows_for_vectors_of_any_range(kind, contrast):
+    """Values of a neighbour that a row does not see take nothing from it. Beyond
+    the bound above a row may lose, of each block, 16 products' low halves: 2^-58 of
+    sqrt(A_ii A_jj) times the element's largest |x_j|, which is at most 2^8 times
+    the largest one that the row sees: 2^-45 sum_j sqrt(A_ii A_jj) |x_j| over
+    the row's entries with room for the roundings to powers of two."""
+    from paper_2602_16312_gb300 import aggmg
+    wl = WORKLOADS[kind]()
+    mesh = _mesh(wl, contrast)
+    hier = aggmg.Hierarchy(mesh, 1.0 / wl.dt, wl.maps, precision="f64")
+    ref = Rows(mesh, 1.0 / wl.dt)
+    d = np.zeros(ref.shape)
+    for k in np.nonzero(ref.rows == ref.cols)[0]:
+        d[ref.rows[k]] = np.sqrt(np.diag(ref.A[k]).astype(float))
+    seen = (ref.A != 0).astype(float)
+    for name, x in _vectors(wl, np.random.default_rng(5)).items():
+        y, size = ref.product(x)
+        part = np.zeros(ref.shape)
+        np.add.at(part, ref.rows, (seen * (d * np.abs(x.reshape(ref.shape)))[ref.cols][:, None, :]).sum(2))
+        tol = (ref.terms + 8) * 2.0 ** -53 * size + 2.0 ** -45 * (d * part).ravel()
+        for level in (0, -1):
+            off = np.abs(_apply(hier, x, level) - y)
+            worst = int(np.argmax(np.where(tol > 0, off / np.where(tol > 0, tol, 1), 0)))
+            assert (off <= tol).all(), (name, level, worst, float(off[worst]), float(size[worst]), float(tol[worst]))
+    hier.close()
