@@ -360,37 +360,45 @@ class Engine : public EngineBase {
   }
 
   // ---- symmetric level-0 blocks (sym_op.cuh)
-  // Whether the assembled operator is symmetric up to rounding, relative to
-  // sqrt(A_ii A_jj).
-  static bool sym_check(const FaceBlocks& fb, int64_t n) {
+  // Largest |A_ij - A_ji| of the assembled operator, relative to sqrt(A_ii A_jj)
+  // (infinite with a NaN or a face that the two sides do not share). The assembly's
+  // own rounding leaves up to 1.3e-15 (squares, cubes and shells of p = 2, 3,
+  // contrasts of 1e6 included). The symmetric blocks hold one of the two entries, or
+  // their mean: in float64 up to kAsymF64, within what a row's sum rounds, in float32
+  // up to kAsymF32, far below a rounding. More asymmetry keeps the face-structured form.
+  static constexpr double kAsymF64 = 7.2e-15, kAsymF32 = 1e-11;
+  static double asymmetry(const FaceBlocks& fb, int64_t n) {
     using S = SymShape<B>;
     using FI = FaceIdx<S::D, S::N>;
     const int nf = S::NFACE, NF = S::NF;
-    int bad = 0;
-#pragma omp parallel for schedule(static) reduction(+ : bad)
+    double worst = 0.0;
+#pragma omp parallel for schedule(static) reduction(max : worst)
     for (int64_t u = 0; u < n; ++u) {
       const double* D = &fb.diag[(size_t)u * B * B];
       auto dg = [&](int64_t e, int i) { return std::sqrt(std::fabs(fb.diag[(size_t)e * B * B + (size_t)i * B + i])); };
-      auto off = [&](double a, double b, double sc) { return !(std::fabs(a - b) <= 1e-11 * sc); };
+      auto see = [&](double a, double b, double sc) {
+        if (!(std::fabs(a - b) <= worst * sc)) worst = sc > 0.0 ? std::fabs(a - b) / sc : INFINITY;
+        if (!(worst >= 0.0)) worst = INFINITY;
+      };
       for (int i = 0; i < B; ++i)
-        for (int j = 0; j < i; ++j) bad += off(D[i * B + j], D[j * B + i], dg(u, i) * dg(u, j));
+        for (int j = 0; j < i; ++j) see(D[i * B + j], D[j * B + i], dg(u, i) * dg(u, j));
       for (int f = 0; f < nf; ++f) {
         const int64_t nb = fb.nbr[(size_t)u * nf + f];
         if (nb < 0) continue;
         const int fn = fb.code[(size_t)u * nf + f];
-        if (fb.nbr[(size_t)nb * nf + fn] != u || fb.code[(size_t)nb * nf + fn] != f) { bad += 1; continue; }
+        if (fb.nbr[(size_t)nb * nf + fn] != u || fb.code[(size_t)nb * nf + fn] != f) { worst = INFINITY; continue; }
         const double* R = &fb.R[((size_t)u * nf + f) * NF * B];
         const double* Rn = &fb.R[((size_t)nb * nf + fn) * NF * B];
         const double* Cn = &fb.C[((size_t)nb * nf + fn) * (B - NF) * NF];
         for (int j = 0; j < NF; ++j) {
           for (int c = 0; c < NF; ++c)
-            bad += off(R[j * B + FI::face(fn, c)], Rn[c * B + FI::face(f, j)], dg(u, FI::face(f, j)) * dg(nb, FI::face(fn, c)));
+            see(R[j * B + FI::face(fn, c)], Rn[c * B + FI::face(f, j)], dg(u, FI::face(f, j)) * dg(nb, FI::face(fn, c)));
           for (int c = 0; c < B - NF; ++c)
-            bad += off(R[j * B + FI::off(fn, c)], Cn[c * NF + j], dg(u, FI::face(f, j)) * dg(nb, FI::off(fn, c)));
+            see(R[j * B + FI::off(fn, c)], Cn[c * NF + j], dg(u, FI::face(f, j)) * dg(nb, FI::off(fn, c)));
         }
       }
     }
-    return bad == 0;
+    return worst;
   }
 
   // v 2^k as a fixed-point entry (low half balanced)
@@ -1327,14 +1335,14 @@ class Engine : public EngineBase {
       face_entries_ = (double)m.ne * B * B + (double)nface * (2.0 * fb.NF * B - (double)fb.NF * fb.NF);
       constexpr bool kDouble = std::is_same<T, double>::value;
       const bool assembled = kDouble || fine_operator != 1;   // the V-cycle's level-0 operator
-      const bool symmetric = sym_check(fb, m.ne);
+      const double asym = asymmetry(fb, m.ne);
       // float64 forms: where fixed point holds the rows to a double's accuracy
       std::vector<int16_t> sc, ds, dk;
       int kA = 0;
-      const bool fixed = symmetric && (kOuterSym || (kCycleSym && kDouble)) && sym_scales(fb, m.ne, sc, kA);
+      const bool fixed = asym <= kAsymF64 && (kOuterSym || (kCycleSym && kDouble)) && sym_scales(fb, m.ne, sc, kA);
       osym_ = fixed && kOuterSym;
-      sym_ = symmetric && kCycleSym && assembled;
-      if (kDouble) sym_ = sym_ && fixed && (nlev_ == 1 || block_scales(h.lev[0].Dinv, m.ne, ds, dk));
+      sym_ = kCycleSym && assembled && (kDouble ? fixed : asym <= kAsymF32);
+      if (kDouble) sym_ = sym_ && (nlev_ == 1 || block_scales(h.lev[0].Dinv, m.ne, ds, dk));
       if (osym_ || (sym_ && kDouble)) {
         if ((rc = upload_sym<double>(fb, m.ne, sc, kA, A0s_, err))) return rc;
       }

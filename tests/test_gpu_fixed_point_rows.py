@@ -164,3 +164,32 @@ def test_rows_for_vectors_of_any_range(kind, contrast):
             worst = int(np.argmax(np.where(tol > 0, off / np.where(tol > 0, tol, 1), 0)))
             assert (off <= tol).all(), (name, level, worst, float(off[worst]), float(size[worst]), float(tol[worst]))
     hier.close()
+
+
+@pytest.mark.parametrize("skew", [1e-11, 1e-12])
+@pytest.mark.parametrize("kind", sorted(WORKLOADS))
+def test_rows_with_a_slightly_unsymmetric_conductivity(kind, skew):
+    """D_01 = D_10 + skew sqrt(D_00 D_11): the operator's entries and not the means
+    of (i, j) and (j, i) are multiplied. The bound takes what the symmetric form may
+    differ by where it is kept (7.2e-15 of sqrt(A_ii A_jj))."""
+    from paper_2602_16312_gb300 import aggmg
+    wl = WORKLOADS[kind]()
+    D = wl.conductivity.copy()
+    D[:, 0, 1] += skew * np.sqrt(D[:, 0, 0] * D[:, 1, 1])
+    mesh = aggmg.Mesh.from_workload(wl, conductivity=D)
+    c = 1.0 / wl.dt
+    hier = aggmg.Hierarchy(mesh, c, wl.maps, precision="f64")
+    ref = Rows(mesh, c)
+    d = np.zeros(ref.shape)
+    for k in np.nonzero(ref.rows == ref.cols)[0]:
+        d[ref.rows[k]] = np.sqrt(np.diag(ref.A[k]).astype(float))
+    x = np.random.default_rng(2).standard_normal(wl.n_dofs)
+    y, size = ref.product(x)
+    root = np.zeros(ref.shape)
+    # rms of a sum of random signs: the skew of every entry is bounded on its own
+    np.add.at(root, ref.rows, ((ref.A != 0) * (d * x.reshape(ref.shape))[ref.cols][:, None, :].astype(float) ** 2).sum(2))
+    tol = (ref.terms + 8) * 2.0 ** -53 * size + 7.2e-15 * (d * np.sqrt(root)).ravel()
+    for level in (0, -1):
+        off = np.abs(_apply(hier, x, level) - y)
+        assert (off <= tol).all(), (level, float((off / tol).max()))
+    hier.close()
