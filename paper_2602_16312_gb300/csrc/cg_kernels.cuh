@@ -270,16 +270,17 @@ constexpr int kMaxGates = 3;
 __host__ __device__ inline int ionic_gates(int model) { return model == 2 ? 3 : 1; }
 
 __device__ __forceinline__ double unit_step(double z, double z0) { return z >= z0 ? 1.0 : 0.0; }
+// The smoothed step S = (1 + tanh(k (z - z0))) / 2 = 1 / (1 + exp(t)), t = -2 k (z - z0),
+// and 1 / (tau + dtau S). Where exp(t) is so large that tau exp(t) might overflow (t
+// >= 50, tested on the high word), S is exp(-t) to the last bit.
 __device__ __forceinline__ double smooth_step(double z, double z0, double k) {
-  return 0.5 * (1.0 + tanh(k * (z - z0)));
+  return 1.0 / (1.0 + exp(-2.0 * k * (z - z0)));
 }
-
-// (1 + tanh(k (z - z0))) / 2 = 1 / (1 + e), with e = exp(-2 k (z - z0)) kept finite
-// (a NaN stays one)
-__device__ __forceinline__ double smooth_exp(double z, double z0, double k) {
-  double t = -2.0 * k * (z - z0);
-  t = t > 700.0 ? 700.0 : t;
-  return exp(t);
+__device__ __forceinline__ double smooth_rate(double z, double z0, double k, double tau, double dtau) {
+  const double t = -2.0 * k * (z - z0);
+  if (__double2hiint(t) >= 0x40490000) return 1.0 / (tau + dtau * exp(-t));
+  const double e1 = 1.0 + exp(t);
+  return e1 / (dtau + tau * e1);
 }
 
 // Bueno-Orovio (Section 2.3.2, Eq. BuenoOrovio). The float64 pipe bounds these
@@ -296,15 +297,12 @@ __device__ __forceinline__ void bueno_orovio_rates(const IonicParams& q, double 
   const double b0 = -hv1 * q.inv.tau1plus;
   const double w0inf = 1.0 - hv1m;
   double a1 = 0.0;                                    // behind 1 - H_V2
-  if (hv2 == 0.0) {
-    const double e1 = 1.0 + smooth_exp(u, p.V2m, p.k2);
-    a1 = e1 / ((p.tau2pp - p.tau2p) + p.tau2p * e1);
-  }
+  if (hv2 == 0.0) a1 = smooth_rate(u, p.V2m, p.k2, p.tau2p, p.tau2pp - p.tau2p);
   const double b1 = -hv2 * q.inv.tau2plus;
   const double ut = u * q.inv.tau2inf;
   const double w1inf = hvo * (p.winf_star - 1.0 + ut) + 1.0 - ut;
   const double a2 = hv2 != 0.0 ? q.inv.a2_hi : q.inv.a2_lo;
-  const double w2inf = 1.0 / (1.0 + smooth_exp(u, p.V3, p.k3));
+  const double w2inf = smooth_step(u, p.V3, p.k3);
   H[0] = (b0 - a0) * w[0] + a0 * w0inf;
   H[1] = (b1 - a1) * w[1] + a1 * w1inf;
   H[2] = -a2 * w[2] + a2 * w2inf;
@@ -315,10 +313,7 @@ __device__ __forceinline__ double bueno_orovio_current(const IonicParams& q, dou
   const double hv1 = unit_step(u, p.V1), hv2 = unit_step(u, p.V2), hvo = unit_step(u, p.Vo);
   const double ifi = -hv1 * (u - p.V1) * (p.Vhat - u) * w[0] * q.inv.taufi;
   double iso = (1.0 - hv2) * (u - p.uo) * (hvo != 0.0 ? q.inv.o_hi : q.inv.o_lo);
-  if (hv2 != 0.0) {
-    const double e1 = 1.0 + smooth_exp(u, p.Vso, p.kso);
-    iso += e1 / ((p.tauso_pp - p.tauso_p) + p.tauso_p * e1);
-  }
+  if (hv2 != 0.0) iso += smooth_rate(u, p.Vso, p.kso, p.tauso_p, p.tauso_pp - p.tauso_p);
   const double isi = -hv2 * w[1] * w[2] * q.inv.tausi;
   return ifi + iso + isi;
 }
