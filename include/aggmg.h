@@ -390,9 +390,11 @@ agg_status agg_theta_gradient(agg_hier_t hier, const double* grad_logD_dev, doub
  * inverse + two axpys), 2 fine residual + restriction, 3 fine prolongation.
  * agg_profile_kernel launches the kernel `reps` times on the hierarchy's own
  * work buffers (valid after any solve or V-cycle) on `stream`, so a caller
- * can time it with events; agg_kernel_cost gives its algorithmic HBM bytes
- * (every matrix, block and vector entry read or written once) and flops per
- * launch. Kernels 1-3 need n_levels >= 2 (else AGG_EUNSUPPORTED).
+ * can time it with events (id 0 with 16 and more DoFs per element: x's fixed-point
+ * copy and the product, two launches); agg_kernel_cost gives its algorithmic HBM bytes
+ * (every matrix, block and vector entry that the kernel works on read or written
+ * once: a coupling that is stored for both of its elements once, in face-structured
+ * form twice) and flops per launch (two per entry of the operator, however stored). Kernels 1-3 need n_levels >= 2 (else AGG_EUNSUPPORTED).
  * Id 5 is the level-0 operator evaluated matrix-free in float64 (the
  * operator of agg_operator_apply level -2, built by the first call), the
  * same product as id 0 from quadrature data instead of stored blocks; its

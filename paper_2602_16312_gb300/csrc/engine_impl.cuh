@@ -1769,26 +1769,47 @@ class Engine : public EngineBase {
     persistent = persist_ ? 1 : 0;
   }
 
+  // Bytes of the float64 product's and of the V-cycle's level-0 operator: face-
+  // structured, every coupling in both directions and a neighbour id and a face code
+  // per face; symmetric, each coupling once, a neighbour id, a block id and a
+  // face code per face, and in float64 a scale exponent per row.
+  double face_bytes(double entry) const { return face_entries_ * entry + (double)lev_[0].n * 2 * FaceShape<B>::D * 5.0; }
+  double sym_bytes(double entry, bool scales) const {
+    const double n0 = (double)lev_[0].n, bb = (double)B * B, tri = 0.5 * B * (B + 1);
+    return (n0 * tri + 0.5 * (face_entries_ - n0 * bb)) * entry + n0 * 2 * FaceShape<B>::D * 9.0 + (scales ? n0 * B * 2.0 : 0.0);
+  }
+  double a0_bytes() const { return osym_ ? sym_bytes(8, true) : face_bytes(8); }
+  double l0_bytes() const {
+    if (use_mf0()) return (double)mf_bytes_;
+    return sym_ ? sym_bytes(sizeof(T), std::is_same<T, double>::value) : face_bytes(sizeof(T));
+  }
+  // a fixed-point copy: an entry per DoF, an exponent per element
+  double fx_bytes() const { return (double)lev_[0].n * (B * 8.0 + 4.0); }
+  bool fx_cycle() const { return sym_ && std::is_same<T, double>::value; }
+
   int kernel_cost(int id, double& bytes, double& flops) const override {
     if (id >= 1 && id <= 4 && nlev_ < 2) return AGG_EUNSUPPORTED;
     const double n0 = (double)lev_[0].n, N = n0 * B, bb = (double)B * B;
     const double sT = sizeof(T), sD = sizeof(TD);
     const double bd = (B <= 32) ? (double)SymPad<TD, B>::NP : bb;   // stored smoother entries
-    // face-structured operator: its stored entries and, per face slot, a
-    // neighbour id and a face code
-    const double fidx = n0 * 2 * FaceShape<B>::D * 5.0;
-    const double fe = face_entries_;
+    const double fe = face_entries_;                   // multiply-adds of a product
+    const double fx = fx_cycle() ? fx_bytes() : 0.0;   // a fixed-point copy, read or written
+    const double sc = fx_cycle() ? 2 * N : 0.0;        // scale exponents
     switch (id) {
-      case 0: bytes = fe * 8 + fidx + 2 * N * 8; flops = 2 * fe; break;
+      // (fixed point: x in, its copy out, and the product's read of it; two launches)
+      case 0: bytes = a0_bytes() + 2 * N * 8 + (osym_ ? 2 * fx_bytes() + 2 * N : 0.0); flops = 2 * fe; break;
       case 1:
-        bytes = (use_mf0() ? (double)mf_bytes_ : fe * sT + fidx) + n0 * bd * sD + 5 * N * sT;
+        bytes = l0_bytes() + n0 * bd * sD + 5 * N * sT + 2 * fx + sc + (sc > 0.0 ? 2 * n0 : 0.0);
         flops = 2 * fe + 2 * n0 * bb + 4 * N;
         break;
-      case 2:
-        bytes = (use_mf0() ? (double)mf_bytes_ : fe * sT + fidx) + n0 * bb * sT + 3 * N * sT;
+      case 2:                                           // (fixed point: the copy in place of x)
+        bytes = l0_bytes() + n0 * bb * sT + 3 * N * sT + (fx_cycle() ? fx - N * 8 : 0.0);
         flops = 2 * fe + 2 * n0 * bb + N;
         break;
-      case 3: bytes = n0 * bb * sT + 2 * N * sT + (double)lev_[1].n * B * sT + n0 * 4; flops = 2 * n0 * bb + N; break;
+      case 3:
+        bytes = n0 * bb * sT + 2 * N * sT + (double)lev_[1].n * B * sT + n0 * 4 + fx + sc;
+        flops = 2 * n0 * bb + N;
+        break;
       case 4: iteration_cost(bytes, flops); break;
       case 5:
         if (!mf64_ready_) return AGG_EUNSUPPORTED;
@@ -1801,22 +1822,22 @@ class Engine : public EngineBase {
   }
 
   // Algorithmic bytes and flops of one iteration of the solve body: the
-  // float64 SpMV, the CG update, one V-cycle over every level, the z and p
-  // updates. Each launch reads its operator, block and vector entries once
+  // float64 SpMV, the CG update, one V-cycle over every level, (r, z) and the p
+  // update. Each launch reads its operator, block and vector entries once
   // and writes each output once; flops count two per stored matrix entry
   // used (the matrix-free level-0 operator as its assembled counterpart).
   void iteration_cost(double& bytes, double& flops) const {
     const double bb = (double)B * B, sT = sizeof(T), sD = sizeof(TD);
     const double n0 = (double)lev_[0].n, N = n0 * B, fe = face_entries_;
-    const double fidx = n0 * 2 * FaceShape<B>::D * 5.0;
     const double deg = degree_;
-    // outer CG: SpMV (p in, q out), update (x, r, p, q in; x, r out; the
-    // float32 copy of r and the flexible (r, z_old) read in the reduced-
-    // precision forms), z = V(r) with (r, z), p = z + beta p
+    // outer CG: SpMV (p in, q out; in fixed point p's copy in too), update (x, r, p, q
+    // in; x, r out; the float32 copy of r and the flexible (r, z_old) read in the
+    // reduced-precision forms), (r, z), p = z + beta p (with p's fixed-point copy out)
     const bool lowp = !std::is_same<T, double>::value;
-    bytes = fe * 8 + fidx + 2 * N * 8;
-    bytes += 6 * N * 8 + (lowp ? N * 4 + N * 8 : 0.0);
-    bytes += N * sT + 2 * N * 8 + 3 * N * 8;
+    bytes = a0_bytes() + 2 * N * 8 + (osym_ ? fx_bytes() : 0.0);
+    bytes += 6 * N * 8 + (lowp ? N * 4 + N * sT : 0.0);
+    bytes += N * sT + N * 8;
+    bytes += N * sT + 2 * N * 8 + (osym_ ? fx_bytes() + 2 * N : 0.0);
     flops = 2 * fe + 12 * N;
     for (int l = 0; l < nlev_; ++l) {
       const double nl = (double)lev_[l].n, Nl = nl * B;
@@ -1829,8 +1850,15 @@ class Engine : public EngineBase {
       const double Nc = (double)lev_[l + 1].n * B;
       double op, opf, dinv;
       if (l == 0) {
-        op = use_mf0() ? (double)mf_bytes_ : fe * sT + fidx;
+        op = l0_bytes();
         opf = 2 * fe;
+        if (fx_cycle()) {
+          // 2 deg smoother steps write the iterate's copy, all but the first read one
+          // (and the scales of the block inverses), the restriction reads it in place
+          // of the iterate, the prolongation writes it
+          const double f = fx_bytes(), s = 2 * N + 2 * n0;
+          bytes += 2 * deg * (f + s) + (2 * deg - 1) * f + (f - N * 8) + f + 2 * N;
+        }
         dinv = nl * ((B <= 32) ? (double)SymPad<TD, B>::NP : bb) * sD;
       } else {
         const double nz = (double)nnzb_[l];
