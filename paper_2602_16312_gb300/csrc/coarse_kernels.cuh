@@ -126,11 +126,12 @@ struct RowValues {
 // over the neighbours, so the row is held: loaded before the operator product that
 // precedes its use. Chebyshev step, restriction, us: 250^2 Q2 float64 16.7 -> 12.9,
 // 13.5 -> 10.0; 101^2 Q3 6.9 -> 5.5, 7.0 -> 5.6; Q2 shell 11.2 -> 7.9, 9.6 -> 8.0. Not
-// held: float32 rows of up to 9 entries (PCG on 181^2 Q2 4.7 ms, held 5.3 ms), and
+// held: float32 rows of up to 9 entries (PCG on 181^2 Q2 4.7 ms, held 5.3 ms), float64
+// rows of 8 (V-cycle of Q1 cubes of 20^3 and 40^3: 359 and 615 us, held 385 and 646), and
 // 64-DoF rows, which would take 64 or 128 registers.
 template <typename T, typename TD, int B, bool TR>
 struct RowBlock {
-  static constexpr bool kHeld = (B <= 32) && (B > 9 || std::is_same<T, double>::value);
+  static constexpr bool kHeld = (B <= 32) && (B > 9 || (B != 8 && std::is_same<T, double>::value));
   TD v[kHeld ? B : 1];
   static __device__ __forceinline__ TD at(const TD* __restrict__ M, const RowOf<B>& L, int c) {
     return M[(size_t)L.unit * B * B + (TR ? L.r * B + c : c * B + L.r)];
