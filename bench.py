@@ -30,8 +30,8 @@ METRIC = "time-steps/s and MDoF/s of MG-PCG at 1e-8 rel. residual; % of HBM peak
 UNIT = "time-steps/s"
 
 
-def kernel_names(B, form, fine):
-    """Level-0 kernels by id for B DoFs per element (symmetric conductivities):
+def kernel_names(n, B, form, fine):
+    """Level-0 kernels by id for n elements of B DoFs (symmetric conductivities):
     the float64 product of the outer CG and the Chebyshev step."""
     sym = "k_sym" if B > 32 else "k_symw"
     product = f"{sym}<double> (symmetric blocks in fixed point)" if B >= 16 else "k_spmv<double> (face-structured blocks)"
@@ -39,8 +39,10 @@ def kernel_names(B, form, fine):
         step = "k_mf_cheb (matrix-free float32 operator)"
     elif form == "f64":
         step = f"{sym}<double> (symmetric blocks in fixed point)" if B >= 9 else "k_cheb<double> (face-structured blocks)"
-    else:
+    elif B >= 16 or n <= (30000 if B == 4 else 65536):
         step = f"{sym}<float> (symmetric blocks)"
+    else:
+        step = "k_cheb<float> (face-structured blocks)"
     return {0: f"fine float64 SpMV, outer CG: {product}", 1: f"fine Chebyshev block-Jacobi step: {step}"}
 
 
@@ -470,7 +472,7 @@ def run_ours(args, rank, world):
                        "note": "bytes of one iteration x (iterations + 1 per step) / timed region"})
     except aggmg.AggError:
         pass
-    names = kernel_names((wl.degree + 1) ** wl.mesh.dim, args.form, args.fine)
+    names = kernel_names(wl.mesh.n_elements, (wl.degree + 1) ** wl.mesh.dim, args.form, args.fine)
     fp64_pipe = [k for k in names if "double" in names[k] and "fixed point" not in names[k]]
     if kid in fp64_pipe:
         roof = {"bound": "alu", "achieved": kflops / t_k / 1e9, "peak": FP64_PEAK_GFLOPS, "unit": "GFLOP/s"}

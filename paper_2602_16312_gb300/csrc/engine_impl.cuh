@@ -177,10 +177,18 @@ class Engine : public EngineBase {
   // up to 9 DoFs keep the face-structured float64 product (512^2 Q2 square: 126
   // against 143 us; 16 DoFs: 20 against 60 us; 27: 242 against 430 us on the
   // 40^3 cube; 64: 125 against 560 us on 18^3), of up to 8 the float64 V-cycle
-  // too. An unsymmetric assembly (unsymmetric conductivity tensors) keeps the
+  // too. Float32 V-cycles with up to 9 DoFs take the symmetric blocks up to kSymMost
+  // elements: one thread per element leaves a small mesh's SMs idle (Q2 square, 100^2:
+  // V-cycle 224 us, symmetric 200; Q1 cube, 20^3: 214, 179), but once the mesh fills
+  // the GPU its 16-byte chunks read short blocks faster than the rings of k_symw do
+  // (Q2 square, 256^2: 297 and 296 us; 362^2: 424, 465; Q1 square, 150^2: 166, 162;
+  // 200^2: 169, 175; 500^2: 259, 317; Q1 cube, 40^3: 355, 342; 64^3: 863, 946). With 16
+  // and more DoFs symmetric is faster at every size (Q3 square 400^2: 1,143, 902 us;
+  // Q2 cube 56^3: 3,244, 2,759). An unsymmetric assembly (unsymmetric conductivity tensors) keeps the
   // face-structured form throughout.
   static constexpr bool kOuterSym = (B >= 16);
   static constexpr bool kCycleSym = std::is_same<T, float>::value || (B >= 9);
+  static constexpr int64_t kSymMost = (B >= 16 || std::is_same<T, double>::value) ? INT64_MAX : (B == 4 ? 30000 : 65536);
   bool osym_ = false, sym_ = false;
   using SymDinv = typename SymSmem<T, TD, B, SYM_CHEB, 2>::SD;
   using SymP = typename SymSmem<T, TD, B, SYM_RESTRICT, 0>::SD;
@@ -1341,7 +1349,7 @@ class Engine : public EngineBase {
       int kA = 0;
       const bool fixed = asym <= kAsymF64 && (kOuterSym || (kCycleSym && kDouble)) && sym_scales(fb, m.ne, sc, kA);
       osym_ = fixed && kOuterSym;
-      sym_ = kCycleSym && assembled && (kDouble ? fixed : asym <= kAsymF32);
+      sym_ = kCycleSym && assembled && (kDouble ? fixed : asym <= kAsymF32 && m.ne <= kSymMost);
       if (kDouble) sym_ = sym_ && (nlev_ == 1 || block_scales(h.lev[0].Dinv, m.ne, ds, dk));
       if (osym_ || (sym_ && kDouble)) {
         if ((rc = upload_sym<double>(fb, m.ne, sc, kA, A0s_, err))) return rc;
