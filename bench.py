@@ -36,7 +36,7 @@ def kernel_names(n, B, form, fine):
     sym = "k_sym" if B > 32 else "k_symw"
     product = f"{sym}<double> (symmetric blocks in fixed point)" if B >= 16 else "k_spmv<double> (face-structured blocks)"
     if fine == "mf":
-        step = "k_mf_cheb (matrix-free float32 operator)"
+        step = f"{'k_mf_cheb' if B >= 9 else 'k_cheb'} (matrix-free float32 operator)"
     elif form == "f64":
         step = f"{sym}<double> (symmetric blocks in fixed point)" if B >= 9 else "k_cheb<double> (face-structured blocks)"
     elif B >= 16 or n <= (30000 if B == 4 else 65536):

@@ -1017,10 +1017,17 @@ class Engine : public EngineBase {
     return xo;
   }
 
+  // Matrix-free level 0 through the staged kernels of mf_kernels.cuh: from 9 DoFs on.
+  // With 4 and 8 the lanes of a straight load lie 16 or 32 bytes apart, and the stages
+  // only add latency (Chebyshev step, residual + restriction of Q1 cubes, staged and
+  // straight, us: 24^3 24.8, 22.7 and 22.7, 20.7; 64^3 141, 134 and 131, 121; V-cycle of Q1
+  // squares: 16^2 83 and 79, 300^2 212 and 205, 512^2 317 and 317).
+  template <typename Op>
+  static constexpr bool kStagedMf = kMf && B >= 9 && std::is_same<Op, MfOpT>::value;
   // Chebyshev step (KIND as in k_cheb) on level v with operator op
   template <int KIND, typename Op>
   void cheb_step(const Op& op, Lev& v, const T* xo, T* xn, T c1, T c2, cudaStream_t s, const CGState* st) {
-    if constexpr (kMf && std::is_same<Op, MfOpT>::value)
+    if constexpr (kStagedMf<Op>)
       k_mf_cheb<T, TD, B, KIND, Op><<<bgrid(0, v.nsl), NTB, 0, s>>>(op, v.Dinv, v.rhs, xo, xn, v.d, c1, c2, v.nsl, st);
     else
       k_cheb<T, TD, B, KIND, Op><<<bgrid(0, v.nsl), NTB, 0, s>>>(op, v.Dinv, v.rhs, xo, xn, v.d, c1, c2, v.nsl, st);
@@ -1028,7 +1035,7 @@ class Engine : public EngineBase {
 
   template <typename Op>
   void resid_restrict(const Op& op, Lev& v, const T* x, cudaStream_t s, const CGState* st) {
-    if constexpr (kMf && std::is_same<Op, MfOpT>::value)
+    if constexpr (kStagedMf<Op>)
       k_mf_restrict<T, B, Op><<<bgrid(0, v.nsl), NTB, 0, s>>>(op, v.P, v.rhs, x, v.S, v.nsl, st);
     else
       k_resid_restrict<T, B, Op><<<bgrid(0, v.nsl), NTB, 0, s>>>(op, v.P, v.rhs, x, v.S, st);
