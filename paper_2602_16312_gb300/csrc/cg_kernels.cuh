@@ -12,7 +12,7 @@
 
 namespace aggmg {
 
-enum { TK_PQ = 0, TK_R = 1, TK_Z = 2, TK_R0 = 3 };
+enum { TK_R = 0, TK_R0 = 1 };
 
 // Loop control of the WHILE node, launched after the PCG set-up and at the end
 // of every iteration: ends the loop once the solve is done, and after

@@ -164,7 +164,7 @@ class Engine : public EngineBase {
       return AGG_OK;
     }
   }
-  // level 0 in face-structured form: float64 for the outer CG, and the
+  // level 0 in face-structured form (where not symmetric): float64 for the outer CG, and the
   // V-cycle precision copy for the assembled smoother (the same data when
   // the V-cycle is float64)
   using A0Op = FaceOp<double, B>;
@@ -655,9 +655,12 @@ class Engine : public EngineBase {
     return AGG_OK;
   }
 
+  // index of a k_sym kernel: the outer product's, then the V-cycle's
   static constexpr int sym_slot(bool outer, int op, int kind) {
     return op == SYM_SPMV ? (outer ? kind : 3) : (op == SYM_CHEB ? 4 + kind : 7);
   }
+  static constexpr int kOuter = sym_slot(true, SYM_SPMV, 0), kCycle = sym_slot(false, SYM_SPMV, 0);
+  static constexpr int kCheb = sym_slot(false, SYM_CHEB, 0), kRestrict = sym_slot(false, SYM_RESTRICT, 0);
   // Shared-memory limit and resident blocks of one k_sym kernel
   template <typename TT, typename TDD, int OP, int KIND>
   int prepare_sym(int slot, std::string& err) {
@@ -682,17 +685,17 @@ class Engine : public EngineBase {
   int prepare_sym_kernels(bool matrix_free, std::string& err) {
     int rc;
     if (osym_) {
-      if ((rc = prepare_sym<double, double, SYM_SPMV, 0>(0, err))) return rc;
-      if ((rc = prepare_sym<double, double, SYM_SPMV, 1>(1, err))) return rc;
-      if ((rc = prepare_sym<double, double, SYM_SPMV, 2>(2, err))) return rc;
+      if ((rc = prepare_sym<double, double, SYM_SPMV, 0>(kOuter, err))) return rc;
+      if ((rc = prepare_sym<double, double, SYM_SPMV, 1>(kOuter + 1, err))) return rc;
+      if ((rc = prepare_sym<double, double, SYM_SPMV, 2>(kOuter + 2, err))) return rc;
     }
-    if (matrix_free && B == 64 && (rc = prepare_sym<T, TD, SYM_CHEB, 0>(4, err))) return rc;
+    if (matrix_free && B == 64 && (rc = prepare_sym<T, TD, SYM_CHEB, 0>(kCheb, err))) return rc;
     if (!sym_) return AGG_OK;
-    if ((rc = prepare_sym<T, TD, SYM_SPMV, 0>(3, err))) return rc;
-    if ((rc = prepare_sym<T, TD, SYM_CHEB, 0>(4, err))) return rc;
-    if ((rc = prepare_sym<T, TD, SYM_CHEB, 1>(5, err))) return rc;
-    if ((rc = prepare_sym<T, TD, SYM_CHEB, 2>(6, err))) return rc;
-    return prepare_sym<T, TD, SYM_RESTRICT, 0>(7, err);
+    if ((rc = prepare_sym<T, TD, SYM_SPMV, 0>(kCycle, err))) return rc;
+    if ((rc = prepare_sym<T, TD, SYM_CHEB, 0>(kCheb, err))) return rc;
+    if ((rc = prepare_sym<T, TD, SYM_CHEB, 1>(kCheb + 1, err))) return rc;
+    if ((rc = prepare_sym<T, TD, SYM_CHEB, 2>(kCheb + 2, err))) return rc;
+    return prepare_sym<T, TD, SYM_RESTRICT, 0>(kRestrict, err);
   }
   template <int OP, int KIND, typename TT, typename TDD>
   int64_t sym_grid(int slot, int64_t n) const {
@@ -700,12 +703,11 @@ class Engine : public EngineBase {
       using M = SymRing<TT, TDD, BS, OP, KIND>;
       return std::min<int64_t>(cdiv(n, M::EPW * M::NWARP), sym_blocks_[slot]);
     } else {
-      return std::min<int64_t>(cdiv(n, SymSmem<TT, TDD, B, OP, KIND>::U), sym_blocks_[slot]);
+      return std::min<int64_t>(n, sym_blocks_[slot]);
     }
   }
-  // One k_sym launch: a block per U elements, at most the resident ones (each
-  // then loops over the element groups, a group per step, so that the groups
-  // in flight stay neighbours and share face blocks through the L2).
+  // One launch: at most the resident blocks (each then loops over the elements, so
+  // that those in flight stay neighbours and share face blocks through the L2).
   template <int OP, int KIND, typename TT, typename TDD, typename SD>
   void launch_sym(int slot, const SymView<TT, B>& A, SymBlk<SD> ext, SymVec<TT> xv, const TT* rhs, const TT* x, TT* out,
                   TT* d, FxVec fo, TT c1, TT c2, CGState* st, cudaStream_t s) {
@@ -725,7 +727,7 @@ class Engine : public EngineBase {
   void spmv0(const double* x, const double* rhs, double* y, FxVec fx, CGState* st, cudaStream_t s) {
     if (osym_) {
       if (MODE != 2) make_fx(x, fx, st, s);          // MODE 2: written with p
-      launch_sym<SYM_SPMV, MODE, double, double>(MODE, A0s_, SymBlk<double>{}, SymVec<double>{fx.X, fx.E}, rhs, x, y,
+      launch_sym<SYM_SPMV, MODE, double, double>(kOuter + MODE, A0s_, SymBlk<double>{}, SymVec<double>{fx.X, fx.E}, rhs, x, y,
                                                  nullptr, FxVec{}, 0.0, 0.0, st, s);
     }
     else
@@ -735,10 +737,10 @@ class Engine : public EngineBase {
   // symmetric blocks in the V-cycle precision
   template <int KIND>
   void sym_cheb(Lev& v, const T* xo, T* xn, T c1, T c2, cudaStream_t s, CGState* st) {
-    launch_sym<SYM_CHEB, KIND, T, TD>(4 + KIND, fs_, (kStream || KIND == 0) ? sdinv_ : sdinvm_, sym_vec(xo), v.rhs, xo, xn, v.d, fx_of(xn), c1, c2, st, s);
+    launch_sym<SYM_CHEB, KIND, T, TD>(kCheb + KIND, fs_, (kStream || KIND == 0) ? sdinv_ : sdinvm_, sym_vec(xo), v.rhs, xo, xn, v.d, fx_of(xn), c1, c2, st, s);
   }
   void sym_restrict(Lev& v, const T* x, cudaStream_t s, CGState* st) {
-    launch_sym<SYM_RESTRICT, 0, T, TD>(7, fs_, sPT_, sym_vec(x), v.rhs, x, v.S, nullptr, FxVec{}, T(0), T(0), st, s);
+    launch_sym<SYM_RESTRICT, 0, T, TD>(kRestrict, fs_, sPT_, sym_vec(x), v.rhs, x, v.S, nullptr, FxVec{}, T(0), T(0), st, s);
   }
   void sym_prolong(Lev& v, const T* ec, T* x, cudaStream_t s, CGState* st) {
     k_sym_prolong<T, B><<<cdiv(v.n, SymRows<B>::U), SymRows<B>::NT, 0, s>>>(sP_, v.parent, ec, x, fs_.sc, fx_of(x).X,
@@ -1084,10 +1086,10 @@ class Engine : public EngineBase {
   // blocks of the float64 product that writes (p, q)
   int pq_blocks() const {
     if (!osym_) return (int)bgrid(0, lev_[0].nsl);
-    return (int)sym_grid<SYM_SPMV, 2, double, double>(2, lev_[0].n);
+    return (int)sym_grid<SYM_SPMV, 2, double, double>(kOuter + 2, lev_[0].n);
   }
   // the buffer that holds the V-cycle's result: 2 degree - 1 swaps of the iterates
-  T* vcycle_result() const { return nlev_ == 1 ? lev_[0].xa : (((2 * degree_ - 1) & 1) ? lev_[0].xb : lev_[0].xa); }
+  T* vcycle_result() const { return nlev_ == 1 ? lev_[0].xa : lev_[0].xb; }
 
   // z = V(r), beta, p. In the iteration body the float32 cast of r and the
   // flexible-beta product (r, z_old) come fused in k_cg_update.
@@ -1297,7 +1299,7 @@ class Engine : public EngineBase {
       if ((rc = upload(&v.perm, hl.perm.data(), hl.perm.size(), err))) return rc;
       const bool coarsest = (l == nlev_ - 1);
       if (!coarsest) {
-        // level 0 keeps its slot structure only (its operator is face-structured)
+        // level 0 keeps its slot structure only (its operator: below)
         if ((rc = upload_sell<T>(hl.A, v.nsl, &v.slice_ptr, &v.cols, &v.vals, err, l > 0))) return rc;
         if (l > 0 || fine_operator == 1) {        // (level 0 else: below, with its operator)
           if ((rc = upload_dinv(hl.Dinv, hl.n, v.nsl, &v.Dinv, err))) return rc;
@@ -1340,7 +1342,7 @@ class Engine : public EngineBase {
       }
       if ((rc = dalloc(&v.xa, v.nvec, err))) return rc;
     }
-    // face-structured level-0 operators: float64 (outer CG) and, for the
+    // level-0 operators, symmetric or face-structured: float64 (outer CG) and, for the
     // assembled smoother, the V-cycle precision
     {
       FaceBlocks fb;
@@ -1549,7 +1551,7 @@ class Engine : public EngineBase {
         k_op_apply<T, B, MfOpT><<<bgrid(0, v.nsl), NTB, 0, s>>>(mfop_, v.xa, v.xb);
       else if (sym_) {
         if constexpr (std::is_same<T, double>::value) make_fx(v.xa, fxa_, nullptr, s);
-        launch_sym<SYM_SPMV, 0, T, TD>(3, fs_, SymBlk<T>{}, sym_vec(v.xa), nullptr, v.xa, v.xb, nullptr,
+        launch_sym<SYM_SPMV, 0, T, TD>(kCycle, fs_, SymBlk<T>{}, sym_vec(v.xa), nullptr, v.xa, v.xb, nullptr,
                                        FxVec{}, T(0), T(0), nullptr, s);
       } else
         k_op_apply<T, B, L0Op><<<bgrid(0, v.nsl), NTB, 0, s>>>(fop_, v.xa, v.xb);

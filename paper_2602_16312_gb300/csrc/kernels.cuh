@@ -34,7 +34,7 @@ struct CGState {
   int iter, done, status, max_it, flexible, use_cond;
   int guard;                  // WHILE-body executions of this solve (hard stop)
   unsigned long long cond;    // cudaGraphConditionalHandle of the WHILE node
-  unsigned ticket[4];         // last-block tickets, one per reduction kind
+  unsigned ticket[2];         // last-block tickets, one per reduction kind
 };
 
 // Grid-wide barrier state of the persistent coarse-level kernel: arrival

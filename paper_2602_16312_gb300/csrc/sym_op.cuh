@@ -285,7 +285,7 @@ struct SymSmem {
   using L = SymLay<ST, B>;
   static constexpr bool kFx = std::is_same<T, double>::value;
   static constexpr bool kProduct = !(OP == SYM_CHEB && KIND == 0);
-  static constexpr int U = 1, G = kProduct ? 4 : 1;
+  static constexpr int G = kProduct ? 4 : 1;
   // with an operator product, the block inverse or P^T is read from memory, column
   // by column and a group's columns per thread, instead of shared memory, where only
   // one stage would fit: adjoint step of the 18^3 Q3 cube 21.3 -> 19.5 ms
@@ -294,15 +294,15 @@ struct SymSmem {
   static constexpr int KX = (OP == SYM_CHEB && !kProduct) ? SymLay<SD, B>::KD : 0;
   static constexpr int KXM = SymLay<SD, B>::KP, CPG = B / G;   // block entries in memory, columns per group
   static constexpr int NX = kProduct ? 1 + S::NFACE : 0;
-  static constexpr int NTH = round_to(U * B * G, 32);
-  static constexpr size_t kBlk = (size_t)U * KE * sizeof(ST);
-  static constexpr size_t kExt = (size_t)U * KX * sizeof(SD);
-  static constexpr size_t kXs = round_to(U * NX * S::BX * (int)sizeof(SX), 16);
-  static constexpr size_t kEx = kFx ? round_to(U * NX * 4, 16) : 0;
+  static constexpr int NTH = round_to(B * G, 32);
+  static constexpr size_t kBlk = (size_t)KE * sizeof(ST);
+  static constexpr size_t kExt = (size_t)KX * sizeof(SD);
+  static constexpr size_t kXs = round_to(NX * S::BX * (int)sizeof(SX), 16);
+  static constexpr size_t kEx = kFx ? round_to(NX * 4, 16) : 0;
   static constexpr size_t kStage = kBlk + kExt + kXs + kEx;
-  static constexpr size_t kPart = kProduct ? round_to(U * S::NFACE * B * (int)sizeof(Sum), 16) : 0;
-  static constexpr size_t kRed = round_to((G - 1) * U * B * (int)sizeof(Sum), 16);
-  static constexpr size_t kTs = (OP == SYM_SPMV) ? 0 : round_to(U * S::BX * (int)sizeof(SX), 16);
+  static constexpr size_t kPart = kProduct ? round_to(S::NFACE * B * (int)sizeof(Sum), 16) : 0;
+  static constexpr size_t kRed = round_to((G - 1) * B * (int)sizeof(Sum), 16);
+  static constexpr size_t kTs = (OP == SYM_SPMV) ? 0 : round_to(S::BX * (int)sizeof(SX), 16);
   static constexpr size_t kRest = kPart + kRed + kTs + round_to((1 + 2 * (1 + S::NFACE)) * (int)sizeof(int), 16);
   static constexpr int kStages = (2 * kStage + kRest <= 225 * 1024) ? 2 : 1;
   static constexpr size_t bytes = kStages * kStage + kRest;
@@ -437,7 +437,7 @@ __device__ __forceinline__ void fx_store(double v, bool active, int slot, int64_
 // (ext: column by column, LDP apart; KIND 0 of SYM_CHEB: packed triangles, which
 // without a product leave room for two stages: 64 DoFs, 24^3, 108 -> 22 us)
 // x: the vector itself (own values); xv: what the products read. The blocks of
-// a launch loop over tiles of U elements, so that the tiles in flight are
+// a launch loop over the elements, so that the elements in flight are
 // neighbours and share face blocks through the L2.
 // A face costs a row NF products with the neighbour's face DoFs, and its NF face
 // rows BO more; those are dealt to all B threads of the element (B / NF partial
@@ -458,11 +458,11 @@ static __global__ void __launch_bounds__(SymSmem<T, TD, B, OP, KIND>::NTH)
   using XSum = typename XAcc::Sum;
   using L = typename M::L;
   constexpr bool kFxExt = M::kFx && OP == SYM_CHEB;   // the block inverses are in fixed point
-  constexpr int U = M::U, G = M::G, NFACE = S::NFACE, BX = S::BX, NF = S::NF, BO = S::BO, N = S::N;
+  constexpr int G = M::G, NFACE = S::NFACE, BX = S::BX, NF = S::NF, BO = S::BO, N = S::N;
   constexpr bool kFx = M::kFx;
   constexpr int kShare = BO / N;                      // off-face terms of a face row per thread
   constexpr int FPG = (G == 1) ? NFACE : (NFACE + G - 2) / (G - 1);   // faces per group
-  static_assert(U == 1 && B == 64, "two warps hold an element's rows");
+  static_assert(B == 64, "two warps hold an element's rows");
   if (st && st->done) return;
   extern __shared__ __align__(16) unsigned char sym_sm[];
   Sum* spart = reinterpret_cast<Sum*>(sym_sm + M::kStages * M::kStage);
@@ -471,104 +471,94 @@ static __global__ void __launch_bounds__(SymSmem<T, TD, B, OP, KIND>::NTH)
   int* smax = reinterpret_cast<int*>(sym_sm + M::kStages * M::kStage + M::kPart + M::kRed + M::kTs);
 
   const int tid = threadIdx.x;
-  const int g = (G == 1) ? 0 : tid / (U * B);
-  const int slot = (tid - g * U * B) / B;
-  const int r = tid - g * U * B - slot * B;
-  const bool mine = (G == 1) ? tid < U * B : g < G;
-  const int64_t ntiles = (A.n + U - 1) / U;
+  const int g = tid / B, r = tid - g * B;
   double part = 0.0;
   // the group's k-th face
   auto face_of = [&](int k) { return G == 1 ? k : g - 1 + k * (G - 1); };
 
   int2 info[FPG];
   int8_t code[FPG];
-  auto load_info = [&](int64_t tile) {
+  auto load_info = [&](int64_t unit) {
     if constexpr (M::kProduct) {
-      const int64_t unit = tile * U + slot;
 #pragma unroll
       for (int k = 0; k < FPG; ++k) {
         info[k] = make_int2(-1, 0);
         code[k] = 0;
-        if (mine && unit < A.n && (G == 1 || g > 0) && face_of(k) < NFACE) {
+        if ((G == 1 || g > 0) && face_of(k) < NFACE) {
           info[k] = A.info[unit * NFACE + face_of(k)];
           code[k] = A.code[unit * NFACE + face_of(k)];
         }
       }
     }
   };
-  // copies of a tile into stage `sg` (its face info has been loaded)
-  auto issue = [&](int64_t tile, int sg) {
-    const int64_t unit = tile * U + slot;
-    if (mine && unit < A.n) {
-      unsigned char* base = sym_sm + sg * M::kStage;
-      ST* eb = reinterpret_cast<ST*>(base) + slot * M::KE;
-      SX* ex = reinterpret_cast<SX*>(base + M::kBlk + M::kExt) + slot * M::NX * BX;
-      int* ee = reinterpret_cast<int*>(base + M::kBlk + M::kExt + M::kXs) + slot * M::NX;
-      if constexpr (M::KX > 0) {
-        constexpr int QD = 16 / (int)sizeof(SD);
-        const SD* src = ext.v + (size_t)unit * M::KX;
-        SD* dst = reinterpret_cast<SD*>(base + M::kBlk) + slot * M::KX;
-        for (int p = r + B * g; p < M::KX / QD; p += B * G) cp_async16(dst + p * QD, src + p * QD);
+  // copies of an element into stage `sg` (its face info has been loaded)
+  auto issue = [&](int64_t unit, int sg) {
+    unsigned char* base = sym_sm + sg * M::kStage;
+    ST* eb = reinterpret_cast<ST*>(base);
+    SX* ex = reinterpret_cast<SX*>(base + M::kBlk + M::kExt);
+    int* ee = reinterpret_cast<int*>(base + M::kBlk + M::kExt + M::kXs);
+    if constexpr (M::KX > 0) {
+      constexpr int QD = 16 / (int)sizeof(SD);
+      const SD* src = ext.v + (size_t)unit * M::KX;
+      SD* dst = reinterpret_cast<SD*>(base + M::kBlk);
+      for (int p = r + B * g; p < M::KX / QD; p += B * G) cp_async16(dst + p * QD, src + p * QD);
+    }
+    if constexpr (M::kProduct) {
+      if (g == 0) {
+        const ST* src = A.diag + (size_t)unit * L::KD;
+#pragma unroll 4
+        for (int p = r; p < L::KD / L::Q; p += B) cp_async16(eb + p * L::Q, src + p * L::Q);
+        cp_async_x(ex + r, xv.X + (size_t)unit * B + r);
+        if (kFx && r == 0) cp_async4(ee, xv.E + unit);
       }
-      if constexpr (M::kProduct) {
-        if (g == 0) {
-          const ST* src = A.diag + (size_t)unit * L::KD;
-#pragma unroll 4
-          for (int p = r; p < L::KD / L::Q; p += B) cp_async16(eb + p * L::Q, src + p * L::Q);
-          cp_async_x(ex + r, xv.X + (size_t)unit * B + r);
-          if (kFx && r == 0) cp_async4(ee, xv.E + unit);
-        }
 #pragma unroll
-        for (int k = 0; k < FPG; ++k) {
-          const int f = face_of(k);
-          if (info[k].x < 0) {
-            if (kFx && r == 0 && (G == 1 || g > 0)) ee[f + 1] = kFxNone;
-            continue;
-          }
-          const ST* src = A.face + (size_t)info[k].y * L::KB;
-          ST* dst = eb + L::KD + f * L::KB;
-#pragma unroll 4
-          for (int p = r; p < L::KB / L::Q; p += B) cp_async16(dst + p * L::Q, src + p * L::Q);
-          bool on;
-          int pos = face_first<B>(code[k], r, on);
-          if (!on) pos += S::XO - NF;
-          cp_async_x(ex + (f + 1) * BX + pos, xv.X + (size_t)info[k].x * B + r);
-          if (kFx && r == 0) cp_async4(ee + f + 1, xv.E + info[k].x);
+      for (int k = 0; k < FPG; ++k) {
+        const int f = face_of(k);
+        if (info[k].x < 0) {
+          if (kFx && r == 0 && (G == 1 || g > 0)) ee[f + 1] = kFxNone;
+          continue;
         }
+        const ST* src = A.face + (size_t)info[k].y * L::KB;
+        ST* dst = eb + L::KD + f * L::KB;
+#pragma unroll 4
+        for (int p = r; p < L::KB / L::Q; p += B) cp_async16(dst + p * L::Q, src + p * L::Q);
+        bool on;
+        int pos = face_first<B>(code[k], r, on);
+        if (!on) pos += S::XO - NF;
+        cp_async_x(ex + (f + 1) * BX + pos, xv.X + (size_t)info[k].x * B + r);
+        if (kFx && r == 0) cp_async4(ee + f + 1, xv.E + info[k].x);
       }
     }
   };
 
-  int64_t tile = blockIdx.x;
+  int64_t unit = blockIdx.x;
   unsigned mask = 0, next_mask = 0;                   // the group's faces with a neighbour (and its orientation)
-  auto face_mask = [&](int64_t t) {
+  auto face_mask = [&](int64_t u) {
     unsigned m = 0;
     if constexpr (M::kProduct) {
 #pragma unroll
       for (int k = 0; k < FPG; ++k)
-        if (info[k].x >= 0) m |= (info[k].x < t * U + slot ? 3u : 1u) << (2 * k);
+        if (info[k].x >= 0) m |= (info[k].x < u ? 3u : 1u) << (2 * k);
     }
     return m;
   };
   int sg = 0;
-  if (tile < ntiles) {
-    load_info(tile);
-    issue(tile, 0);
-    mask = face_mask(tile);
-    if (M::kStages == 2 && tile + gridDim.x < ntiles) load_info(tile + gridDim.x);
+  if (unit < A.n) {
+    load_info(unit);
+    issue(unit, 0);
+    mask = face_mask(unit);
+    if (M::kStages == 2 && unit + gridDim.x < A.n) load_info(unit + gridDim.x);
   }
   asm volatile("cp.async.commit_group;" ::: "memory");
-  for (; tile < ntiles; tile += gridDim.x) {
-    const int64_t unit = tile * U + slot;
-    const bool active = mine && unit < A.n;
-    const bool lead = active && g == 0;
+  for (; unit < A.n; unit += gridDim.x) {
+    const bool lead = g == 0;
     const size_t o = (size_t)unit * B + r;
-    const int64_t next = tile + gridDim.x;
+    const int64_t next = unit + gridDim.x;
     if constexpr (M::kStages == 2) {
-      if (next < ntiles) {
+      if (next < A.n) {
         issue(next, sg ^ 1);
         next_mask = face_mask(next);
-        if (next + gridDim.x < ntiles) load_info(next + gridDim.x);
+        if (next + gridDim.x < A.n) load_info(next + gridDim.x);
       }
       asm volatile("cp.async.commit_group;\n\tcp.async.wait_group 1;" ::: "memory");
     } else {
@@ -577,19 +567,17 @@ static __global__ void __launch_bounds__(SymSmem<T, TD, B, OP, KIND>::NTH)
     if (OP != SYM_SPMV && tid == 0) smax[0] = kFxNone;
     __syncthreads();
     unsigned char* base = sym_sm + sg * M::kStage;
-    const ST* eb = reinterpret_cast<ST*>(base) + slot * M::KE;
-    const SD* sext = reinterpret_cast<SD*>(base + M::kBlk) + slot * M::KX;
-    const SX* ex = reinterpret_cast<SX*>(base + M::kBlk + M::kExt) + slot * M::NX * BX;
-    const int* ee = reinterpret_cast<int*>(base + M::kBlk + M::kExt + M::kXs) + slot * M::NX;
+    const ST* eb = reinterpret_cast<ST*>(base);
+    const SD* sext = reinterpret_cast<SD*>(base + M::kBlk);
+    const SX* ex = reinterpret_cast<SX*>(base + M::kBlk + M::kExt);
+    const int* ee = reinterpret_cast<int*>(base + M::kBlk + M::kExt + M::kXs);
     T own = T(0), rh = T(0), dv = T(0);               // loaded ahead of their use
     int ti = 0, ui = 0;                               // scale exponents of the row and of its block inverse
     SD ev[M::kExtMem ? M::CPG : 1];
     if constexpr (M::kExtMem) {
-      if (active) {
-        const SD* e = ext.v + (size_t)unit * M::KXM + (size_t)(g * M::CPG) * S::LDP + r;
+      const SD* e = ext.v + (size_t)unit * M::KXM + (size_t)(g * M::CPG) * S::LDP + r;
 #pragma unroll
-        for (int c = 0; c < M::CPG; ++c) ev[c] = e[c * S::LDP];
-      }
+      for (int c = 0; c < M::CPG; ++c) ev[c] = e[c * S::LDP];
     }
     if (lead) {
       if (M::kProduct && (KIND == 2 || OP == SYM_CHEB)) own = x[o];
@@ -613,52 +601,50 @@ static __global__ void __launch_bounds__(SymSmem<T, TD, B, OP, KIND>::NTH)
           lo = min(lo, ee[k]);
         }
       }
-      if (active) {
-        if (g == 0) {
-          Acc acc;
-          sym_tri<T, B>(eb, r, ex, acc);
-          sum = sum_shift(acc.sum(), kFx ? E - ee[0] : 0);
-        }
-        Sum* pp = spart + slot * NFACE * B + r;
-        constexpr int kFaceUnroll = (S::D == 2) ? FPG : 1;
-#pragma unroll kFaceUnroll
-        for (int k = 0; k < FPG; ++k) {
-          if (G > 1 && g == 0) break;
-          const int f = face_of(k);
-          const unsigned m = mask >> (2 * k);
-          if (!(m & 1)) {
-            pp[f * B] = Sum(0);
-            continue;
-          }
-          const bool tr = m & 2;                      // the block is the neighbour's: row of K^T
-          bool on;
-          const int pos = face_first<B>(f, r, on);
-          const ST* F = eb + L::KD + f * L::KB;
-          const ST* Gb = F + NF * S::LDF;
-          const SX* xf = ex + (f + 1) * BX;
-          const int sh = kFx ? E - ee[f + 1] : 0;
-          Acc acc;
-          sym_dot<T, NF>(tr ? (on ? F + pos * S::LDF : Gb + (pos - NF) * S::LDG) : F + pos, tr ? 1 : S::LDF, xf, acc);
-          sum += sum_shift(acc.sum(), sh);
-          // this thread's share of face row j's off-face terms
-          const int j = r % NF, a0 = r / NF * kShare;
-          Acc pa;
-          sym_dot_any<T, kShare>(tr ? F + j * S::LDF + NF + a0 : Gb + a0 * S::LDG + j, tr ? 1 : S::LDG, xf + S::XO + a0, pa);
-          pp[f * B] = sum_shift(pa.sum(), sh);
-        }
-        if (G > 1 && g > 0) sred[(g - 1) * U * B + slot * B + r] = sum;
+      if (g == 0) {
+        Acc acc;
+        sym_tri<T, B>(eb, r, ex, acc);
+        sum = sum_shift(acc.sum(), kFx ? E - ee[0] : 0);
       }
+      Sum* pp = spart + r;
+      constexpr int kFaceUnroll = (S::D == 2) ? FPG : 1;
+#pragma unroll kFaceUnroll
+      for (int k = 0; k < FPG; ++k) {
+        if (G > 1 && g == 0) break;
+        const int f = face_of(k);
+        const unsigned m = mask >> (2 * k);
+        if (!(m & 1)) {
+          pp[f * B] = Sum(0);
+          continue;
+        }
+        const bool tr = m & 2;                        // the block is the neighbour's: row of K^T
+        bool on;
+        const int pos = face_first<B>(f, r, on);
+        const ST* F = eb + L::KD + f * L::KB;
+        const ST* Gb = F + NF * S::LDF;
+        const SX* xf = ex + (f + 1) * BX;
+        const int sh = kFx ? E - ee[f + 1] : 0;
+        Acc acc;
+        sym_dot<T, NF>(tr ? (on ? F + pos * S::LDF : Gb + (pos - NF) * S::LDG) : F + pos, tr ? 1 : S::LDF, xf, acc);
+        sum += sum_shift(acc.sum(), sh);
+        // this thread's share of face row j's off-face terms
+        const int j = r % NF, a0 = r / NF * kShare;
+        Acc pa;
+        sym_dot_any<T, kShare>(tr ? F + j * S::LDF + NF + a0 : Gb + a0 * S::LDG + j, tr ? 1 : S::LDG, xf + S::XO + a0, pa);
+        pp[f * B] = sum_shift(pa.sum(), sh);
+      }
+      if (G > 1 && g > 0) sred[(g - 1) * B + r] = sum;
       __syncthreads();
       if (lead) {
 #pragma unroll
-        for (int k = 0; k < G - 1; ++k) sum += sred[k * U * B + slot * B + r];
+        for (int k = 0; k < G - 1; ++k) sum += sred[k * B + r];
 #pragma unroll
         for (int f = 0; f < NFACE; ++f) {
           bool on;
           const int j = face_first<B>(f, r, on);
           if (on) {
 #pragma unroll
-            for (int a = 0; a < N; ++a) sum += spart[(slot * NFACE + f) * B + a * NF + j];
+            for (int a = 0; a < N; ++a) sum += spart[f * B + a * NF + j];
           }
         }
         if constexpr (kFx) {
@@ -680,12 +666,12 @@ static __global__ void __launch_bounds__(SymSmem<T, TD, B, OP, KIND>::NTH)
       const T t = rh - y;
       int Et = 0;
       if constexpr (kFxExt) {
-        if (lead) atomicMax(smax + slot, fx_exp(t, ui));
+        if (lead) atomicMax(smax, fx_exp(t, ui));
         __syncthreads();
-        if (lead) Et = smax[slot];
+        if (lead) Et = smax[0];
       }
       using TS = typename std::conditional<OP == SYM_CHEB, SX, T>::type;
-      TS* ts = reinterpret_cast<TS*>(sts) + slot * BX;
+      TS* ts = reinterpret_cast<TS*>(sts);
       XSum* xred = reinterpret_cast<XSum*>(sred);
       if (lead) {
         if constexpr (kFxExt) ts[r] = fx_split(t, Et - ui);
@@ -694,21 +680,19 @@ static __global__ void __launch_bounds__(SymSmem<T, TD, B, OP, KIND>::NTH)
       __syncthreads();
       T res = T(0);
       XSum es = XSum(0);
-      if (active) {
-        XAcc acc;
-        if constexpr (M::kExtMem) {
+      XAcc acc;
+      if constexpr (M::kExtMem) {
 #pragma unroll
-          for (int c = 0; c < M::CPG; ++c) acc.fma(sym_val(ev[c]), ts[g * M::CPG + c]);
-        } else {
-          sym_tri<T, B>(sext, r, ts, acc);
-        }
-        es = acc.sum();
-        if (G > 1 && g > 0) xred[(g - 1) * U * B + slot * B + r] = es;
+        for (int c = 0; c < M::CPG; ++c) acc.fma(sym_val(ev[c]), ts[g * M::CPG + c]);
+      } else {
+        sym_tri<T, B>(sext, r, ts, acc);
       }
+      es = acc.sum();
+      if (G > 1 && g > 0) xred[(g - 1) * B + r] = es;
       if (G > 1) __syncthreads();
       if (lead) {
 #pragma unroll
-        for (int k = 0; k < G - 1; ++k) es += xred[k * U * B + slot * B + r];
+        for (int k = 0; k < G - 1; ++k) es += xred[k * B + r];
         T sv;
         if constexpr (kFxExt) sv = Et == kFxInf ? nan("") : fx_scale(es, ui + Et + kFxBias - ext.k[unit]);
         else sv = es;
@@ -751,7 +735,7 @@ static __global__ void __launch_bounds__(SymSmem<T, TD, B, OP, KIND>::NTH)
     if constexpr (M::kStages == 2) {
       sg ^= 1;
       mask = next_mask;
-    } else if (next < ntiles) {
+    } else if (next < A.n) {
       load_info(next);
       issue(next, 0);
       mask = face_mask(next);
@@ -810,6 +794,7 @@ static __global__ void __launch_bounds__(SymRing<T, TD, B, OP, KIND>::NTH, SymRi
   constexpr bool kFxExt = M::kFx && OP == SYM_CHEB;   // the block inverses are in fixed point
   constexpr int EPW = M::EPW, NFACE = S::NFACE, BX = S::BX, NF = S::NF, BO = S::BO, N = S::N, NS = M::NS;
   constexpr int K0 = M::K0, K1 = M::K1, NB = K1 - K0;
+  static_assert(NS - 1 <= NB, "the first copies are one element's");
   constexpr bool kFx = M::kFx;
   constexpr int kShare = BO / N;                      // off-face terms of a face row per lane
   if (st && st->done) return;
@@ -882,11 +867,7 @@ static __global__ void __launch_bounds__(SymRing<T, TD, B, OP, KIND>::NTH, SymRi
   int slot = 0;
 #pragma unroll
   for (int j = 0; j < NS - 1; ++j) {
-    if (j < NB) {
-      if (gw < ntiles) issue(gw, K0 + j, ic, cc, j);
-    } else if (gw + nw < ntiles) {
-      issue(gw + nw, K0 + j - NB, in1, cn1, j);
-    }
+    if (gw < ntiles) issue(gw, K0 + j, ic, cc, j);
     asm volatile("cp.async.commit_group;" ::: "memory");
   }
   double dot = 0.0;
