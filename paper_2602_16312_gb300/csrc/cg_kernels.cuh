@@ -287,7 +287,7 @@ __device__ __forceinline__ double smooth_rate(double z, double z0, double k, dou
 // (2 FMAs per SM and clock on GB300; a division is ~10 of them, a tanh ~50), so
 // divisions by parameters are products with the inverses in IonicParams::inv,
 // the smoothed steps cost one exponential each, and a term behind a unit step is
-// evaluated on its side only. Gate update of 5.3M DoFs: 1,928 -> 727 us.
+// evaluated on its side only. Gate update of 5.3M DoFs: 1,928 -> 745 us.
 // The three gate rates:
 __device__ __forceinline__ void bueno_orovio_rates(const IonicParams& q, double u, const double* w, double* H) {
   const agg_bueno_orovio_params& p = q.bo;

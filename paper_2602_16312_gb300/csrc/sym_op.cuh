@@ -25,14 +25,15 @@
 // Measured on GB300 against one thread per element on the blocks of both
 // directions (k_spmv / k_cheb with FaceOp), which is FP64-bound in float64 and short
 // of loads in flight in float32:
-//   float64 product, 64^3 Q2 hexahedra: 1,483 -> 990 us (3.3 GB; HBM bound 490 us,
-//     the multiply-adds of three integer products per entry take the rest)
-//   float64 product, 24^3 Q3 hexahedra: 1,340 -> 272 us
-//   float64 smoothing step, 18^3 Q3 hexahedra: 1,475 -> 163 us (one stage: 200 us)
+//   float64 product, 64^3 Q2 hexahedra: 1,483 -> 1,010 us with x's copy (3.5 GB, 520
+//     us at the copy rate; HBM, the shared-memory data path and the integer
+//     multiply-adds are each about half busy: 15 warps per SM overlap them too little)
+//   float64 product, 24^3 Q3 hexahedra: 1,340 -> 276 us
+//   float64 smoothing step, 18^3 Q3 hexahedra: 1,475 -> 183 us (one stage: 220 us)
 //
-// Float64 products run on the integer pipe. GB300 issues 2 float64 FMAs per
-// SM and clock against 64 32-bit integer multiply-adds, so a float64 block
-// product is bound by the FP64 pipe, not by HBM. Here the operator is kept in
+// Float64 products run on the integer pipe. GB300 issues 2 float64 FMAs per SM and clock
+// against 64 32-bit integer multiply-adds (27 that add to 64 bits, as here), so a
+// float64 block product is bound by the FP64 pipe, not by HBM. Here the operator is kept in
 // 60-bit fixed point and x is converted to 58-bit fixed point with one exponent
 // per element; the sum of the products is formed exactly in 64-bit integers (up
 // to the product of the low halves, 2^-60 of the row's scale) and rounded once.
@@ -46,13 +47,14 @@
 // instead lost the ratio of its diagonal entries: worst row against 80-bit arithmetic,
 // relative to (|A| |x|)_i, Q2 shell 2.4e-15 -> 1.1e-16 (float64 sums: 6e-16), Q3 cube
 // 1.4e-15 -> 1.2e-16 (7e-16), 2D Q3 stiffness with a contrast of 1e-4 in the
-// conductivity 2.6e-13 -> 1.6e-15, there kept in float64 (3.6e-16). An entry is a1 2^28 + a0 with |a0| <= 2^27, an
-// x is x1 2^31 + x0 with |x0| <= 2^30. With sum_j |A_ij| <= 2^60, |A_ij| <= 2^58
-// (global exponent kA) and |x| <= 2^58, and T <= 304 entries in a row:
+// conductivity 2.6e-13 -> 1.6e-15, there kept in float64 (3.6e-16).
+// An entry is a1 2^28 + a0 with |a0| <= 2^27, an x is x1 2^31 + x0 with |x0| <= 2^30.
+// With sum_j |A_ij| <= 2^60, |A_ij| <= 2^58 (global exponent kA) and |x| <= 2^58, and
+// T <= 304 entries in a row:
 //   hi = sum a1 x1 <= 2^32 2^27,  m1 = sum a1 x0 <= 2^32 2^30,
 //   m2 = sum a0 x1 <= T 2^27 2^27 < 2^62.3,
-// so none overflows, and every a1 and x1 fits 32 bits. A NaN or infinity in the
-// neighbourhood takes a float64 path over the same entries.
+// so none overflows, and every a1 and x1 fits 32 bits. Vectors of wide range, NaN and
+// infinities: see SymVec.
 #pragma once
 #include "face_op.cuh"
 #include "kernels.cuh"
@@ -248,6 +250,13 @@ __device__ __forceinline__ void sym_tri(const ST* m, int r, const typename SymNu
 }
 
 enum { SYM_SPMV = 0, SYM_CHEB = 1, SYM_RESTRICT = 2 };
+// Stored entry and sum of the blocks that follow a product: block inverses (float64: fixed
+// point), transfer blocks (T)
+template <typename T, typename TD, int OP>
+using SymExt = typename std::conditional<OP != SYM_CHEB, T,
+    typename std::conditional<std::is_same<T, double>::value, int2, TD>::type>::type;
+template <typename T, int OP>
+using SymExtAcc = typename std::conditional<OP == SYM_CHEB, typename SymNum<T>::Acc, PlAcc<T>>::type;
 
 // A vector as the kernels read it: T = double: fixed point, X[unit B + i] and one
 // exponent per element (the largest biased exponent of its scaled x); T = float: the
@@ -280,8 +289,8 @@ struct SymSmem {
   using ST = typename SymNum<T>::ST;
   using SX = typename SymNum<T>::SX;
   using Sum = typename SymNum<T>::Acc::Sum;
-  using SD = typename std::conditional<OP == SYM_CHEB, typename std::conditional<std::is_same<T, double>::value, ST, TD>::type, T>::type;
-  using XAcc = typename std::conditional<OP == SYM_CHEB, typename SymNum<T>::Acc, PlAcc<T>>::type;   // block inverse / transfer sums
+  using SD = SymExt<T, TD, OP>;
+  using XAcc = SymExtAcc<T, OP>;
   using L = SymLay<ST, B>;
   static constexpr bool kFx = std::is_same<T, double>::value;
   static constexpr bool kProduct = !(OP == SYM_CHEB && KIND == 0);
@@ -761,8 +770,8 @@ struct SymRing {
   using ST = typename SymNum<T>::ST;
   using SX = typename SymNum<T>::SX;
   using Sum = typename SymNum<T>::Acc::Sum;
-  using SD = typename std::conditional<OP == SYM_CHEB, typename std::conditional<std::is_same<T, double>::value, ST, TD>::type, T>::type;
-  using XAcc = typename std::conditional<OP == SYM_CHEB, typename SymNum<T>::Acc, PlAcc<T>>::type;   // block inverse / transfer sums
+  using SD = SymExt<T, TD, OP>;
+  using XAcc = SymExtAcc<T, OP>;
   using L = SymLay<ST, B>;
   static constexpr bool kFx = std::is_same<T, double>::value;
   static constexpr bool kProduct = !(OP == SYM_CHEB && KIND == 0);
