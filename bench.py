@@ -6,7 +6,7 @@ A "step" is one time step of the hot path: ionic update + right-hand side
 by one V-cycle per iteration. Workload: 512x512 jittered quads, DG Q2
 (2,359,296 DoFs), 30-degree fibres, 4 agglomerated levels, FitzHugh-Nagumo,
 dt = 0.05. Every vector and matrix is resident in HBM; the fine matrix
-(0.85 GB float64) is far larger than L2, so every step streams from HBM.
+(0.55 GB float64) is far larger than L2, so every step streams from HBM.
 
   python bench.py [--steps K] [--warmup W] [--form f32|f64|bf16s] [--impl reference]
 
