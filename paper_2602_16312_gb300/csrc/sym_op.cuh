@@ -272,7 +272,7 @@ using SymExtAcc = typename std::conditional<OP == SYM_CHEB, typename SymNum<T>::
 // beside the unit off by 6e-5 of (|A| |x|)_i before.) Of random vectors and CG
 // directions (from stimuli and fronts) at most 0.4% of the elements were kept as
 // doubles, mostly none; 4% of a first direction from a front on the thin shell. Cost on
-// the 40^3 Q2 product (272 us): 1% of the elements 285 us, every one 1,590 us.
+// the 40^3 Q2 product (270 us): 1% of the elements 285 us, every one 1,590 us.
 template <typename T> struct SymVec {
   const typename SymNum<T>::SX* X;
   const int* E;
@@ -360,7 +360,8 @@ __device__ __forceinline__ double sym_wide_row(const SymView<double, B>& A, int6
   return y;
 }
 // The same as a call: k_sym is faster with it (V-cycle of the 18^3 Q3 cube 2,288 inline,
-// 2,272 us), k_symw<9> inline (V-cycle on 250^2 Q2 556, 542 us).
+// 2,272 us), and the products of k_symw (40^3 Q2 272, 266 us); its smoothing steps are
+// faster inline (V-cycle on 250^2 Q2 556 with the call, 542 us).
 template <int B>
 __device__ __noinline__ double sym_wide_row_call(SymView<double, B> A, int64_t unit, int r, double y, const int2* X,
                                                  const int* E) {
@@ -966,7 +967,9 @@ static __global__ void __launch_bounds__(SymRing<T, TD, B, OP, KIND>::NTH, SymRi
         if (M::kProduct && active) {
           if constexpr (kFx) {
             y = fx_scale(sum, ti - A.kA + E + kFxBias);
-            if (lo < kFxWide / 2) y = sym_wide_row<B>(A, unit, r, E < kFxWide / 2 ? 0.0 : y, xv.X, xv.E);
+            const double y0 = E < kFxWide / 2 ? 0.0 : y;
+            if (lo < kFxWide / 2)
+              y = OP == SYM_SPMV ? sym_wide_row_call<B>(A, unit, r, y0, xv.X, xv.E) : sym_wide_row<B>(A, unit, r, y0, xv.X, xv.E);
           } else {
             y = sum;
           }
